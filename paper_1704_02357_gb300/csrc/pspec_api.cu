@@ -66,6 +66,22 @@ struct Plan {
   size_t o_rmesh1, o_rmesh2, o_rsums, o_desc, o_cur, o_bout;
 };
 
+// Persistent blocks of the combine and binning passes for nk bins. Their shared memory grows with
+// the bins (8 bytes per bin and block, 4 or 8 per bin and warp), so this is set from the bins of
+// the call and not from the context's max_kbins: with the default max_kbins = 512 a 512^3 binning
+// block takes 134 KB and one fits an SM, with the 160 bins of a survey call 109 KB and two do (a
+// set's binning 6.3 -> 5.1 ms exact-add, 4.3 -> 3.4 ms plain).
+void set_ctas(Plan* pl, bool f64, int nk, int nsm) {
+  if (f64) {
+    pl->ctas_comb = pl->td->ctas(0, nk, nsm, 0);
+    pl->ctas_bin = pl->ctas_bin_plain = pl->td->ctas(1, nk, nsm, 0);
+  } else {
+    pl->ctas_comb = pl->tf->ctas(0, nk, nsm, pl->xp);
+    pl->ctas_bin = pl->tf->ctas(pl->has_ytab ? 2 : 1, nk, nsm, pl->xp);
+    pl->ctas_bin_plain = pl->tf->ctas(1, nk, nsm, pl->xp);
+  }
+}
+
 pspec_status build_plan(const pspec_params* p, int max_kbins, int nsm, Plan* pl, std::string* why) {
   if (!p) { *why = "params is NULL"; return PSPEC_EINVAL; }
   if (!good_nmesh(p->nmesh)) { *why = "nmesh must be even, 16..1024 and 2^a, or 48..768 and 3*2^a"; return PSPEC_EUNSUPPORTED; }
@@ -127,14 +143,7 @@ pspec_status build_plan(const pspec_params* p, int max_kbins, int nsm, Plan* pl,
     if (pl->has_ytab) need = std::max(need, pl->tf->smem_bin_pipe(max_kbins));
     if (need > kSmemMaxBlock) { *why = "max_kbins too large for this mesh (shared memory)"; return PSPEC_EINVAL; }
   }
-  if (f64) {
-    pl->ctas_comb = pl->td->ctas(0, max_kbins, nsm, 0);
-    pl->ctas_bin = pl->ctas_bin_plain = pl->td->ctas(1, max_kbins, nsm, 0);
-  } else {
-    pl->ctas_comb = pl->tf->ctas(0, max_kbins, nsm, pl->xp);
-    pl->ctas_bin = pl->tf->ctas(pl->has_ytab ? 2 : 1, max_kbins, nsm, pl->xp);
-    pl->ctas_bin_plain = pl->tf->ctas(1, max_kbins, nsm, pl->xp);
-  }
+  set_ctas(pl, f64, max_kbins, nsm);
   pl->nblk_sum = 2 * nsm;
 
   size_t o = 0;
@@ -413,6 +422,7 @@ pspec_status upload_bins(Ctx* c, const double* edges, int nk) {
     kmag[n2] = kf * std::sqrt(x);
     if (b >= 0) {
       if (hi[b] == 0) lo[b] = n2;
+  set_ctas(&c->pl, c->p.precision == PSPEC_FP64, nk, c->nsm);
       hi[b] = n2 + 1;
       n2_cut = n2 + 1;
     }
