@@ -147,16 +147,45 @@ __global__ void __launch_bounds__(kSumThreads) k_catalog_partials(PaintArgs a_in
   }
 }
 
-// Neumaier-compensated FP64 accumulator (the block partials are few).
+// Neumaier-compensated FP64 accumulator (the block partials are few). The magnitudes are compared
+// as integers: FP64 compares run on the narrow FP64 pipe.
 struct Neu {
   double s = 0.0, c = 0.0;
   __device__ __forceinline__ void add(double x) {
     const double t = s + x;
-    c += (fabs(s) >= fabs(x)) ? (s - t) + x : (x - t) + s;
+    const bool s_larger = (__double_as_longlong(s) & 0x7fffffffffffffffll) >= (__double_as_longlong(x) & 0x7fffffffffffffffll);
+    c += ((s_larger ? s : x) - t) + (s_larger ? x : s);
     s = t;
   }
   __device__ __forceinline__ double val() const { return s + c; }
 };
+
+// Compensated sum of one column of the block partials by one warp (every lane of it): each lane
+// adds every 32nd partial, then the lanes' (sum, compensation) pairs are added in a tree. An FP64
+// warp instruction holds GB300's FP64 pipe for 64 cycles however few lanes are active, so one
+// thread walking the 304 partials of a catalog column by column took 190 us for a mock's sums and
+// 448 us for two weighted catalogs; with one warp per column it is a chain of ~15 additions.
+__device__ __forceinline__ Neu column_sum(const double* __restrict__ part, int nb, int col) {
+  Neu a;
+  const int lane = threadIdx.x & 31;
+#pragma unroll 4
+  for (int b = lane; b < nb; b += 32) a.add(part[b * kSumVals + col]);
+  for (int o = 16; o > 0; o >>= 1) {
+    const double s2 = __shfl_down_sync(0xffffffffu, a.s, o), c2 = __shfl_down_sync(0xffffffffu, a.c, o);
+    a.add(s2);
+    a.c += c2;
+  }
+  return a;  // lane 0
+}
+// Columns 0..3 of the data (warps 0..3) and randoms (warps 4..7) partials; nbd or nbr = 0 leaves
+// zeros. All threads of a 256-thread block.
+__device__ __forceinline__ void all_column_sums(const double* pd, int nbd, const double* pr, int nbr, double (&sum)[8]) {
+  const int w = threadIdx.x >> 5;
+  const Neu a = w < 4 ? column_sum(pd, nbd, w) : column_sum(pr, nbr, w - 4);
+  if ((threadIdx.x & 31) == 0) sum[w] = a.val();
+  __syncthreads();
+}
+constexpr int kFinalThreads = 256;
 
 // The fixed-point scale 2^S of the exact paint for meshes whose values are all bounded by
 // `bound` in magnitude: every cell sum then stays below 2^61 in units of 2^-S.
@@ -168,35 +197,26 @@ __device__ double fix_scale(double bound) {
   return ldexp(1.0, S);
 }
 
-// One thread adds the block partials in a fixed order: deterministic alpha, I, S. `fix`
+// One block adds the block partials in a fixed order: deterministic alpha, I, S. `fix`
 // (nullable) receives the exact paint's fixed-point scale for data (+v) and randoms
 // (-alpha v) painted together.
-__global__ void k_catalog_final(const double* pd, int nbd, const double* pr, int nbr, double* d, double* fix) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  Neu wd, sd, wr, sr, ir;
-  double ad = 0.0, ar = 0.0;
-  for (int b = 0; b < nbd; b++) {
-    wd.add(pd[b * kSumVals + 0]);
-    sd.add(pd[b * kSumVals + 1]);
-    ad += pd[b * kSumVals + 3];
-  }
-  for (int b = 0; b < nbr; b++) {
-    wr.add(pr[b * kSumVals + 0]);
-    sr.add(pr[b * kSumVals + 1]);
-    ir.add(pr[b * kSumVals + 2]);
-    ar += pr[b * kSumVals + 3];
-  }
-  const double alpha = wd.val() / wr.val();
-  d[D_WD] = wd.val();
-  d[D_WR] = wr.val();
+__global__ void __launch_bounds__(kFinalThreads) k_catalog_final(const double* pd, int nbd, const double* pr, int nbr,
+                                                                 double* d, double* fix) {
+  __shared__ double sum[8];
+  all_column_sums(pd, nbd, pr, nbr, sum);
+  if (threadIdx.x != 0) return;
+  const double wd = sum[0], sd = sum[1], ad = sum[3], wr = sum[4], sr = sum[5], ir = sum[6], ar = sum[7];
+  const double alpha = wd / wr;
+  d[D_WD] = wd;
+  d[D_WR] = wr;
   d[D_ALPHA] = alpha;
-  d[D_I] = alpha * ir.val();
-  d[D_S] = sd.val() + alpha * alpha * sr.val();
+  d[D_I] = alpha * ir;
+  d[D_S] = sd + alpha * alpha * sr;
   d[D_NONFINITE] = 0.0;
   d[D_WRAPPED] = 0.0;
-  d[D_SD] = sd.val();
-  d[D_SR] = sr.val();
-  d[D_IR] = ir.val();
+  d[D_SD] = sd;
+  d[D_SR] = sr;
+  d[D_IR] = ir;
   if (fix) *fix = fix_scale(ad + fabs(alpha) * ar);
 }
 
@@ -225,7 +245,7 @@ void launch_catalog_partials(const PaintArgs& a, double* partials, int nblocks, 
 
 void launch_catalog_final(const double* part_d, int nb_d, const double* part_r, int nb_r, double* derived,
                           cudaStream_t s, double* fix) {
-  k_catalog_final<<<1, 32, 0, s>>>(part_d, nb_d, part_r, nb_r, derived, fix);
+  k_catalog_final<<<1, kFinalThreads, 0, s>>>(part_d, nb_d, part_r, nb_r, derived, fix);
 }
 
 void launch_derive_uniform(int64_t n_d, int64_t n_r, double wf, double nbar, double* derived, cudaStream_t s) {
@@ -500,27 +520,36 @@ __global__ void __launch_bounds__(256) k_ptile_prep(PaintArgs a_in, int is_rando
   }
 }
 
-// Exclusive prefix sum of the tile counts (one block): off[] and cursor[].
+// Places in the tile-sorted copy: off[] and cursor[]. Each block takes 1024 tiles, one a thread, adds
+// their counts up in an exclusive prefix sum and reserves the block's range with one atomic add on
+// the counter behind the counts (cleared with them). The ranges of the blocks lie in any order: a
+// tile only needs a range of its own. (One block scanning all tiles, each thread a run of them
+// twice over, took 85 us at 512^3 and 177 us at 768^3.)
 __global__ void __launch_bounds__(1024) k_ptile_scan(TileArgs ta, int ntiles) {
-  __shared__ unsigned part[1024];
-  const int per = (ntiles + blockDim.x - 1) / blockDim.x;
-  const int b0 = threadIdx.x * per;
-  unsigned s = 0;
-  for (int i = b0; i < b0 + per && i < ntiles; i++) s += ta.cnt[i];
-  part[threadIdx.x] = s;
+  __shared__ unsigned wsum[32], base;
+  const int i = blockIdx.x * 1024 + threadIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const unsigned n = i < ntiles ? ta.cnt[i] : 0u;
+  unsigned inc = n;
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
+  }
+  if (lane == 31) wsum[w] = inc;
   __syncthreads();
-  for (int o = 1; o < (int)blockDim.x; o <<= 1) {
-    const unsigned add = threadIdx.x >= (unsigned)o ? part[threadIdx.x - o] : 0u;
-    __syncthreads();
-    part[threadIdx.x] += add;
-    __syncthreads();
+  if (w == 0) {
+    unsigned v = wsum[lane];
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned u = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += u;
+    }
+    wsum[lane] = v;
+    if (lane == 31) base = atomicAdd(&ta.cnt[ntiles], v);
   }
-  unsigned run = part[threadIdx.x] - s;
-  for (int i = b0; i < b0 + per && i < ntiles; i++) {
-    ta.off[i] = run;
-    ta.cursor[i] = run;
-    run += ta.cnt[i];
-  }
+  __syncthreads();
+  if (i >= ntiles) return;
+  const unsigned at = base + (w ? wsum[w - 1] : 0u) + inc - n;
+  ta.off[i] = at;
+  ta.cursor[i] = at;
 }
 
 // Each record goes to every tile its footprint touches (the order within a tile is free: the
@@ -611,10 +640,14 @@ __device__ __forceinline__ void tile_scatter(unsigned* acc, int hi_off, const in
 // One block per tile (every tile, so that empty tiles store their zeros): sums its records into
 // shared 64-bit accumulators (lo words of both meshes, then hi words), then stores each cell of
 // the tile once, four cells along z per 16-byte store. A tile without records stores zeros and
-// skips the accumulators.
+// skips the accumulators. With cached randoms meshes r1, r2 (batched mocks; r1 null: none) it stores
+// cell - alpha * randoms cell instead: the same FMA as a pass of its own over the meshes, which
+// would read and write each once more (135 us a mesh at 384^3).
 template <int WIN, bool INTER>
 __global__ void __launch_bounds__(256) k_ptile_paint(TileArgs ta, float* __restrict__ m1, float* __restrict__ m2,
-                                                     int N, const double* __restrict__ fix) {
+                                                     int N, const double* __restrict__ fix,
+                                                     const float* __restrict__ r1, const float* __restrict__ r2,
+                                                     const double* __restrict__ alpha) {
   extern __shared__ __align__(16) unsigned acc[];  // lo [NM][kPT^3], then hi [NM][kPT^3]
   constexpr int NM = INTER ? 2 : 1;
   constexpr int HI = NM * kPT3;
@@ -630,11 +663,19 @@ __global__ void __launch_bounds__(256) k_ptile_paint(TileArgs ta, float* __restr
     const int lx = cell / (kPT * kPT), ly = (cell / kPT) % kPT, lz = cell % kPT;
     return ((int64_t)(tx * kPT + lx) * N + (ty * kPT + ly)) * N + tz * kPT + lz;
   };
+  const float al = r1 ? (float)*alpha : 0.f;
+  auto store = [&](int mesh, int64_t g, float4 v) {
+    if (r1) {
+      const float4 r = __ldg(reinterpret_cast<const float4*>((mesh ? r2 : r1) + g));
+      v = make_float4(fmaf(-al, r.x, v.x), fmaf(-al, r.y, v.y), fmaf(-al, r.z, v.z), fmaf(-al, r.w, v.w));
+    }
+    *reinterpret_cast<float4*>((mesh ? m2 : m1) + g) = v;
+  };
   if (n == 0) {
     for (int i = threadIdx.x; i < NM * kPT3 / 4; i += blockDim.x) {
       int mesh;
       const int64_t g = group(i, mesh);
-      *reinterpret_cast<float4*>((mesh ? m2 : m1) + g) = make_float4(0.f, 0.f, 0.f, 0.f);
+      store(mesh, g, make_float4(0.f, 0.f, 0.f, 0.f));
     }
     return;  // uniform over the block: no barrier is left behind
   }
@@ -670,8 +711,7 @@ __global__ void __launch_bounds__(256) k_ptile_paint(TileArgs ta, float* __restr
     auto cell = [&](unsigned l, unsigned h) {
       return ll2f_rn_int((long long)(((unsigned long long)h << 32) | l)) * inv;
     };
-    *reinterpret_cast<float4*>((mesh ? m2 : m1) + g) =
-        make_float4(cell(lo.x, hi.x), cell(lo.y, hi.y), cell(lo.z, hi.z), cell(lo.w, hi.w));
+    store(mesh, g, make_float4(cell(lo.x, hi.x), cell(lo.y, hi.y), cell(lo.z, hi.z), cell(lo.w, hi.w)));
   }
 }
 
@@ -693,7 +733,9 @@ void launch_ptile_prep(const PaintArgs& a, int window, int interlaced, int is_ra
   }
 }
 
-void launch_ptile_scan(const TileArgs& ta, int ntiles, cudaStream_t s) { k_ptile_scan<<<1, 1024, 0, s>>>(ta, ntiles); }
+void launch_ptile_scan(const TileArgs& ta, int ntiles, cudaStream_t s) {
+  k_ptile_scan<<<(ntiles + 1023) / 1024, 1024, 0, s>>>(ta, ntiles);
+}
 
 void launch_ptile_scatter(const TileArgs& ta, int64_t total, const DevCat* dc, const int* cur, int N, int nblocks,
                           cudaStream_t s) {
@@ -708,63 +750,54 @@ template <typename K> static void set_smem_attr(K kernel, size_t bytes) {
 }
 
 void launch_ptile_paint(const TileArgs& ta, int window, int interlaced, float* m1, float* m2, int N,
-                        const double* fix, cudaStream_t s) {
+                        const double* fix, const float* r1, const float* r2, const double* alpha, cudaStream_t s) {
   const int ntiles = (N / kPT) * (N / kPT) * (N / kPT);
   const size_t smem = (size_t)(interlaced ? 2 : 1) * kPT3 * sizeof(unsigned long long);
   if (window == PSPEC_WINDOW_CIC) {
     if (interlaced) {
       set_smem_attr(k_ptile_paint<PSPEC_WINDOW_CIC, true>, smem);
-      k_ptile_paint<PSPEC_WINDOW_CIC, true><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix);
+      k_ptile_paint<PSPEC_WINDOW_CIC, true><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
     } else {
-      k_ptile_paint<PSPEC_WINDOW_CIC, false><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix);
+      k_ptile_paint<PSPEC_WINDOW_CIC, false><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
     }
   } else {
     if (interlaced) {
       set_smem_attr(k_ptile_paint<PSPEC_WINDOW_TSC, true>, smem);
-      k_ptile_paint<PSPEC_WINDOW_TSC, true><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix);
+      k_ptile_paint<PSPEC_WINDOW_TSC, true><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
     } else {
-      k_ptile_paint<PSPEC_WINDOW_TSC, false><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix);
+      k_ptile_paint<PSPEC_WINDOW_TSC, false><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
     }
   }
 }
 
 // ------------------------------------------------------------------ batched mocks
 // rsums = (W_r, S_r, I_r, fixed-point scale of the randoms mesh painted alone) of the cached randoms.
-__global__ void k_randoms_sums(const double* pr, int nbr, double* rsums) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  Neu wr, sr, ir;
-  double ar = 0.0;
-  for (int b = 0; b < nbr; b++) {
-    wr.add(pr[b * kSumVals + 0]);
-    sr.add(pr[b * kSumVals + 1]);
-    ir.add(pr[b * kSumVals + 2]);
-    ar += pr[b * kSumVals + 3];
-  }
-  rsums[0] = wr.val();
-  rsums[1] = sr.val();
-  rsums[2] = ir.val();
-  rsums[3] = fix_scale(ar);
+__global__ void __launch_bounds__(kFinalThreads) k_randoms_sums(const double* pr, int nbr, double* rsums) {
+  __shared__ double sum[8];
+  all_column_sums(pr, 0, pr, nbr, sum);
+  if (threadIdx.x != 0) return;
+  rsums[0] = sum[4];
+  rsums[1] = sum[5];
+  rsums[2] = sum[6];
+  rsums[3] = fix_scale(sum[7]);
 }
 
-__global__ void k_catalog_final_cached(const double* pd, int nbd, const double* rsums, double* d) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  Neu wd, sd;
-  double ad = 0.0;
-  for (int b = 0; b < nbd; b++) {
-    wd.add(pd[b * kSumVals + 0]);
-    sd.add(pd[b * kSumVals + 1]);
-    ad += pd[b * kSumVals + 3];
-  }
+__global__ void __launch_bounds__(kFinalThreads) k_catalog_final_cached(const double* pd, int nbd,
+                                                                        const double* __restrict__ rsums, double* d) {
+  __shared__ double sum[8];
+  all_column_sums(pd, nbd, pd, 0, sum);
+  if (threadIdx.x != 0) return;
+  const double wd = sum[0], sd = sum[1], ad = sum[3];
   const double Wr = rsums[0], Sr = rsums[1], Ir = rsums[2];
-  const double alpha = wd.val() / Wr;
-  d[D_WD] = wd.val();
+  const double alpha = wd / Wr;
+  d[D_WD] = wd;
   d[D_WR] = Wr;
   d[D_ALPHA] = alpha;
   d[D_I] = alpha * Ir;
-  d[D_S] = sd.val() + alpha * alpha * Sr;
+  d[D_S] = sd + alpha * alpha * Sr;
   d[D_NONFINITE] = 0.0;
   d[D_WRAPPED] = 0.0;
-  d[D_SD] = sd.val();
+  d[D_SD] = sd;
   d[D_SR] = Sr;
   d[D_IR] = Ir;
   d[D_FIX] = fix_scale(ad);  // the mock's data mesh is painted alone
@@ -797,11 +830,11 @@ __global__ void k_advance(int* cur) {
 }
 
 void launch_randoms_sums(const double* part_r, int nb_r, double* rsums, cudaStream_t s) {
-  k_randoms_sums<<<1, 32, 0, s>>>(part_r, nb_r, rsums);
+  k_randoms_sums<<<1, kFinalThreads, 0, s>>>(part_r, nb_r, rsums);
 }
 void launch_catalog_final_cached(const double* part_d, int nb_d, const double* rsums, double* derived,
                                  cudaStream_t s) {
-  k_catalog_final_cached<<<1, 32, 0, s>>>(part_d, nb_d, rsums, derived);
+  k_catalog_final_cached<<<1, kFinalThreads, 0, s>>>(part_d, nb_d, rsums, derived);
 }
 void launch_axpy_randoms(float* mesh, const float* rmesh, int64_t n, const double* derived, cudaStream_t s) {
   k_axpy_randoms<float><<<2048, 256, 0, s>>>(mesh, rmesh, n, derived);

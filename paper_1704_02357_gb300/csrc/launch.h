@@ -98,8 +98,8 @@ void launch_paint(const PaintArgs& a, int window, int interlaced, int is_randoms
 constexpr int kPaintTile = 16;
 constexpr int kPaintRecordsMax = 8;
 struct TileArgs {
-  unsigned* cnt;     // [ntiles] records per tile (cleared before prep)
-  unsigned* off;     // [ntiles] exclusive prefix of cnt
+  unsigned* cnt;     // [ntiles + 1] records per tile, then the records placed so far (cleared before prep)
+  unsigned* off;     // [ntiles] first record of the tile in the sorted copy
   unsigned* cursor;  // [ntiles] scatter cursors
   uint4* rec;        // [particles] records in input order
   unsigned* tile_of; // [particles] first tile of each record (all ones: left out)
@@ -110,8 +110,9 @@ void launch_ptile_prep(const PaintArgs& a, int window, int interlaced, int is_ra
 void launch_ptile_scan(const TileArgs& ta, int ntiles, cudaStream_t s);
 void launch_ptile_scatter(const TileArgs& ta, int64_t total, const DevCat* dc, const int* cur, int N, int nblocks,
                           cudaStream_t s);
+// r1, r2 (nullable, batched mocks): cached randoms meshes; mesh = painted - *alpha * randoms.
 void launch_ptile_paint(const TileArgs& ta, int window, int interlaced, float* m1, float* m2, int N,
-                        const double* fix, cudaStream_t s);
+                        const double* fix, const float* r1, const float* r2, const double* alpha, cudaStream_t s);
 
 // Transform passes, one table of launchers per supported mesh side N (pass_*.cu).
 // Tables: tw_half (L = N/2), tw_full (L = N), twr (exp(-2 pi i k/N), k < N/2).

@@ -190,7 +190,7 @@ pspec_status build_plan(const pspec_params* p, int max_kbins, int nsm, Plan* pl,
   pl->max_particles = f64 ? 0 : p->max_particles;
   pl->ntiles = (N / kPaintTile) * (N / kPaintTile) * (N / kPaintTile);
   if (pl->max_particles > 0) {
-    pl->o_tcnt = take((size_t)pl->ntiles * sizeof(unsigned));
+    pl->o_tcnt = take((size_t)(pl->ntiles + 1) * sizeof(unsigned));
     pl->o_toff = take((size_t)pl->ntiles * sizeof(unsigned));
     pl->o_tcur = take((size_t)pl->ntiles * sizeof(unsigned));
     pl->o_prec = take((size_t)pl->max_particles * 16);
@@ -404,6 +404,7 @@ pspec_status upload_tables(Ctx* c) {
 pspec_status upload_bins(Ctx* c, const double* edges, int nk) {
   std::vector<double> e(edges, edges + nk + 1);
   if (e == c->edges) return PSPEC_OK;
+  set_ctas(&c->pl, c->p.precision == PSPEC_FP64, nk, c->nsm);
   const Plan& pl = c->pl;
   std::vector<double> t(nk + 1);
   for (int b = 0; b <= nk; b++) {
@@ -422,7 +423,6 @@ pspec_status upload_bins(Ctx* c, const double* edges, int nk) {
     kmag[n2] = kf * std::sqrt(x);
     if (b >= 0) {
       if (hi[b] == 0) lo[b] = n2;
-  set_ctas(&c->pl, c->p.precision == PSPEC_FP64, nk, c->nsm);
       hi[b] = n2 + 1;
       n2_cut = n2 + 1;
     }
@@ -553,7 +553,7 @@ pspec_status do_paint(Ctx* c, const pspec_catalog* d, const pspec_catalog* r) {
   if (sizeof(T) == 4 && c->tune.paint_binned && pl.max_particles > 0 && total <= pl.max_particles) {
     // exact tile-binned paint: every cell of both meshes is stored, nothing to clear
     TileArgs ta = tile_args(c);
-    e = cudaMemsetAsync(ta.cnt, 0, (size_t)pl.ntiles * sizeof(unsigned), c->stream);
+    e = cudaMemsetAsync(ta.cnt, 0, (size_t)(pl.ntiles + 1) * sizeof(unsigned), c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "tile counts clear");
     float* f1 = reinterpret_cast<float*>(m1);
     float* f2 = reinterpret_cast<float*>(m2);
@@ -566,7 +566,7 @@ pspec_status do_paint(Ctx* c, const pspec_catalog* d, const pspec_catalog* r) {
     TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scan(ta, pl.ntiles, c->stream); }));
     TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scatter(ta, total, nullptr, nullptr, N, nb, c->stream); }));
     TRY(run(c, PSPEC_K_PAINT, nmesh * pl.Sr, [&] {
-      launch_ptile_paint(ta, c->p.window, c->p.interlaced, f1, f2, N, der + D_FIX, c->stream);
+      launch_ptile_paint(ta, c->p.window, c->p.interlaced, f1, f2, N, der + D_FIX, nullptr, nullptr, nullptr, c->stream);
     }));
     c->bytes_paint = bytes + cat_bytes(d) + cat_bytes(r) + nmesh * pl.Sr;
     return PSPEC_OK;
@@ -757,10 +757,12 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
 }
 
 // Paint `a` (a data catalog, or randoms with is_randoms = 2) into m1/m2 (zeroed here):
-// tile-binned when `binned`, else direct atomics. `max_count` bounds the particles.
+// tile-binned when `binned`, else direct atomics. `max_count` bounds the particles. With r1 (and r2)
+// the cached randoms meshes times alpha are subtracted: as the tiles are stored, or in a pass of
+// their own after direct painting.
 template <typename T>
 pspec_status paint_one(Ctx* c, const PaintArgs& a, int is_randoms, bool binned, int64_t max_count, T* m1, T* m2,
-                       const double* fix) {
+                       const double* fix, const T* r1 = nullptr, const T* r2 = nullptr) {
   const Plan& pl = c->pl;
   const int N = pl.g.N;
   const int nb = 16 * c->nsm;
@@ -770,16 +772,17 @@ pspec_status paint_one(Ctx* c, const PaintArgs& a, int is_randoms, bool binned, 
   const double pbytes = (a.pos_f32 ? 12.0 : 24.0) * (double)max_count;
   if (binned && sizeof(T) == 4) {
     TileArgs ta = tile_args(c);
-    e = cudaMemsetAsync(ta.cnt, 0, (size_t)pl.ntiles * sizeof(unsigned), c->stream);
+    e = cudaMemsetAsync(ta.cnt, 0, (size_t)(pl.ntiles + 1) * sizeof(unsigned), c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "tile counts clear");
     TRY(run(c, PSPEC_K_PAINT, pbytes, [&] {
       launch_ptile_prep(a, c->p.window, c->p.interlaced, is_randoms, der, ta, 0, N, nb, c->stream);
     }));
     TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scan(ta, pl.ntiles, c->stream); }));
     TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scatter(ta, a.count, a.dc, a.cur, N, nb, c->stream); }));
-    TRY(run(c, PSPEC_K_PAINT, nmesh * pl.Sr, [&] {
+    TRY(run(c, PSPEC_K_PAINT, (r1 ? 2.0 : 1.0) * nmesh * pl.Sr, [&] {
       launch_ptile_paint(ta, c->p.window, c->p.interlaced, reinterpret_cast<float*>(m1), reinterpret_cast<float*>(m2),
-                         N, fix, c->stream);
+                         N, fix, reinterpret_cast<const float*>(r1), reinterpret_cast<const float*>(r2), der + D_ALPHA,
+                         c->stream);
     }));
   } else {
     e = cudaMemsetAsync(m1, 0, pl.Sr, c->stream);
@@ -788,6 +791,9 @@ pspec_status paint_one(Ctx* c, const PaintArgs& a, int is_randoms, bool binned, 
     TRY(run(c, PSPEC_K_PAINT, pbytes + nmesh * pl.Sr, [&] {
       launch_paint<T>(a, c->p.window, c->p.interlaced, is_randoms, der, m1, m2, N, nb, c->stream);
     }));
+    const int64_t n = (int64_t)N * N * N;
+    if (r1) TRY(run(c, PSPEC_K_OTHER, 3.0 * pl.Sr, [&] { launch_axpy_randoms(m1, r1, n, der, c->stream); }));
+    if (r1 && m2) TRY(run(c, PSPEC_K_OTHER, 3.0 * pl.Sr, [&] { launch_axpy_randoms(m2, r2, n, der, c->stream); }));
   }
   return PSPEC_OK;
 }
@@ -821,11 +827,8 @@ pspec_status enqueue_mock(Ctx* c, bool binned, int64_t max_count, const int32_t*
   }));
   T* m1 = c->at<T>(pl.o_mesh1);
   T* m2 = c->p.interlaced ? c->at<T>(pl.o_mesh2) : nullptr;
-  TRY(paint_one<T>(c, a, 0, binned, max_count, m1, m2, der + D_FIX));
-  const int64_t n = (int64_t)pl.g.N * pl.g.N * pl.g.N;
-  TRY(run(c, PSPEC_K_OTHER, 3.0 * pl.Sr, [&] { launch_axpy_randoms(m1, c->at<T>(pl.o_rmesh1), n, der, c->stream); }));
-  if (m2)
-    TRY(run(c, PSPEC_K_OTHER, 3.0 * pl.Sr, [&] { launch_axpy_randoms(m2, c->at<T>(pl.o_rmesh2), n, der, c->stream); }));
+  TRY(paint_one<T>(c, a, 0, binned, max_count, m1, m2, der + D_FIX, c->at<T>(pl.o_rmesh1),
+                   m2 ? c->at<T>(pl.o_rmesh2) : nullptr));
   double* out = c->at<double>(pl.o_out);
   TRY(do_multipoles<T>(c, ells, n_ells, nk, out + 2 * (size_t)nk, out, out + nk));
   TRY(run(c, PSPEC_K_OTHER, 0.0, [&] {
