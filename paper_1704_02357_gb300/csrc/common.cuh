@@ -46,6 +46,8 @@ template <typename C> using ux_of = ux<typename BaseOf<C>::type>;
 
 __device__ __forceinline__ float4 ldg_u(const float4* p) { return __ldg(p); }
 __device__ __forceinline__ double2 ldg_u(const double2* p) { return __ldg(p); }
+__device__ __forceinline__ int4 ldg_u(const int4* p) { return __ldg(p); }
+__device__ __forceinline__ int4 uconj(int4 w) { return make_int4(w.x, w.y, -w.z, -w.w); }
 __device__ __forceinline__ float4 uconj(float4 w) { return make_float4(w.x, -w.y, w.z, -w.w); }
 __device__ __forceinline__ double2 uconj(double2 w) { return make_double2(w.x, -w.y); }
 // a * w
@@ -58,7 +60,7 @@ __device__ __forceinline__ double2 umul(double2 a, double2 w) {
 }
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
-// x * K for an irrational constant K: in FP32 as x*K_hi + x*K_lo (K_lo = K - K_hi), so that
+// x * K for an irrational constant K in FP32, as x*K_hi + x*K_lo (K_lo = K - K_hi), so that
 // the product carries no systematic rounding of K (a rounded K = sqrt(1/2) alone scales a
 // quarter of every radix-8 stage's output power by 1 - 3.4e-8).
 template <typename T> struct ConstMul;
@@ -67,14 +69,8 @@ template <> struct ConstMul<float> {
   __device__ __forceinline__ constexpr ConstMul(double k) : hi((float)k), lo((float)(k - (double)(float)k)) {}
   __device__ __forceinline__ float operator()(float x) const { return fmaf(x, hi, x * lo); }
 };
-template <> struct ConstMul<double> {
-  double k;
-  __device__ __forceinline__ constexpr ConstMul(double k_) : k(k_) {}
-  __device__ __forceinline__ double operator()(double x) const { return x * k; }
-};
-
 // ------------------------------------------------------------------ butterflies
-// Small DFTs in registers. dir = -1: exp(-2 pi i jk/R) (forward); +1: inverse.
+// Small DFTs in registers (FP32; fx_engine.cuh has the fixed-point forms of radix 8 and 3). dir = -1: exp(-2 pi i jk/R) (forward); +1: inverse.
 template <typename C, int R> struct Dft;
 
 template <typename C> struct Dft<C, 2> {

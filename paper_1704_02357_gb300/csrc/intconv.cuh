@@ -42,6 +42,15 @@ PSPEC_HD float ic_float(unsigned u) {
   return f;
 #endif
 }
+PSPEC_HD double ic_double(unsigned long long u) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)u);
+#else
+  double f;
+  std::memcpy(&f, &u, sizeof f);
+  return f;
+#endif
+}
 // leading zeros of a nonzero 64-bit value
 PSPEC_HD int ic_clz64(unsigned long long a) {
 #ifdef __CUDA_ARCH__

@@ -18,6 +18,7 @@
 #include <cmath>
 #include "launch.h"
 #include "fft_engine.cuh"
+#include "fx_engine.cuh"
 #include "xp_engine.cuh"
 
 namespace pspec {
@@ -56,6 +57,9 @@ template <int N, bool XP> struct ZShape {
   static constexpr int ROWS = (S::ROWS * S::Tz / Tz) > 0 ? (S::ROWS * S::Tz / Tz) : 1;
   static constexpr int ZT = ROWS * Tz;
 };
+
+// FP64 rows go through fixed point, 8 elements (four registers each) per thread too.
+template <typename T, int N, bool XP> using ZRow = ZShape<N, XP || sizeof(T) == 8>;
 
 // ------------------------------------------------------------------ spectrum storage order
 // s[((kz / TW * N + i) * N + j) * TW + kz % TW]: a y-pass slab (i, kz tile) is one contiguous
@@ -122,12 +126,12 @@ __device__ __forceinline__ T per_mode_w2(T v, const cx<T>* __restrict__ iw, int 
 
 // ------------------------------------------------------------------ pass z: r2c of plain rows
 template <typename T, int N>
-__global__ void __launch_bounds__(Shape<N>::ZT, min_blocks<T, Shape<N>::EZ>(Shape<N>::ZT))
+__global__ void __launch_bounds__(ZRow<T, N, false>::ZT, min_blocks<T, ZRow<T, N, false>::E>(ZRow<T, N, false>::ZT))
     k_r2c_z(const T* __restrict__ in, cx<T>* __restrict__ out, const ux<T>* __restrict__ twh,
             const ux<T>* __restrict__ twr) {
   using C = cx<T>;
-  using S = Shape<N>;
-  constexpr int L = S::NH, E = S::EZ, Tc = S::Tz;
+  using S = ZRow<T, N, false>;
+  constexpr int L = N / 2, E = S::E, Tc = S::Tz;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   const int r = threadIdx.x / Tc, t = threadIdx.x - r * Tc;
@@ -136,24 +140,30 @@ __global__ void __launch_bounds__(Shape<N>::ZT, min_blocks<T, Shape<N>::EZ>(Shap
   C v[E];
 #pragma unroll
   for (int e = 0; e < E; e++) v[e] = src[t + Tc * e];
-  fft_ct<C, E, L, kPaddedRows, 1, -1, S::ZW>(v, sm, t, r, twh);
-  C zm[E];
-  if constexpr (S::ZW) {
-    row_mirrors<C, E, Tc>(v, zm, t);
-  } else {
+  if constexpr (sizeof(T) == 8) {
+    fx_row_r2c<E, L, S::ZW>(v, sm, t, r, twh, twr);
 #pragma unroll
-    for (int e = 0; e < E; e++) sm[sidx<kPaddedRows, L, 1>(r, t + Tc * e)] = v[e];
-    __syncthreads();
+    for (int e = 0; e < E; e++) out[Lay<N>::row(row, t + Tc * e)] = v[e];
+  } else {
+    fft_ct<C, E, L, kPaddedRows, 1, -1, S::ZW>(v, sm, t, r, twh);
+    C zm[E];
+    if constexpr (S::ZW) {
+      row_mirrors<C, E, Tc>(v, zm, t);
+    } else {
+#pragma unroll
+      for (int e = 0; e < E; e++) sm[sidx<kPaddedRows, L, 1>(r, t + Tc * e)] = v[e];
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < E; e++) {
+        const int k = t + Tc * e;
+        zm[e] = sm[sidx<kPaddedRows, L, 1>(r, k ? L - k : 0)];
+      }
+    }
 #pragma unroll
     for (int e = 0; e < E; e++) {
       const int k = t + Tc * e;
-      zm[e] = sm[sidx<kPaddedRows, L, 1>(r, k ? L - k : 0)];
+      out[Lay<N>::row(row, k)] = r2c_unpack<C, T>(v[e], zm[e], ldg_u(twr + k));
     }
-  }
-#pragma unroll
-  for (int e = 0; e < E; e++) {
-    const int k = t + Tc * e;
-    out[Lay<N>::row(row, k)] = r2c_unpack<C, T>(v[e], zm[e], ldg_u(twr + k));
   }
 }
 
@@ -161,31 +171,42 @@ __global__ void __launch_bounds__(Shape<N>::ZT, min_blocks<T, Shape<N>::EZ>(Shap
 // Rows of L stored modes (the kz = N/2 mode taken as 0) -> N reals, times `scale`.
 // XP: exact-add pack and stages (FP32 only).
 template <typename T, int N, bool XP>
-__global__ void __launch_bounds__(ZShape<N, XP>::ZT, min_blocks<T, ZShape<N, XP>::E>(ZShape<N, XP>::ZT))
+__global__ void __launch_bounds__(ZRow<T, N, XP>::ZT, min_blocks<T, ZRow<T, N, XP>::E>(ZRow<T, N, XP>::ZT))
     k_c2r_z(const cx<T>* __restrict__ in, T* __restrict__ out, const ux<T>* __restrict__ twh,
             const ux<T>* __restrict__ twr, T scale) {
   using C = cx<T>;
-  using S = ZShape<N, XP>;
+  using S = ZRow<T, N, XP>;
   constexpr int L = N / 2, E = S::E, Tc = S::Tz;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   const int r = threadIdx.x / Tc, t = threadIdx.x - r * Tc;
   const int row = blockIdx.x * S::ROWS + r;
   C v[E];
+  if constexpr (sizeof(T) == 8) {
+    C m[E];
 #pragma unroll
-  for (int e = 0; e < E; e++) {
-    const int k = t + Tc * e;
-    const C xk = in[Lay<N>::row(row, k)];
-    if constexpr (XP) {
-      v[e] = c2r_pack_xp(xk, k ? in[Lay<N>::row(row, L - k)] : mk(T(0), T(0)), uconj(ldg_u(twr + k)));
-    } else {
-      const C xm = k ? cconj(in[Lay<N>::row(row, L - k)]) : mk(T(0), T(0));
-      const C ev = cscale(cadd(xk, xm), T(0.5));
-      const C od = umul(cscale(csub(xk, xm), T(0.5)), uconj(ldg_u(twr + k)));
-      v[e] = mk(ev.x - od.y, ev.y + od.x);  // E + i O
+    for (int e = 0; e < E; e++) {
+      const int k = t + Tc * e;
+      v[e] = in[Lay<N>::row(row, k)];
+      m[e] = k ? in[Lay<N>::row(row, L - k)] : mk(T(0), T(0));
     }
+    fx_row_c2r<E, L, S::ZW>(v, m, sm, t, r, twh, twr);
+  } else {
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+      const int k = t + Tc * e;
+      const C xk = in[Lay<N>::row(row, k)];
+      if constexpr (XP) {
+        v[e] = c2r_pack_xp(xk, k ? in[Lay<N>::row(row, L - k)] : mk(T(0), T(0)), uconj(ldg_u(twr + k)));
+      } else {
+        const C xm = k ? cconj(in[Lay<N>::row(row, L - k)]) : mk(T(0), T(0));
+        const C ev = cscale(cadd(xk, xm), T(0.5));
+        const C od = umul(cscale(csub(xk, xm), T(0.5)), uconj(ldg_u(twr + k)));
+        v[e] = mk(ev.x - od.y, ev.y + od.x);  // E + i O
+      }
+    }
+    fft_any<XP, C, E, L, kPaddedRows, 1, +1, S::ZW>(v, sm, t, r, twh);
   }
-  fft_any<XP, C, E, L, kPaddedRows, 1, +1, S::ZW>(v, sm, t, r, twh);
   C* dst = reinterpret_cast<C*>(out + (int64_t)row * N);
 #pragma unroll
   for (int e = 0; e < E; e++) dst[t + Tc * e] = cscale(v[e], scale);
@@ -207,7 +228,7 @@ __global__ void __launch_bounds__(ylm_thread_cap(LT), sizeof(T) == 4 ? ylm_min_b
                                                   const float* __restrict__ rtab,
                                                   const __grid_constant__ YTab<T> yt) {
   using C = cx<T>;
-  using S = ZShape<N, XP>;
+  using S = ZRow<T, N, XP>;
   constexpr int L = N / 2, E = S::E, Tc = S::Tz;
   extern __shared__ __align__(16) unsigned char smraw[];
   T* stage = reinterpret_cast<T*>(smraw);  // [nseq][N] reals, then the exchange buffer
@@ -331,22 +352,28 @@ __global__ void __launch_bounds__(ylm_thread_cap(LT), sizeof(T) == 4 ? ylm_min_b
     for (int e = 0; e < E; e++) v[e] = stc[sq * L + t + Tc * e];
     __syncthreads();  // the staging area becomes the exchange buffer
   }
-  fft_any<XP, C, E, L, kPaddedRows, 1, -1, S::ZW>(v, xb, t, sq, twh);
-  // mirrors through shared memory (shuffles would raise this kernel's register count, measured slower)
-#pragma unroll
-  for (int e = 0; e < E; e++) xb[sidx<kPaddedRows, L, 1>(sq, t + Tc * e)] = v[e];
-  fft_sync<S::ZW>();
   const int s = sq / rows, r = sq - s * rows;
   C* dst = out + s * spec_stride;
   const int64_t grow = row0 + r;
+  if constexpr (sizeof(T) == 8) {
+    fx_row_r2c<E, L, S::ZW>(v, xb, t, sq, twh, twr);
 #pragma unroll
-  for (int e = 0; e < E; e++) {
-    const int k = t + Tc * e;
-    const C zm = xb[sidx<kPaddedRows, L, 1>(sq, k ? L - k : 0)];
-    if constexpr (XP)
-      dst[Lay<N>::row(grow, k)] = r2c_unpack_xp(v[e], zm, ldg_u(twr + k));
-    else
-      dst[Lay<N>::row(grow, k)] = r2c_unpack<C, T>(v[e], zm, ldg_u(twr + k));
+    for (int e = 0; e < E; e++) dst[Lay<N>::row(grow, t + Tc * e)] = v[e];
+  } else {
+    fft_any<XP, C, E, L, kPaddedRows, 1, -1, S::ZW>(v, xb, t, sq, twh);
+    // mirrors through shared memory (shuffles would raise this kernel's register count, measured slower)
+#pragma unroll
+    for (int e = 0; e < E; e++) xb[sidx<kPaddedRows, L, 1>(sq, t + Tc * e)] = v[e];
+    fft_sync<S::ZW>();
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+      const int k = t + Tc * e;
+      const C zm = xb[sidx<kPaddedRows, L, 1>(sq, k ? L - k : 0)];
+      if constexpr (XP)
+        dst[Lay<N>::row(grow, k)] = r2c_unpack_xp(v[e], zm, ldg_u(twr + k));
+      else
+        dst[Lay<N>::row(grow, k)] = r2c_unpack<C, T>(v[e], zm, ldg_u(twr + k));
+    }
   }
 }
 
@@ -356,20 +383,22 @@ __global__ void __launch_bounds__(ylm_thread_cap(LT), sizeof(T) == 4 ? ylm_min_b
 // with ky^2 + kz^2 >= n2_cut are not stored: every mode of their x column lies beyond the
 // last bin, and the binning pass skips those columns (INT_MAX stores everything).
 // XP: exact-add stages (FP32 only).
-template <int N, bool XP> constexpr int col_elems() { return XP ? Shape<N>::EYX : Shape<N>::EY; }
+template <typename T, int N, bool XP> constexpr int col_elems() {
+  return sizeof(T) == 8 ? Shape<N>::E : (XP ? Shape<N>::EYX : Shape<N>::EY);
+}
 
 // Exact-add blocks of 256 threads: three per SM (80 registers) beat two (104), measured.
 template <int N, bool XP> constexpr int y_min_blocks(int threads) {
-  return XP && threads == 256 ? 3 : min_blocks<float, col_elems<N, XP>()>(threads);
+  return XP && threads == 256 ? 3 : min_blocks<float, col_elems<float, N, XP>()>(threads);
 }
 template <typename T, int N, int DIR, int TW, bool XP>
-__global__ void __launch_bounds__(TW * (N / col_elems<N, XP>()),
-                                  sizeof(T) == 4 ? y_min_blocks<N, XP>(TW * (N / col_elems<N, XP>()))
-                                                 : min_blocks<T, col_elems<N, XP>()>(TW * (N / col_elems<N, XP>())))
+__global__ void __launch_bounds__(TW * (N / col_elems<T, N, XP>()),
+                                  sizeof(T) == 4 ? y_min_blocks<N, XP>(TW * (N / col_elems<T, N, XP>()))
+                                                 : min_blocks<T, col_elems<T, N, XP>()>(TW * (N / col_elems<T, N, XP>())))
     k_fft_y(cx<T>* __restrict__ data, int64_t spec_stride, const ux<T>* __restrict__ twf, int n2_cut) {
   using C = cx<T>;
   using S = Shape<N>;
-  constexpr int NH = S::NH, E = col_elems<N, XP>(), Tc = N / E;
+  constexpr int NH = S::NH, E = col_elems<T, N, XP>(), Tc = N / E;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   static_assert(Lay<N>::TW % TW == 0, "a y tile lies within one storage tile");
@@ -393,12 +422,12 @@ __global__ void __launch_bounds__(TW * (N / col_elems<N, XP>()),
 
 // ------------------------------------------------------------------ pass x (plain)
 template <typename T, int N, int DIR, bool XP>
-__global__ void __launch_bounds__(Shape<N>::TW * (N / col_elems<N, XP>()),
-                                  min_blocks<T, col_elems<N, XP>()>(Shape<N>::TW * (N / col_elems<N, XP>())))
+__global__ void __launch_bounds__(Shape<N>::TW * (N / col_elems<T, N, XP>()),
+                                  min_blocks<T, col_elems<T, N, XP>()>(Shape<N>::TW * (N / col_elems<T, N, XP>())))
     k_fft_x(const cx<T>* in, cx<T>* out, const ux<T>* __restrict__ twf) {
   using C = cx<T>;
   using S = Shape<N>;
-  constexpr int NH = S::NH, E = col_elems<N, XP>(), Tc = N / E, TW = S::TW;
+  constexpr int NH = S::NH, E = col_elems<T, N, XP>(), Tc = N / E, TW = S::TW;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   const int c = threadIdx.x % TW, t = threadIdx.x / TW;
@@ -443,7 +472,7 @@ __global__ void __launch_bounds__(Shape<N>::CT, min_blocks<T, Shape<N>::E>(Shape
     C v[E];
 #pragma unroll
     for (int e = 0; e < E; e++) v[e] = B[off + (t + Tc * e) * si];
-    fft_ct<C, E, N, kInterleaved, TW, -1>(v, sm, t, c, twf);
+    fft_any<false, C, E, N, kInterleaved, TW, -1>(v, sm, t, c, twf);
     const int ny = sfreq<N>(j);
     const C iwy = ldg_c(invw + j), iwz = ldg_c(invw + N + kz);
     const T wyz = iwy.x * iwz.x, lyz = iwy.y + iwz.y;
@@ -741,13 +770,14 @@ template <typename T, int N> struct Passes {
   }
 
   static void r2c_z(const T* in, C* out, const U* twh, const U* twr, cudaStream_t s) {
-    const size_t smem = (size_t)S::ROWS * padded_len(S::NH) * sizeof(C);
+    using Z = ZRow<T, N, false>;
+    const size_t smem = (size_t)Z::ROWS * padded_len(S::NH) * sizeof(C);
     set_smem(k_r2c_z<T, N>, smem);
-    k_r2c_z<T, N><<<N * N / S::ROWS, S::ZT, smem, s>>>(in, out, twh, twr);
+    k_r2c_z<T, N><<<N * N / Z::ROWS, Z::ZT, smem, s>>>(in, out, twh, twr);
   }
   // Launchers taking `xp` run the exact-add variant of their kernel when it is set (FP32 only).
   template <bool XP> static void c2r_z_v(const C* in, T* out, const U* twh, const U* twr, T scale, cudaStream_t s) {
-    using Z = ZShape<N, XP>;
+    using Z = ZRow<T, N, XP>;
     const size_t smem = (size_t)Z::ROWS * padded_len(S::NH) * sizeof(C);
     set_smem(k_c2r_z<T, N, XP>, smem);
     k_c2r_z<T, N, XP><<<N * N / Z::ROWS, Z::ZT, smem, s>>>(in, out, twh, twr, scale);
@@ -767,7 +797,7 @@ template <typename T, int N> struct Passes {
   static void ylm_z_v(const T* f, C* out, int64_t stride, int ell, int h0, int M, const U* twh, const U* twr,
                       const T* axis, int rows, const float* rtab, cudaStream_t s) {
     const size_t smem = smem_ylm(M, rows);
-    const dim3 grid(N * N / rows), block(M * rows * ZShape<N, XP>::Tz);
+    const dim3 grid(N * N / rows), block(M * rows * ZRow<T, N, XP>::Tz);
     set_smem(k_ylm_r2c_z<T, N, LT, XP>, smem);
     k_ylm_r2c_z<T, N, LT, XP><<<grid, block, smem, s>>>(f, out, stride, ell, h0, M, twh, twr, axis, rows, rtab,
                                                          host_ytab<T>());
@@ -799,7 +829,7 @@ template <typename T, int N> struct Passes {
   template <int TWV, bool XP>
   static void fft_y_tw(C* data, int64_t stride, int nspec, const U* twf, int dir, int n2_cut, cudaStream_t s) {
     const size_t smem = (size_t)N * TWV * sizeof(C);
-    const int threads = TWV * (N / col_elems<N, XP>());
+    const int threads = TWV * (N / col_elems<T, N, XP>());
     dim3 grid(N * (S::NH / TWV), nspec);
     if (dir < 0) {
       set_smem(k_fft_y<T, N, -1, TWV, XP>, smem);
@@ -828,7 +858,7 @@ template <typename T, int N> struct Passes {
   template <bool XP> static void fft_x_v(const C* in, C* out, const U* twf, int dir, cudaStream_t s) {
     const size_t smem = smem_col();
     const unsigned grid = N * (S::NH / S::TW);
-    const int threads = S::TW * (N / col_elems<N, XP>());
+    const int threads = S::TW * (N / col_elems<T, N, XP>());
     if (dir < 0) {
       set_smem(k_fft_x<T, N, -1, XP>, smem);
       k_fft_x<T, N, -1, XP><<<grid, threads, smem, s>>>(in, out, twf);
@@ -911,7 +941,7 @@ template <typename T, int N> struct Passes {
     t.E = S::E;
     t.tw = S::TW;
     t.rows_z = S::ROWS;
-    t.tz = S::Tz;
+    t.tz = ZRow<T, N, false>::Tz;
     t.tz_xp = ZShape<N, sizeof(T) == 4>::Tz;
     t.r2c_z = &r2c_z;
     t.c2r_z = &c2r_z;

@@ -321,6 +321,24 @@ float4 unit_factor12(double a) {
   return make_float4((float)c12, (float)s12, (float)(c - c12), (float)(s - s12));
 }
 
+// Twiddle exp(-2 pi i t/n) as the transform stages take it: unit_factor in FP32; in FP64 contexts four
+// integers {c_h, c_l, s_h, s_l} of the fixed-point stages, each component h 2^-30 + l 2^-62.
+template <typename T> ux<T> twiddle(int t, int n) { return unit_factor<T>(-2.0 * M_PI * t / n); }
+template <> ux<double> twiddle<double>(int t, int n) {
+  const long double a = -2.0L * std::acos(-1.0L) * t / n;
+  int32_t w[4];
+  for (int i = 0; i < 2; i++) {
+    const int64_t q = (int64_t)std::llrint((i ? std::sin(a) : std::cos(a)) * 4611686018427387904.0L);  // 2^62
+    const int64_t h = (q + (1ll << 31)) >> 32;
+    w[2 * i] = (int32_t)h;
+    w[2 * i + 1] = (int32_t)std::max<int64_t>(q - h * (1ll << 32), INT_MIN + 1);  // its negative is needed too
+  }
+  ux<double> u;
+  static_assert(sizeof u == sizeof w, "one table entry");
+  std::memcpy(&u, w, sizeof u);
+  return u;
+}
+
 template <typename T>
 pspec_status upload_tables(Ctx* c) {
   const Plan& pl = c->pl;
@@ -330,11 +348,11 @@ pspec_status upload_tables(Ctx* c) {
   std::vector<U> twh(NH), twf(N), twr(NH), phase(3 * N);
   std::vector<C> invw(N + NH);
   std::vector<T> axis(3 * N);
+  for (int t = 0; t < N; t++) twf[t] = twiddle<T>(t, N);
   for (int t = 0; t < NH; t++) {
-    twh[t] = unit_factor<T>(-2.0 * M_PI * t / NH);
-    twr[t] = unit_factor<T>(-2.0 * M_PI * t / N);
+    twh[t] = twf[2 * t];
+    twr[t] = twf[t];
   }
-  for (int t = 0; t < N; t++) twf[t] = unit_factor<T>(-2.0 * M_PI * t / N);
   const double H = c->p.box_size / N;
   for (int d = 0; d < 3; d++)
     for (int i = 0; i < N; i++) axis[d * N + i] = T(c->p.box_corner[d] + i * H - c->p.observer[d]);

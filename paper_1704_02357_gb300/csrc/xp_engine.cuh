@@ -21,7 +21,7 @@
 // add level. Every operation whose exactness the scheme relies on uses the _rn intrinsics or an
 // FMA whose result is exact, and the compiler never contracts the intrinsics into a multiply-add.
 #pragma once
-#include "fft_engine.cuh"
+#include "fx_engine.cuh"
 
 namespace pspec {
 
@@ -281,11 +281,14 @@ __device__ __forceinline__ void fft_xp(float2 (&v)[E], float2* sm, int t, int se
   });
 }
 
-// The transform the kernels call: exact-add stages when XP, else the plain engine.
+// The transform the kernels call: exact-add stages when XP, fixed point for FP64 values, else the
+// plain engine.
 template <bool XP, typename C, int E, int L, int LAYOUT, int NSEQ, int DIR, bool WARP = false>
 __device__ __forceinline__ void fft_any(C (&v)[E], C* sm, int t, int seq, const ux_of<C>* __restrict__ tw) {
   if constexpr (XP)
     fft_xp<E, L, LAYOUT, NSEQ, DIR, WARP>(v, sm, t, seq, tw);
+  else if constexpr (std::is_same<C, double2>::value)
+    fft_fx<E, L, LAYOUT, NSEQ, DIR, WARP>(v, sm, t, seq, tw);
   else
     fft_ct<C, E, L, LAYOUT, NSEQ, DIR, WARP>(v, sm, t, seq, tw);
 }
