@@ -90,6 +90,91 @@ template <> const YTab<double>& host_ytab<double>() {
   return t;
 }
 
+// ------------------------------------------------------------------ Y_lm polynomials (FP64 contexts)
+namespace {
+// A polynomial in (x, y, z), homogeneous of degree n <= kPolyLmax: c[p][i] of x^p y^i z^(n-p-i).
+struct Hom {
+  int n = 0;
+  long double c[kPolyLmax + 1][kPolyLmax + 1] = {};
+};
+// a * P * Q with Q given by its terms (exponents of x, y, z all of one degree)
+struct Term {
+  long double c;
+  int x, y;
+};
+Hom mul(const Hom& P, const Term* t, int nt, int deg) {
+  Hom R;
+  R.n = P.n + deg;
+  for (int p = 0; p <= P.n; p++)
+    for (int i = 0; i + p <= P.n; i++)
+      for (int k = 0; k < nt; k++) R.c[p + t[k].x][i + t[k].y] += P.c[p][i] * t[k].c;
+  return R;
+}
+Hom lin(long double a, const Hom& P, long double b, const Hom& Q) {
+  Hom R;
+  R.n = P.n;
+  for (int p = 0; p <= R.n; p++)
+    for (int i = 0; i + p <= R.n; i++) R.c[p][i] = a * P.c[p][i] + b * Q.c[p][i];
+  return R;
+}
+
+PolyTab build_poly() {
+  PolyTab t = {};
+  const Term x[1] = {{1.0L, 1, 0}}, y[1] = {{1.0L, 0, 1}}, z[1] = {{1.0L, 0, 0}};
+  const Term r2[3] = {{1.0L, 2, 0}, {1.0L, 0, 2}, {1.0L, 0, 0}};
+  const long double pi = std::acos(-1.0L);
+  Hom re, im;  // Re, Im (x + i y)^a
+  re.c[0][0] = 1.0L;
+  long double ca = 1.0L / std::sqrt(4.0L * pi);  // c_a of the recurrence
+  for (int a = 0; a <= kPolyLmax; a++) {
+    if (a > 0) {
+      const Hom nr = lin(1.0L, mul(re, x, 1, 1), -1.0L, mul(im, y, 1, 1));
+      im = lin(1.0L, mul(im, x, 1, 1), 1.0L, mul(re, y, 1, 1));
+      re = nr;
+      ca *= -std::sqrt((2.0L * a + 1.0L) / (2.0L * a));
+    }
+    const long double n = a ? std::sqrt(2.0L) * ca : ca;
+    for (int part = 0; part < (a ? 2 : 1); part++) {
+      Hom qm1, qm2;
+      for (int l = a; l <= kPolyLmax; l++) {
+        Hom cur;
+        if (l == a) {
+          cur = lin(n, part ? im : re, 0.0L, re);
+        } else {
+          const long double A = std::sqrt((4.0L * l * l - 1.0L) / ((long double)l * l - (long double)a * a));
+          cur = mul(qm1, z, 1, 1);
+          if (l > a + 1) {
+            const long double B = std::sqrt(((l - 1.0L) * (l - 1.0L) - (long double)a * a) / (4.0L * (l - 1.0L) * (l - 1.0L) - 1.0L));
+            cur = lin(A, cur, -A * B, mul(qm2, r2, 3, 2));
+          } else {
+            cur = lin(A, cur, 0.0L, cur);
+          }
+        }
+        qm2 = qm1;
+        qm1 = cur;
+        if (l == 0) continue;
+        const int h = a == 0 ? 0 : (part ? 2 * a : 2 * a - 1);
+        const int NP = poly_np(l), NI = l + 1;
+        for (int k = 0; k < NP; k++) {
+          const int px = poly_par_x(h) + 2 * k, pz = poly_par_z(l, h) + 2 * k;
+          for (int i = 0; i < NI; i++) {
+            const int at = poly_base(l) + (h * NP + k) * NI + i;
+            if (px + i <= l) t.kx[at] = (double)cur.c[px][i];
+            if (pz + i <= l) t.rz[at] = (double)cur.c[i][l - pz - i];  // x^i y^(l-pz-i) z^pz
+          }
+        }
+      }
+    }
+  }
+  return t;
+}
+}  // namespace
+
+const PolyTab& host_poly() {
+  static const PolyTab t = build_poly();
+  return t;
+}
+
 // ------------------------------------------------------------------ Y_lm(khat) table
 // Position m of a k-space table of the binning pass -> its mode (i, j, kz): one block of N x tw
 // values per x tile (j, kz tile), rows i, m = ((kz / tw * N + j) * N + i) * tw + kz % tw.

@@ -79,10 +79,21 @@ template <int N> struct Lay {
   __device__ static __forceinline__ int64_t table_tile(int kt, int j) { return ((int64_t)kt * N + j) * N * TW; }
 };
 
+// kz columns per block of the y and x passes: the storage tile's, but at most 256 threads in FP64, whose
+// fixed-point stages take 72 registers a thread and more: three blocks of 256 threads share an SM where
+// one of 512 would run alone, and each covers the others' barriers (512^3, per spectrum: y pass
+// 1.08 -> 0.72 ms).
+template <typename T, int N> constexpr int col_block_tile() {
+  int tw = Shape<N>::TW;
+  while (sizeof(T) == 8 && tw > 1 && tw * Shape<N>::Tc > 256) tw /= 2;
+  return tw;
+}
+
 // Resident blocks per SM the register allocation must allow. Threads holding 24 complex
 // elements (3 * 2^a meshes) get at least 128 registers in FP32; 8 elements fit in 64.
+// FP64 columns and rows (fixed point): at most 128 registers for up to 256 threads.
 template <typename T, int E> constexpr int min_blocks(int threads) {
-  if constexpr (sizeof(T) != 4) return 1;
+  if constexpr (sizeof(T) != 4) return E > 8 || threads > 256 ? 1 : 2;
   if constexpr (E > 8) return threads >= 512 ? 1 : 65536 / (((threads + 31) / 32) * 32 * 128);
   return threads >= 512 ? 2 : (threads >= 256 ? 3 : 4);
 }
@@ -220,12 +231,98 @@ __global__ void __launch_bounds__(ZRow<T, N, XP>::ZT, min_blocks<T, ZRow<T, N, X
 // into the M spectra. With the Y_lm(rhat) table and sequences within one warp, each thread loads
 // its own slots of f and of the table and multiplies them in registers: no staging, and no block
 // barrier.
+template <typename T, int N> __host__ __device__ constexpr size_t ylm_stage_bytes(int M, int rows) {
+  return (size_t)M * rows * (N * sizeof(T) > padded_len(N / 2) * sizeof(cx<T>) ? N * sizeof(T)
+                                                                              : padded_len(N / 2) * sizeof(cx<T>));
+}
+
+// 1/x and 1/sqrt(x) of a positive normal FP64 number: the hardware's approximation (about 20 bits) and
+// two Newton steps, within an ulp or two. (The divisions and square roots of the library take three
+// times the FP64 operations; the pipe runs two per clock and SM.)
+__device__ __forceinline__ double rcp_newton(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+__device__ __forceinline__ double rsqrt_newton(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(0.5 * y, fma(-(x * y), y, 1.0), y);
+  return fma(0.5 * y, fma(-(x * y), y, 1.0), y);
+}
+
+// f Y_lm(rhat) of `rows` rows and M harmonics into the staging area (FP64 contexts): per row the
+// coefficients of the powers of z of each r^l Y_lm, then per node l/2 multiply-adds a harmonic at most and
+// one product with f / r^l (times z for odd powers). All threads of the block. 25 FP64 operations a
+// node for the nine harmonics of l = 4, 16 for l = 2, where the recurrence took about 90 and 55.
+template <int N, int LT>
+__device__ __forceinline__ void poly_weights(const double* __restrict__ f, const double* __restrict__ axis,
+                                             const double* __restrict__ poly, int ell, int h0, int M, int row0, int rows,
+                                             double* cf, double* stage) {
+  const int NP = poly_np(ell), NI = ell + 1;
+  for (int q = threadIdx.x; q < rows * M * NP; q += blockDim.x) {
+    const int k = q % NP, rs = q / NP, s = rs % M, r = rs / M;
+    const int grow = row0 + r, i = grow / N, j = grow - i * N;
+    const double x = axis[i], y = axis[N + j];
+    const int n = ell - (poly_par_z(ell, h0 + s) + 2 * k);  // degree in x and y
+    const double* c = poly + ((h0 + s) * NP + k) * NI;
+    double acc = 0.0;
+    if (n >= 0) {
+      acc = c[n];
+      double yp = 1.0;
+      for (int p = n - 1; p >= 0; p--) {
+        yp *= y;
+        acc = fma(acc, x, c[p] * yp);
+      }
+    }
+    cf[q] = acc;
+  }
+  __syncthreads();
+  for (int r = 0; r < rows; r++) {
+    const int grow = row0 + r, i = grow / N, j = grow - i * N;
+    const double vx = axis[i], vy = axis[N + j], rho2 = vx * vx + vy * vy;
+    const double* cr = cf + r * M * NP;
+    for (int kk = threadIdx.x; kk < N; kk += blockDim.x) {
+      const double z = axis[2 * N + kk], z2 = z * z, r2 = rho2 + z2;
+      double g = f[(int64_t)grow * N + kk];
+      if (ell & 1) {
+        const double inv = rsqrt_newton(r2), inv2 = inv * inv;
+        g *= inv;
+        for (int p = 1; p < ell; p += 2) g *= inv2;
+      } else {
+        const double inv2 = rcp_newton(r2);
+        for (int p = 0; p < ell; p += 2) g *= inv2;
+      }
+      if (r2 == 0.0) g = 0.0;  // the node at the observer
+      const double gz = g * z;
+      double* st = stage + r * N + kk;
+      auto one = [&](int s, int a) {
+        const double* c = cr + s * NP;
+        const int deg = (ell - a) >> 1;
+        double v = c[deg];
+#pragma unroll
+        for (int p = deg - 1; p >= 0; p--) v = fma(v, z2, c[p]);
+        st[s * rows * N] = v * (((ell - a) & 1) ? gz : g);
+      };
+      if (LT > 0 && h0 == 0 && M == 2 * LT + 1) {
+#pragma unroll
+        for (int s = 0; s < 2 * LT + 1; s++) one(s, harm_a(s));
+      } else {
+        for (int s = 0; s < M; s++) one(s, harm_a(h0 + s));
+      }
+    }
+  }
+}
+
 template <typename T, int N, int LT, bool XP>
-__global__ void __launch_bounds__(ylm_thread_cap(LT), sizeof(T) == 4 ? ylm_min_blocks(LT, XP) : 0) k_ylm_r2c_z(const T* __restrict__ f, cx<T>* __restrict__ out,
+__global__ void __launch_bounds__(ylm_thread_cap(LT), sizeof(T) == 4 ? ylm_min_blocks(LT, XP)
+                                                                     : (N % 3 == 0 ? 1 : (LT == 4 ? 3 : (LT == 2 ? 5 : 1)))) k_ylm_r2c_z(const T* __restrict__ f, cx<T>* __restrict__ out,
                                                   int64_t spec_stride, int ell, int h0, int M,
                                                   const ux<T>* __restrict__ twh, const ux<T>* __restrict__ twr,
                                                   const T* __restrict__ axis, int rows,
                                                   const float* __restrict__ rtab,
+                                                  const double* __restrict__ poly,
                                                   const __grid_constant__ YTab<T> yt) {
   using C = cx<T>;
   using S = ZRow<T, N, XP>;
@@ -274,10 +371,16 @@ __global__ void __launch_bounds__(ylm_thread_cap(LT), sizeof(T) == 4 ? ylm_min_b
       }
     }
   }
+  if constexpr (sizeof(T) == 8 && LT >= 0) {
+    if (poly) {
+      T* cf = reinterpret_cast<T*>(smraw + ylm_stage_bytes<T, N>(M, rows));
+      poly_weights<N, LT>(f, axis, poly, LT > 0 ? LT : ell, h0, M, row0, rows, cf, stage);
+    }
+  }
   for (int r = 0; r < rows; r++) {
     const int grow = row0 + r;
-    if constexpr (sizeof(T) == 4 && LT >= 0) {
-      if (rtab) continue;
+    if constexpr (LT >= 0) {
+      if (sizeof(T) == 4 ? rtab != nullptr : poly != nullptr) continue;
     }
     const int i = grow / N, j = grow - i * N;
     const T vx = axis[i], vy = axis[N + j];
@@ -391,6 +494,7 @@ template <typename T, int N, bool XP> constexpr int col_elems() {
 template <int N, bool XP> constexpr int y_min_blocks(int threads) {
   return XP && threads == 256 ? 3 : min_blocks<float, col_elems<float, N, XP>()>(threads);
 }
+template <typename T, int N> constexpr int col_threads() { return col_block_tile<T, N>() * Shape<N>::Tc; }
 template <typename T, int N, int DIR, int TW, bool XP>
 __global__ void __launch_bounds__(TW * (N / col_elems<T, N, XP>()),
                                   sizeof(T) == 4 ? y_min_blocks<N, XP>(TW * (N / col_elems<T, N, XP>()))
@@ -421,19 +525,19 @@ __global__ void __launch_bounds__(TW * (N / col_elems<T, N, XP>()),
 }
 
 // ------------------------------------------------------------------ pass x (plain)
+// A block of TW columns is part of a storage tile when TW is narrower (FP64).
 template <typename T, int N, int DIR, bool XP>
-__global__ void __launch_bounds__(Shape<N>::TW * (N / col_elems<T, N, XP>()),
-                                  min_blocks<T, col_elems<T, N, XP>()>(Shape<N>::TW * (N / col_elems<T, N, XP>())))
+__global__ void __launch_bounds__(col_block_tile<T, N>() * (N / col_elems<T, N, XP>()),
+                                  min_blocks<T, col_elems<T, N, XP>()>(col_block_tile<T, N>() * (N / col_elems<T, N, XP>())))
     k_fft_x(const cx<T>* in, cx<T>* out, const ux<T>* __restrict__ twf) {
   using C = cx<T>;
-  using S = Shape<N>;
-  constexpr int NH = S::NH, E = col_elems<T, N, XP>(), Tc = N / E, TW = S::TW;
+  constexpr int E = col_elems<T, N, XP>(), Tc = N / E, TW = col_block_tile<T, N>(), SUB = Lay<N>::TW / TW;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   const int c = threadIdx.x % TW, t = threadIdx.x / TW;
-  const int kt = blockIdx.x / N, j = blockIdx.x - kt * N;  // tiles in storage order
+  const int part = blockIdx.x % SUB, tile = blockIdx.x / SUB, kt = tile / N, j = tile - kt * N;  // in storage order
   constexpr int64_t si = Lay<N>::XI;
-  const int64_t off = Lay<N>::at(0, j, kt * TW + c);
+  const int64_t off = Lay<N>::at(0, j, kt * Lay<N>::TW + part * TW + c);
   C v[E];
 #pragma unroll
   for (int e = 0; e < E; e++) v[e] = in[off + (t + Tc * e) * si];
@@ -447,17 +551,17 @@ __global__ void __launch_bounds__(Shape<N>::TW * (N / col_elems<T, N, XP>()),
 // where some n_d = -N/2 when the inverse transform follows; stored as F0.
 // Binned: sum over modes of mult |X|^2 (slot SLOT_P0). Persistent over tiles.
 template <typename T, int N>
-__global__ void __launch_bounds__(Shape<N>::CT, min_blocks<T, Shape<N>::E>(Shape<N>::CT))
+__global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E>(col_threads<T, N>()))
     k_combine_x(const cx<T>* B, cx<T>* F0, const ux<T>* __restrict__ twf, int interlaced, int compensate,
                 int roundtrip, const ux<T>* __restrict__ phase, const cx<T>* __restrict__ invw, BinArgs ba) {
   using C = cx<T>;
   using S = Shape<N>;
-  constexpr int NH = S::NH, E = S::E, Tc = S::Tc, TW = S::TW;
+  constexpr int NH = S::NH, E = S::E, Tc = S::Tc, TW = col_block_tile<T, N>(), SUB = Lay<N>::TW / TW;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   WarpBins<T> wb;
   wb.nk = ba.nk;
-  wb.nwarps = (S::CT + 31) >> 5;
+  wb.nwarps = (TW * Tc + 31) >> 5;
   wb.b = reinterpret_cast<double*>(sm + N * TW);
   wb.w = reinterpret_cast<T*>(wb.b + ba.nk);
   wb.init();
@@ -466,8 +570,8 @@ __global__ void __launch_bounds__(Shape<N>::CT, min_blocks<T, Shape<N>::E>(Shape
   constexpr int64_t si = Lay<N>::XI;
   __syncthreads();
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int kt = tile / N, j = tile - kt * N;  // tiles in storage order
-    const int kz = kt * TW + c;
+    const int st = tile / SUB, kt = st / N, j = st - kt * N;  // tiles in storage order
+    const int kz = kt * Lay<N>::TW + (tile % SUB) * TW + c;
     const int64_t off = Lay<N>::at(0, j, kz);
     C v[E];
 #pragma unroll
@@ -524,29 +628,29 @@ __global__ void __launch_bounds__(Shape<N>::CT, min_blocks<T, Shape<N>::E>(Shape
 template <typename C> __device__ __forceinline__ C f0_for(C f, int odd) { return odd ? mk(-f.y, f.x) : f; }
 
 template <typename T, int N, bool YT, bool XP>
-__global__ void __launch_bounds__(Shape<N>::CT, min_blocks<T, Shape<N>::E>(Shape<N>::CT))
+__global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E>(col_threads<T, N>()))
     k_bin_x(const cx<T>* G, int64_t spec_stride, int ell, int h0, int M, const cx<T>* __restrict__ F0,
             const ux<T>* __restrict__ twf, int slot, BinArgs ba, const float* __restrict__ ytab,
             const __grid_constant__ YTab<T> yt) {
   using C = cx<T>;
   using S = Shape<N>;
-  constexpr int NH = S::NH, E = S::E, Tc = S::Tc, TW = S::TW;
+  constexpr int NH = S::NH, E = S::E, Tc = S::Tc, TW = col_block_tile<T, N>(), SUB = Lay<N>::TW / TW;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   C* sF0 = sm + N * TW;
   WarpBins<T> wb;
   wb.nk = ba.nk;
-  wb.nwarps = (S::CT + 31) >> 5;
+  wb.nwarps = (TW * Tc + 31) >> 5;
   wb.b = reinterpret_cast<double*>(sF0 + N * TW);
   wb.w = reinterpret_cast<T*>(wb.b + ba.nk);
   wb.init();
   const int c = threadIdx.x % TW, t = threadIdx.x / TW;
   constexpr int64_t si = Lay<N>::XI, modes = (int64_t)N * N * NH;
   __syncthreads();
-  for (int q = blockIdx.x; q < ba.n_xtiles; q += gridDim.x) {
-    const int tile = ba.xtiles[q];
+  for (int q = blockIdx.x; q < ba.n_xtiles * SUB; q += gridDim.x) {
+    const int tile = ba.xtiles[q / SUB];
     const int kt = tile / N, j = tile - kt * N;  // x tiles in storage order
-    const int kz = kt * TW + c;
+    const int kz = kt * Lay<N>::TW + (q % SUB) * TW + c;
     const int64_t off = Lay<N>::at(0, j, kz);
     const T fy = T(sfreq<N>(j)), fz = T(kz);
     const T r2yz = fy * fy + fz * fz;
@@ -619,6 +723,118 @@ __global__ void __launch_bounds__(Shape<N>::CT, min_blocks<T, Shape<N>::E>(Shape
     wb.fold();
     __syncthreads();
   }
+  for (int b = threadIdx.x; b < ba.nk; b += blockDim.x) atomicAdd(&ba.bins[slot * ba.nk + b], wb.b[b]);
+}
+
+// ------------------------------------------------------------------ pass x + bin of FP64 contexts (polynomials)
+// Per tile: the coefficients of the powers of x of every r^l Y_lm of the group for the block's TW
+// columns (y, z) into shared memory; for each harmonic the x pass and S += r^l Y_lm Ghat per mode (l/2
+// multiply-adds for the weight, two for S); then Re[S conj(F0)] / r^l goes to the bins, 1/r from a
+// table over |n|^2. The recurrence with its square root and division per mode and harmonic took
+// 20 ms of a 512^3 l <= 4 set's 36 ms in this pass.
+constexpr int kPolyMaxCoef = (2 * kPolyLmax + 1) * poly_np(kPolyLmax);  // per column, all harmonics of one l
+template <int N, int LT>
+__global__ void __launch_bounds__(col_threads<double, N>(), Shape<N>::E == 8 && col_threads<double, N>() <= 256 ? 2 : 1)
+    k_bin_fx(const double2* __restrict__ G, int64_t spec_stride, int ell_in, int h0, int M, const double2* __restrict__ F0,
+             const double2* __restrict__ twf, int slot, BinArgs ba, KPoly kp) {
+  using S_ = Shape<N>;
+  constexpr int E = S_::E, Tc = S_::Tc, TW = col_block_tile<double, N>(), SUB = Lay<N>::TW / TW;
+  const int ell = LT > 0 ? LT : ell_in;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  double2* sm = reinterpret_cast<double2*>(smraw);
+  double* xs = reinterpret_cast<double*>(sm + N * TW);  // [N] x, [N] x^2
+  double* cf = xs + 2 * N;                              // [s][k][TW]
+  WarpBins<double> wb;
+  wb.nk = ba.nk;
+  wb.nwarps = (TW * Tc + 31) >> 5;
+  wb.b = cf + kPolyMaxCoef * TW;
+  wb.w = wb.b + ba.nk;
+  wb.init();
+  const int NP = poly_np(ell), NI = ell + 1;
+  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    const double x = (double)sfreq<N>(i);
+    xs[i] = x;
+    xs[N + i] = x * x;
+  }
+  const int c = threadIdx.x % TW, t = threadIdx.x / TW;
+  constexpr int64_t si = Lay<N>::XI;
+  for (int q = blockIdx.x; q < ba.n_xtiles * SUB; q += gridDim.x) {
+    const int tile = ba.xtiles[q / SUB];
+    const int kt = tile / N, j = tile - kt * N;  // x tiles in storage order
+    const int kz0 = kt * Lay<N>::TW + (q % SUB) * TW, kz = kz0 + c;
+    const int64_t off = Lay<N>::at(0, j, kz);
+    __syncthreads();  // the last tile's coefficients and bins are done with
+    for (int u = threadIdx.x; u < M * NP * TW; u += blockDim.x) {
+      const int cc = u % TW, k = (u / TW) % NP, s = u / (TW * NP);
+      const double y = (double)sfreq<N>(j), z = (double)(kz0 + cc);
+      const int n = ell - (poly_par_x(h0 + s) + 2 * k);  // degree in y and z
+      const double* co = kp.kx + ((h0 + s) * NP + k) * NI;
+      double acc = 0.0;
+      if (n >= 0) {
+        acc = co[n];
+        double zp = 1.0;
+        for (int p = n - 1; p >= 0; p--) {
+          zp *= z;
+          acc = fma(acc, y, co[p] * zp);
+        }
+      }
+      cf[u] = acc;
+    }
+    double2 S[E];
+#pragma unroll
+    for (int e = 0; e < E; e++) S[e] = make_double2(0.0, 0.0);
+    for (int s = 0; s < M; s++) {
+      const double2* Gs = G + (int64_t)s * spec_stride;
+      double2 v[E];
+#pragma unroll
+      for (int e = 0; e < E; e++) v[e] = Gs[off + (t + Tc * e) * si];
+      fft_fx<E, N, kInterleaved, TW, -1>(v, sm, t, c, twf);
+      const int par = poly_par_x(h0 + s);
+      const double* cs = cf + s * NP * TW + c;
+      const int top = (ell - par) >> 1;
+#pragma unroll
+      for (int e = 0; e < E; e++) {
+        const int ii = t + Tc * e;
+        const double x2 = xs[N + ii];
+        double w = cs[top * TW];
+        if constexpr (LT > 0) {
+#pragma unroll
+          for (int k = LT / 2 - 1; k >= 0; k--)
+            if (k < top) w = fma(w, x2, cs[k * TW]);
+        } else {
+          for (int k = top - 1; k >= 0; k--) w = fma(w, x2, cs[k * TW]);
+        }
+        if (par) w *= xs[ii];
+        S[e].x = fma(w, v[e].x, S[e].x);
+        S[e].y = fma(w, v[e].y, S[e].y);
+      }
+    }
+    if (j != N / 2) {
+      const double mult = kz ? 2.0 : 1.0;
+      const int ny = sfreq<N>(j);
+#pragma unroll
+      for (int e = 0; e < E; e++) {
+        const int ii = t + Tc * e;
+        if (ii == N / 2) continue;
+        const int nx = sfreq<N>(ii);
+        const int n2 = nx * nx + ny * ny + kz * kz;
+        const int b = ba.bin_of_n2[n2];
+        if (b >= 0 && n2 > 0) {
+          const double2 f0 = f0_for(F0[off + ii * si], ba.odd);
+          double a = S[e].x * f0.x + S[e].y * f0.y;
+          const double ri = kp.rinv[n2];
+          if (ell & 1) a *= ri;
+          const double ri2 = ri * ri;
+          for (int p = 1; p < ell; p += 2) a *= ri2;
+          if (ba.permode_w) a = per_mode_w2<double, N>(a, static_cast<const double2*>(ba.permode_w), ii, j, kz);
+          wb.add(b, mult * a);
+        }
+      }
+    }
+    __syncthreads();
+    wb.fold();
+  }
+  __syncthreads();
   for (int b = threadIdx.x; b < ba.nk; b += blockDim.x) atomicAdd(&ba.bins[slot * ba.nk + b], wb.b[b]);
 }
 
@@ -757,12 +973,14 @@ template <typename T, int N> struct Passes {
   using C = cx<T>;
   using U = ux<T>;
   using S = Shape<N>;
-  static size_t smem_col() { return (size_t)N * S::TW * sizeof(C); }
-  static size_t smem_bins(int nk, int threads = S::CT) {
+  static constexpr int TWB = col_block_tile<T, N>();  // columns of a y or x block
+  static size_t smem_col() { return (size_t)N * TWB * sizeof(C); }
+  static size_t smem_bins(int nk, int threads = col_threads<T, N>()) {
     return (size_t)nk * sizeof(double) + (size_t)((threads + 31) / 32) * nk * sizeof(T);
   }
   static size_t smem_combine(int nk) { return smem_col() + smem_bins(nk); }
   static size_t smem_bin(int nk) { return 2 * smem_col() + smem_bins(nk); }
+  static size_t smem_bin_fx(int nk) { return smem_col() + (2 * N + kPolyMaxCoef * TWB) * sizeof(double) + smem_bins(nk); }
   // pipelined FP32 pass: two G tiles and two Y tiles (float), then the bins
   static size_t smem_bin_pipe(int nk) {
     return 2 * (size_t)N * S::TW * (sizeof(float2) + sizeof(float)) + (size_t)nk * sizeof(double) +
@@ -788,44 +1006,44 @@ template <typename T, int N> struct Passes {
     else
       c2r_z_v<false>(in, out, twh, twr, scale, s);
   }
+  // staging area or exchange buffer, and in FP64 the coefficients of the rows' polynomials
   static size_t smem_ylm(int M, int rows) {
-    const size_t stage = (size_t)M * rows * N * sizeof(T);
-    const size_t xb = (size_t)M * rows * padded_len(S::NH) * sizeof(C);
-    return stage > xb ? stage : xb;
+    return ylm_stage_bytes<T, N>(M, rows) + (sizeof(T) == 8 ? (size_t)M * rows * poly_np(kPolyLmax) * sizeof(T) : 0);
   }
   template <int LT, bool XP>
   static void ylm_z_v(const T* f, C* out, int64_t stride, int ell, int h0, int M, const U* twh, const U* twr,
-                      const T* axis, int rows, const float* rtab, cudaStream_t s) {
+                      const T* axis, int rows, const float* rtab, const double* poly, cudaStream_t s) {
     const size_t smem = smem_ylm(M, rows);
     const dim3 grid(N * N / rows), block(M * rows * ZRow<T, N, XP>::Tz);
     set_smem(k_ylm_r2c_z<T, N, LT, XP>, smem);
     k_ylm_r2c_z<T, N, LT, XP><<<grid, block, smem, s>>>(f, out, stride, ell, h0, M, twh, twr, axis, rows, rtab,
-                                                         host_ytab<T>());
+                                                         poly, host_ytab<T>());
   }
   template <bool XP>
   static void ylm_z_x(const T* f, C* out, int64_t stride, int ell, int h0, int M, const U* twh, const U* twr,
-                      const T* axis, int rows, const float* rtab, cudaStream_t s) {
+                      const T* axis, int rows, const float* rtab, const double* poly, cudaStream_t s) {
     if (rtab && ell >= 0) {  // weights from the table: no recurrence to specialise
-      ylm_z_v<0, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, rtab, s);
+      ylm_z_v<0, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, rtab, poly, s);
       return;
     }
     switch (ell) {  // the headline multipoles get unrolled recurrences
-      case 2: ylm_z_v<2, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, nullptr, s); break;
-      case 4: ylm_z_v<4, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, nullptr, s); break;
+      case 2: ylm_z_v<2, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, nullptr, poly, s); break;
+      case 4: ylm_z_v<4, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, nullptr, poly, s); break;
       // Cartesian monomials of degree 2 and 4 (h = monomial index)
-      case -2: ylm_z_v<-2, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, nullptr, s); break;
-      case -4: ylm_z_v<-4, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, nullptr, s); break;
-      default: ylm_z_v<0, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, nullptr, s);
+      case -2: ylm_z_v<-2, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, nullptr, poly, s); break;
+      case -4: ylm_z_v<-4, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, nullptr, poly, s); break;
+      default: ylm_z_v<0, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, nullptr, poly, s);
     }
   }
   static void ylm_z(const T* f, C* out, int64_t stride, int ell, int h0, int M, const U* twh, const U* twr,
-                    const T* axis, int rows, const float* rtab, int xp, cudaStream_t s) {
+                    const T* axis, int rows, const float* rtab, const double* poly, int xp, cudaStream_t s) {
     if (sizeof(T) == 4 && xp)
-      ylm_z_x<sizeof(T) == 4>(f, out, stride, ell, h0, M, twh, twr, axis, rows, rtab, s);
+      ylm_z_x<sizeof(T) == 4>(f, out, stride, ell, h0, M, twh, twr, axis, rows, rtab, nullptr, s);
     else
-      ylm_z_x<false>(f, out, stride, ell, h0, M, twh, twr, axis, rows, sizeof(T) == 4 ? rtab : nullptr, s);
+      ylm_z_x<false>(f, out, stride, ell, h0, M, twh, twr, axis, rows, sizeof(T) == 4 ? rtab : nullptr,
+                     sizeof(T) == 8 ? poly : nullptr, s);
   }
-  // variant 0: TW columns per block; variant 1: TW/2 (half the threads and shared memory)
+  // variant 0: TWB columns per block; variant 1: TWB/2 (half the threads and shared memory)
   template <int TWV, bool XP>
   static void fft_y_tw(C* data, int64_t stride, int nspec, const U* twf, int dir, int n2_cut, cudaStream_t s) {
     const size_t smem = (size_t)N * TWV * sizeof(C);
@@ -842,11 +1060,11 @@ template <typename T, int N> struct Passes {
   template <bool XP>
   static void fft_y_x(C* data, int64_t stride, int nspec, const U* twf, int dir, int variant, int n2_cut,
                       cudaStream_t s) {
-    constexpr int TW2 = S::TW > 1 ? S::TW / 2 : 1;
-    if (variant == 1 && S::TW > 1)
+    constexpr int TW2 = TWB > 1 ? TWB / 2 : 1;
+    if (variant == 1 && TWB > 1)
       fft_y_tw<TW2, XP>(data, stride, nspec, twf, dir, n2_cut, s);
     else
-      fft_y_tw<S::TW, XP>(data, stride, nspec, twf, dir, n2_cut, s);
+      fft_y_tw<TWB, XP>(data, stride, nspec, twf, dir, n2_cut, s);
   }
   static void fft_y(C* data, int64_t stride, int nspec, const U* twf, int dir, int variant, int n2_cut, int xp,
                     cudaStream_t s) {
@@ -857,8 +1075,8 @@ template <typename T, int N> struct Passes {
   }
   template <bool XP> static void fft_x_v(const C* in, C* out, const U* twf, int dir, cudaStream_t s) {
     const size_t smem = smem_col();
-    const unsigned grid = N * (S::NH / S::TW);
-    const int threads = S::TW * (N / col_elems<T, N, XP>());
+    const unsigned grid = N * (S::NH / TWB);
+    const int threads = TWB * (N / col_elems<T, N, XP>());
     if (dir < 0) {
       set_smem(k_fft_x<T, N, -1, XP>, smem);
       k_fft_x<T, N, -1, XP><<<grid, threads, smem, s>>>(in, out, twf);
@@ -877,7 +1095,14 @@ template <typename T, int N> struct Passes {
                         const U* phase, const C* invw, const BinArgs& ba, int ctas, cudaStream_t s) {
     const size_t smem = smem_combine(ba.nk);
     set_smem(k_combine_x<T, N>, smem);
-    k_combine_x<T, N><<<ctas, S::CT, smem, s>>>(B, F0, twf, interlaced, compensate, roundtrip, phase, invw, ba);
+    k_combine_x<T, N><<<ctas, col_threads<T, N>(), smem, s>>>(B, F0, twf, interlaced, compensate, roundtrip, phase, invw, ba);
+  }
+  template <int LT>
+  static void bin_fx_v(const C* G, int64_t stride, int ell, int h0, int M, const C* F0, const U* twf, int slot,
+                       const BinArgs& ba, int ctas, const KPoly& kp, cudaStream_t s) {
+    const size_t smem = smem_bin_fx(ba.nk);
+    set_smem(k_bin_fx<N, LT>, smem);
+    k_bin_fx<N, LT><<<ctas, col_threads<T, N>(), smem, s>>>(G, stride, ell, h0, M, F0, twf, slot, ba, kp);
   }
   template <bool XP>
   static void bin_x_v(const C* G, int64_t stride, int ell, int h0, int M, const C* F0, const U* twf, int slot,
@@ -893,14 +1118,26 @@ template <typename T, int N> struct Passes {
     }
     if (ytab && sizeof(T) == 4) {
       set_smem(k_bin_x<T, N, true, XP>, smem);
-      k_bin_x<T, N, true, XP><<<ctas, S::CT, smem, s>>>(G, stride, ell, h0, M, F0, twf, slot, ba, ytab, host_ytab<T>());
+      k_bin_x<T, N, true, XP><<<ctas, col_threads<T, N>(), smem, s>>>(G, stride, ell, h0, M, F0, twf, slot, ba, ytab, host_ytab<T>());
     } else {
       set_smem(k_bin_x<T, N, false, XP>, smem);
-      k_bin_x<T, N, false, XP><<<ctas, S::CT, smem, s>>>(G, stride, ell, h0, M, F0, twf, slot, ba, ytab, host_ytab<T>());
+      k_bin_x<T, N, false, XP><<<ctas, col_threads<T, N>(), smem, s>>>(G, stride, ell, h0, M, F0, twf, slot, ba, ytab, host_ytab<T>());
     }
   }
   static void bin_x(const C* G, int64_t stride, int ell, int h0, int M, const C* F0, const U* twf, int slot,
-                    const BinArgs& ba, int ctas, const float* ytab, int xp, cudaStream_t s) {
+                    const BinArgs& ba, int ctas, const float* ytab, const KPoly& kp, int xp, cudaStream_t s) {
+    if constexpr (sizeof(T) == 8) {
+      if (ell <= kPolyLmax) {
+        KPoly k = kp;
+        k.kx += poly_base(ell);
+        switch (ell) {
+          case 2: bin_fx_v<2>(G, stride, ell, h0, M, F0, twf, slot, ba, ctas, k, s); break;
+          case 4: bin_fx_v<4>(G, stride, ell, h0, M, F0, twf, slot, ba, ctas, k, s); break;
+          default: bin_fx_v<0>(G, stride, ell, h0, M, F0, twf, slot, ba, ctas, k, s);
+        }
+        return;
+      }
+    }
     if (sizeof(T) == 4 && xp)
       bin_x_v<sizeof(T) == 4>(G, stride, ell, h0, M, F0, twf, slot, ba, ctas, ytab, s);
     else
@@ -911,24 +1148,30 @@ template <typename T, int N> struct Passes {
     if (which == 0) {
       const size_t smem = smem_combine(nk);
       set_smem(k_combine_x<T, N>, smem);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_combine_x<T, N>, S::CT, smem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_combine_x<T, N>, col_threads<T, N>(), smem);
     } else if (which == 2 && sizeof(T) == 4 && S::E == 8) {
       if constexpr (sizeof(T) == 4 && S::E == 8) {
         const size_t smem = smem_bin_pipe(nk);
         set_smem(k_bin_x_pipe<N, XP>, smem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_x_pipe<N, XP>, S::CT, smem);
       }
+    } else if (which == 3) {
+      if constexpr (sizeof(T) == 8) {
+        const size_t smem = smem_bin_fx(nk);
+        set_smem(k_bin_fx<N, 4>, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_fx<N, 4>, col_threads<T, N>(), smem);
+      }
     } else if (which == 2) {
       const size_t smem = smem_bin(nk);
       set_smem(k_bin_x<T, N, true, XP>, smem);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_x<T, N, true, XP>, S::CT, smem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_x<T, N, true, XP>, col_threads<T, N>(), smem);
     } else {
       const size_t smem = smem_bin(nk);
       set_smem(k_bin_x<T, N, false, XP>, smem);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_x<T, N, false, XP>, S::CT, smem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_x<T, N, false, XP>, col_threads<T, N>(), smem);
     }
     if (per < 1) per = 1;
-    const int ntiles = N * (S::NH / S::TW);
+    const int ntiles = N * (S::NH / TWB);
     return per * nsm < ntiles ? per * nsm : ntiles;
   }
   static int ctas(int which, int nk, int nsm, int xp) {
@@ -954,6 +1197,7 @@ template <typename T, int N> struct Passes {
     t.ctas = &ctas;
     t.smem_combine = &smem_combine;
     t.smem_bin = &smem_bin;
+    t.smem_bin_fx = &smem_bin_fx;
     t.smem_bin_pipe = &smem_bin_pipe;
     return t;
   }

@@ -172,16 +172,46 @@ void launch_rtab_build(float* rtab, int N, int ell_max, const RGeo& g, int nsm, 
 // Cartesian k-space factors mult_q khat^q of every stored mode, q = 0..20 (kCartItems slots).
 void launch_ctab_build(float* ctab, int N, int tw, int nsm, cudaStream_t s);
 
+// FP64 contexts evaluate Y_lm for l <= kPolyLmax from the polynomials r^l Y_lm(x, y, z) = sum over p, i of
+// C x^p y^i z^(l-p-i): in k space a column's (y, z) are fixed, so the coefficients of the powers of x are
+// formed once per column and each mode costs l/2 multiply-adds; in real space a row's (x, y) are fixed and
+// the powers are those of z. The division by r^l is left to the end. Rounding, rms over random
+// directions relative to the largest |Y|: below the recurrence's up to l = 10 (l = 4: 3.1e-16 against
+// 4.3e-16), above it from l = 12 on (1.5e-15 against 1.3e-15), where the recurrence stays.
+constexpr int kPolyLmax = 10;
+// Coefficients of multipole l in a table: [harmonic h][power p = parity + 2 q, q <= l/2][i <= l].
+__host__ __device__ constexpr int poly_np(int l) { return l / 2 + 1; }
+__host__ __device__ constexpr int poly_base(int l) {
+  int b = 0;
+  for (int k = 1; k < l; k++) b += (2 * k + 1) * poly_np(k) * (k + 1);
+  return b;
+}
+constexpr int kPolyItems = poly_base(kPolyLmax + 1);
+// parity of the power of x (k-space table) or z (real-space table) in harmonic h
+__host__ __device__ constexpr int poly_par_x(int h) { return h == 0 ? 0 : ((h & 1) ? ((h + 1) / 2) & 1 : ((h / 2) + 1) & 1); }
+__host__ __device__ constexpr int poly_par_z(int l, int h) { return (l - (h + 1) / 2) & 1; }
+struct PolyTab {
+  double kx[kPolyItems];  // powers of x; i the power of y
+  double rz[kPolyItems];  // powers of z; i the power of x
+};
+const PolyTab& host_poly();
+
 // Launchers with an `xp` argument run the exact-add FP32 variant of their kernel (xp_engine.cuh)
 // when it is nonzero and T is float; FP64 ignores it.
+// k-space side of the polynomials on the device: the table, and 1/|n| per |n|^2 (0 at 0).
+struct KPoly {
+  const double* kx;
+  const double* rinv;
+};
 template <typename T> struct PassTable {
   int N, E, tw, rows_z, tz;
   int tz_xp;  // threads per row of the exact-add z passes
   void (*r2c_z)(const T*, cx<T>*, const ux<T>*, const ux<T>*, cudaStream_t);
   void (*c2r_z)(const cx<T>*, T*, const ux<T>*, const ux<T>*, T, int, cudaStream_t);
-  // ..., rows, Y_lm(rhat) table slot of the group's first harmonic (FP32) or nullptr, xp
+  // ..., rows, Y_lm(rhat) table slot of the group's first harmonic (FP32) or nullptr, real-space
+  // polynomials (FP64), xp
   void (*ylm_z)(const T*, cx<T>*, int64_t, int, int, int, const ux<T>*, const ux<T>*, const T*, int, const float*,
-                int, cudaStream_t);
+                const double*, int, cudaStream_t);
   size_t (*smem_ylm)(int, int);
   // ..., dir, tile variant, n2_cut (outputs with ny^2 + kz^2 >= n2_cut are not stored), xp
   void (*fft_y)(cx<T>*, int64_t, int, const ux<T>*, int, int, int, int, cudaStream_t);
@@ -189,10 +219,13 @@ template <typename T> struct PassTable {
   void (*combine_x)(const cx<T>*, cx<T>*, const ux<T>*, int, int, int, const ux<T>*, const cx<T>*, const BinArgs&,
                     int, cudaStream_t);
   void (*bin_x)(const cx<T>*, int64_t, int, int, int, const cx<T>*, const ux<T>*, int, const BinArgs&, int,
-                const float*, int, cudaStream_t);  // ..., table slot of the group's first harmonic or nullptr, xp
-  int (*ctas)(int, int, int, int);  // (which: 0 combine, 1 bin, 2 pipelined FP32 bin; nk; SMs; xp) -> persistent blocks
+                const float*, const KPoly&, int, cudaStream_t);  // ..., table slot of the group's first harmonic or nullptr,
+                                                                 // k-space polynomials (FP64), xp
+  // (which: 0 combine, 1 bin, 2 pipelined FP32 bin, 3 FP64 bin with polynomials; nk; SMs; xp) -> persistent blocks
+  int (*ctas)(int, int, int, int);
   size_t (*smem_combine)(int);
   size_t (*smem_bin)(int);
+  size_t (*smem_bin_fx)(int);
   size_t (*smem_bin_pipe)(int);
 };
 template <typename T, int N> const PassTable<T>* pass_table_n();

@@ -57,6 +57,7 @@ struct Plan {
   size_t ytab_bytes = 0, o_ytab = 0, ctab_bytes = 0, o_ctab = 0, rtab_bytes = 0, o_rtab = 0;
   size_t o_xtiles;  // x-pass tiles (j, kz-tile) of the binning pass that hold a binned mode, in order
   size_t o_twh12 = 0, o_twf12 = 0, o_twr12 = 0;  // twiddles of the exact-add stages (FP32)
+  size_t o_poly = 0, o_rinv = 0;                 // Y_lm polynomials, 1/|n| per |n|^2 (FP64)
   size_t o_mesh1, o_mesh2, o_f0, o_w, o_f, o_g, o_twh, o_twf, o_twr, o_axis, o_phase, o_invw, o_bin, o_kmag, o_cnt,
       o_lo, o_hi, o_nmodes, o_ksum, o_sums, o_derived, o_bins, o_out, o_tcnt, o_toff, o_tcur, o_prec, o_ptile,
       o_psort, total;
@@ -74,7 +75,8 @@ struct Plan {
 void set_ctas(Plan* pl, bool f64, int nk, int nsm) {
   if (f64) {
     pl->ctas_comb = pl->td->ctas(0, nk, nsm, 0);
-    pl->ctas_bin = pl->ctas_bin_plain = pl->td->ctas(1, nk, nsm, 0);
+    pl->ctas_bin = pl->td->ctas(3, nk, nsm, 0);
+    pl->ctas_bin_plain = pl->td->ctas(1, nk, nsm, 0);
   } else {
     pl->ctas_comb = pl->tf->ctas(0, nk, nsm, pl->xp);
     pl->ctas_bin = pl->tf->ctas(pl->has_ytab ? 2 : 1, nk, nsm, pl->xp);
@@ -138,7 +140,7 @@ pspec_status build_plan(const pspec_params* p, int max_kbins, int nsm, Plan* pl,
   pl->rtab_bytes = (size_t)N * N * N * sizeof(float) * (size_t)ytab_base((p->ell_max & ~1) + 2);
   pl->has_rtab = !f64 && p->ell_max >= 2 && p->ylm_table == 0 && pl->rtab_bytes <= (size_t)PSPEC_YLM_RTABLE_AUTO_MAX;
   {
-    size_t need = f64 ? std::max(pl->td->smem_bin(max_kbins), pl->td->smem_combine(max_kbins))
+    size_t need = f64 ? std::max({pl->td->smem_bin(max_kbins), pl->td->smem_bin_fx(max_kbins), pl->td->smem_combine(max_kbins)})
                       : std::max(pl->tf->smem_bin(max_kbins), pl->tf->smem_combine(max_kbins));
     if (pl->has_ytab) need = std::max(need, pl->tf->smem_bin_pipe(max_kbins));
     if (need > kSmemMaxBlock) { *why = "max_kbins too large for this mesh (shared memory)"; return PSPEC_EINVAL; }
@@ -166,6 +168,10 @@ pspec_status build_plan(const pspec_params* p, int max_kbins, int nsm, Plan* pl,
     pl->o_twh12 = take(NH * sizeof(float4));
     pl->o_twf12 = take(N * sizeof(float4));
     pl->o_twr12 = take(NH * sizeof(float4));
+  }
+  if (f64) {
+    pl->o_poly = take(sizeof(PolyTab));
+    pl->o_rinv = take((size_t)(pl->n2max + 1) * sizeof(double));
   }
   pl->o_axis = take(3 * (size_t)N * pl->esz);
   pl->o_phase = take(3 * (size_t)N * usz);
@@ -391,6 +397,13 @@ pspec_status upload_tables(Ctx* c) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<float4>(pl.o_twh12), twh12.data(), NH * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<float4>(pl.o_twf12), twf12.data(), N * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<float4>(pl.o_twr12), twr12.data(), NH * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
+  }
+  std::vector<double> rinv;
+  if (sizeof(T) == 8) {
+    rinv.resize(pl.n2max + 1, 0.0);
+    for (int n2 = 1; n2 <= pl.n2max; n2++) rinv[n2] = 1.0 / std::sqrt((double)n2);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<PolyTab>(pl.o_poly), &host_poly(), sizeof(PolyTab), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<double>(pl.o_rinv), rinv.data(), rinv.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream);
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<T>(pl.o_axis), axis.data(), 3 * N * sizeof(T), cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<U>(pl.o_phase), phase.data(), 3 * N * sizeof(U), cudaMemcpyHostToDevice, c->stream);
@@ -658,6 +671,8 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
   const int ctas_bin = c->tune.bin_blocks_per_sm > 0 ? std::min(ntiles_x, c->tune.bin_blocks_per_sm * c->nsm)
                                                      : pl.ctas_bin;
   const int ctas_bin_plain = c->tune.bin_blocks_per_sm > 0 ? ctas_bin : pl.ctas_bin_plain;
+  constexpr bool f64 = sizeof(T) == 8;
+  const KPoly kpoly = f64 ? KPoly{c->at<PolyTab>(pl.o_poly)->kx, c->at<double>(pl.o_rinv)} : KPoly{nullptr, nullptr};
   auto acc = [&](double b) {
     bytes += b;
     return b;
@@ -729,6 +744,7 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
       const int tz = pl.xp ? PT->tz_xp : PT->tz;
       const int cap = ylm_thread_cap(ell);
       const int ms_max = std::max(1, std::min(c->tune.ylm_harmonics, cap / tz));
+      const double* rpoly = f64 && ell <= kPolyLmax ? c->at<PolyTab>(pl.o_poly)->rz + poly_base(ell) : nullptr;
       for (int hs = 0; hs < M; hs += ms_max) {
         const int Ms = std::min(ms_max, M - hs);
         int rows = std::max(1, pow2_floor(std::max(1, cap / (Ms * tz))));
@@ -738,7 +754,7 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
                               ? c->at<float>(pl.o_rtab) + (int64_t)(ytab_base(ell) + h0 + hs) * N * N * N
                               : nullptr;
         TRY(run(c, PSPEC_K_YLM_Z, acc(Sr + Ms * Sc + (rt ? Ms * (double)N * N * N * sizeof(float) : 0.0)), [&] {
-          PT->ylm_z(f, G + hs * stride, stride, ell, h0 + hs, Ms, twh_x, twr_x, axis, rows, rt, pl.xp, s);
+          PT->ylm_z(f, G + hs * stride, stride, ell, h0 + hs, Ms, twh_x, twr_x, axis, rows, rt, rpoly, pl.xp, s);
         }));
       }
       TRY(run(c, PSPEC_K_FFT_Y, acc(M * Sc * (c->frac_yr + c->frac_yw)),
@@ -748,7 +764,8 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
       BinArgs bj = ba;
       bj.odd = ell > 0 && (ell & 1);
       TRY(run(c, PSPEC_K_BIN_X, acc((Sc + M * Sc + ybytes) * c->frac_tile), [&] {
-        PT->bin_x(G, stride, ell, h0, M, F0, twf_x, jobs[jb].slot, bj, ytab ? ctas_bin : ctas_bin_plain, ytab, pl.xp, s);
+        PT->bin_x(G, stride, ell, h0, M, F0, twf_x, jobs[jb].slot, bj,
+                  ytab || (f64 && ell <= kPolyLmax) ? ctas_bin : ctas_bin_plain, ytab, kpoly, pl.xp, s);
       }));
       transforms += M;
     }
