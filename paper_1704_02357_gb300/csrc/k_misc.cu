@@ -550,25 +550,31 @@ __global__ void __launch_bounds__(1024) k_ptile_scan(TileArgs ta, int ntiles) {
   const unsigned at = base + (w ? wsum[w - 1] : 0u) + inc - n;
   ta.off[i] = at;
   ta.cursor[i] = at;
+  ta.cursor[ntiles + i] = at + n;
 }
 
 // Each record goes to every tile its footprint touches (the order within a tile is free: the
-// tile's sums are exact).
+// tile's sums are exact): a record that touches one tile only to the front of that tile's range, the
+// copies of the others to its back, so that the tile paint runs the front without tests.
 __global__ void __launch_bounds__(256) k_ptile_scatter(TileArgs ta, int64_t total, const DevCat* dc, const int* cur,
                                                        int N) {
   if (dc) total = dc[*cur].count;
-  const int nts = N / kPT;
+  const int nts = N / kPT, ntiles = nts * nts * nts;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < total; p += (int64_t)gridDim.x * blockDim.x) {
     const unsigned t = ta.tile_of[p];
     if (t == kNoTile) continue;
     const uint4 r = ta.rec[p];
+    if (!((r.x | r.y | r.z) & kSpan2)) {
+      ta.sorted[atomicAdd(&ta.cursor[t], 1u)] = r;
+      continue;
+    }
     const int tb[3] = {(int)(t / (nts * nts)), (int)((t / nts) % nts), (int)(t % nts)};
     const int sx = (r.x & kSpan2) ? 2 : 1, sy = (r.y & kSpan2) ? 2 : 1, sz = (r.z & kSpan2) ? 2 : 1;
     for (int dx = 0; dx < sx; dx++)
       for (int dy = 0; dy < sy; dy++)
         for (int dz = 0; dz < sz; dz++) {
           const int tt = ((((tb[0] + dx) % nts) * nts + (tb[1] + dy) % nts) * nts) + (tb[2] + dz) % nts;
-          const unsigned pos = atomicAdd(&ta.cursor[tt], 1u);
+          const unsigned pos = atomicSub(&ta.cursor[ntiles + tt], 1u) - 1u;
           ta.sorted[pos] = make_uint4((r.x & kCoordMask) | (dx ? kNextTile : 0u),
                                       (r.y & kCoordMask) | (dy ? kNextTile : 0u),
                                       (r.z & kCoordMask) | (dz ? kNextTile : 0u), r.w);
@@ -591,7 +597,7 @@ __device__ __forceinline__ void tile_nodes(int V, int* idx, float* w) {
     const int c = (V + (1 << 23)) >> 24;
     const float d = (float)(V - c * 16777216) * 5.9604644775390625e-8f;
     w[0] = 0.5f * (0.5f - d) * (0.5f - d);
-    w[1] = 0.75f - d * d;
+    w[1] = __fmaf_rn(-d, d, 0.75f);  // one rounding, whatever the compiler contracts elsewhere
     w[2] = 0.5f * (0.5f + d) * (0.5f + d);
     idx[0] = c - 1;
     idx[1] = c;
@@ -613,29 +619,72 @@ __device__ __forceinline__ void add64(unsigned* acc, int c, int hi_off, long lon
   if (h) atomicAdd(acc + c + hi_off, h);
 }
 
-// The contribution v wx wy wz (FP32, rounded as the direct paint rounds it) in units of 2^-S.
-template <int WIN>
+// |X| rounded to an integer (nearest, ties to even) for 0 <= X < 2^62, as f2ll_rn_int. Nearly every
+// contribution has an exponent past its 24 bits (X >= 2^23) and only shifts.
+__device__ __forceinline__ unsigned long long f2ull_mag(float X) {
+  const unsigned b = __float_as_uint(X);
+  const int sh = (int)(b >> 23) - 150;
+  if (sh >= 0) return (unsigned long long)((b & 0x7fffffu) | 0x800000u) << sh;
+  return __float2uint_rn(X);
+}
+
+// The contributions v wx wy wz (FP32, rounded as the direct paint rounds them) in units of 2^-S;
+// vs = |v| 2^S (a power of two: the products round alike), neg its sign. FULL: every cell lies in
+// the tile.
+template <int WIN, bool FULL>
 __device__ __forceinline__ void tile_scatter(unsigned* acc, int hi_off, const int (&ix)[3], const int (&iy)[3],
                                              const int (&iz)[3], const float (&wx)[3], const float (&wy)[3],
-                                             const float (&wz)[3], float v, float scale) {
+                                             const float (&wz)[3], float vs, bool neg) {
   constexpr int K = WIN == PSPEC_WINDOW_CIC ? 2 : 3;
 #pragma unroll
   for (int a = 0; a < K; a++) {
-    if (!in_tile(ix[a])) continue;
-    const float va = v * wx[a];
+    if (!FULL && !in_tile(ix[a])) continue;
+    const float va = vs * wx[a];
 #pragma unroll
     for (int b = 0; b < K; b++) {
-      if (!in_tile(iy[b])) continue;
+      if (!FULL && !in_tile(iy[b])) continue;
       const float vb = va * wy[b];
       const int row = (ix[a] * kPT + iy[b]) * kPT;
 #pragma unroll
       for (int c = 0; c < K; c++) {
-        if (!in_tile(iz[c])) continue;
-        add64(acc, row + iz[c], hi_off, f2ll_rn_int((vb * wz[c]) * scale));
+        if (!FULL && !in_tile(iz[c])) continue;
+        const unsigned long long q = f2ull_mag(vb * wz[c]);
+        add64(acc, row + iz[c], hi_off, (long long)(neg ? 0ull - q : q));
       }
     }
   }
 }
+
+// Both meshes' contributions of one record.
+template <int WIN, bool INTER, bool FULL>
+__device__ __forceinline__ void tile_record(unsigned* acc, const uint4 r, float scale) {
+  constexpr int HI = (INTER ? 2 : 1) * kPT3;
+  const float v = __uint_as_float(r.w), vs = fabsf(v) * scale;
+  const bool neg = (r.w >> 31) != 0u;
+  int V[3] = {(int)(r.x & kCoordMask), (int)(r.y & kCoordMask), (int)(r.z & kCoordMask)};
+  if (!FULL) {
+    V[0] -= (r.x & kNextTile) ? (kPT << 24) : 0;
+    V[1] -= (r.y & kNextTile) ? (kPT << 24) : 0;
+    V[2] -= (r.z & kNextTile) ? (kPT << 24) : 0;
+  }
+  int ix[3], iy[3], iz[3];
+  float wx[3], wy[3], wz[3];
+  tile_nodes<WIN>(V[0], ix, wx);
+  tile_nodes<WIN>(V[1], iy, wy);
+  tile_nodes<WIN>(V[2], iz, wz);
+  tile_scatter<WIN, FULL>(acc, HI, ix, iy, iz, wx, wy, wz, vs, neg);
+  if (INTER) {
+    const int h = 1 << 23;  // half a cell
+    tile_nodes<WIN>(V[0] - h, ix, wx);
+    tile_nodes<WIN>(V[1] - h, iy, wy);
+    tile_nodes<WIN>(V[2] - h, iz, wz);
+    tile_scatter<WIN, FULL>(acc + kPT3, HI, ix, iy, iz, wx, wy, wz, vs, neg);
+  }
+}
+
+// Threads of a tile's block: three blocks' accumulators (64 KB each with interlacing) fit an SM, and the
+// shared atomics need the warps: 512 threads keep 48 warps resident, 256 kept 24.
+constexpr int kTilePaintThreads = 512;
 
 // One block per tile (every tile, so that empty tiles store their zeros): sums its records into
 // shared 64-bit accumulators (lo words of both meshes, then hi words), then stores each cell of
@@ -644,7 +693,7 @@ __device__ __forceinline__ void tile_scatter(unsigned* acc, int hi_off, const in
 // cell - alpha * randoms cell instead: the same FMA as a pass of its own over the meshes, which
 // would read and write each once more (135 us a mesh at 384^3).
 template <int WIN, bool INTER>
-__global__ void __launch_bounds__(256) k_ptile_paint(TileArgs ta, float* __restrict__ m1, float* __restrict__ m2,
+__global__ void __launch_bounds__(kTilePaintThreads, INTER ? 3 : 4) k_ptile_paint(TileArgs ta, float* __restrict__ m1, float* __restrict__ m2,
                                                      int N, const double* __restrict__ fix,
                                                      const float* __restrict__ r1, const float* __restrict__ r2,
                                                      const double* __restrict__ alpha) {
@@ -683,26 +732,9 @@ __global__ void __launch_bounds__(256) k_ptile_paint(TileArgs ta, float* __restr
   const float scale = (float)sc, inv = (float)(1.0 / sc);  // powers of two: exact
   for (int i = threadIdx.x; i < 2 * NM * kPT3 / 4; i += blockDim.x) reinterpret_cast<uint4*>(acc)[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
-  for (unsigned q = threadIdx.x; q < n; q += blockDim.x) {
-    const uint4 r = ta.sorted[o + q];
-    const float v = __uint_as_float(r.w);
-    const int V[3] = {(int)(r.x & kCoordMask) - ((r.x & kNextTile) ? (kPT << 24) : 0),
-                      (int)(r.y & kCoordMask) - ((r.y & kNextTile) ? (kPT << 24) : 0),
-                      (int)(r.z & kCoordMask) - ((r.z & kNextTile) ? (kPT << 24) : 0)};
-    int ix[3], iy[3], iz[3];
-    float wx[3], wy[3], wz[3];
-    tile_nodes<WIN>(V[0], ix, wx);
-    tile_nodes<WIN>(V[1], iy, wy);
-    tile_nodes<WIN>(V[2], iz, wz);
-    tile_scatter<WIN>(acc, HI, ix, iy, iz, wx, wy, wz, v, scale);
-    if (INTER) {
-      const int h = 1 << 23;  // half a cell
-      tile_nodes<WIN>(V[0] - h, ix, wx);
-      tile_nodes<WIN>(V[1] - h, iy, wy);
-      tile_nodes<WIN>(V[2] - h, iz, wz);
-      tile_scatter<WIN>(acc + kPT3, HI, ix, iy, iz, wx, wy, wz, v, scale);
-    }
-  }
+  const unsigned nf = ta.cursor[tile] - o;  // records that touch this tile only
+  for (unsigned q = threadIdx.x; q < nf; q += blockDim.x) tile_record<WIN, INTER, true>(acc, ta.sorted[o + q], scale);
+  for (unsigned q = nf + threadIdx.x; q < n; q += blockDim.x) tile_record<WIN, INTER, false>(acc, ta.sorted[o + q], scale);
   __syncthreads();
   for (int i = threadIdx.x; i < NM * kPT3 / 4; i += blockDim.x) {
     int mesh;
@@ -756,16 +788,16 @@ void launch_ptile_paint(const TileArgs& ta, int window, int interlaced, float* m
   if (window == PSPEC_WINDOW_CIC) {
     if (interlaced) {
       set_smem_attr(k_ptile_paint<PSPEC_WINDOW_CIC, true>, smem);
-      k_ptile_paint<PSPEC_WINDOW_CIC, true><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
+      k_ptile_paint<PSPEC_WINDOW_CIC, true><<<ntiles, kTilePaintThreads, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
     } else {
-      k_ptile_paint<PSPEC_WINDOW_CIC, false><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
+      k_ptile_paint<PSPEC_WINDOW_CIC, false><<<ntiles, kTilePaintThreads, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
     }
   } else {
     if (interlaced) {
       set_smem_attr(k_ptile_paint<PSPEC_WINDOW_TSC, true>, smem);
-      k_ptile_paint<PSPEC_WINDOW_TSC, true><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
+      k_ptile_paint<PSPEC_WINDOW_TSC, true><<<ntiles, kTilePaintThreads, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
     } else {
-      k_ptile_paint<PSPEC_WINDOW_TSC, false><<<ntiles, 256, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
+      k_ptile_paint<PSPEC_WINDOW_TSC, false><<<ntiles, kTilePaintThreads, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
     }
   }
 }

@@ -100,7 +100,7 @@ constexpr int kPaintRecordsMax = 8;
 struct TileArgs {
   unsigned* cnt;     // [ntiles + 1] records per tile, then the records placed so far (cleared before prep)
   unsigned* off;     // [ntiles] first record of the tile in the sorted copy
-  unsigned* cursor;  // [ntiles] scatter cursors
+  unsigned* cursor;  // [2][ntiles] scatter cursors: the front of a tile's range upwards, its back downwards
   uint4* rec;        // [particles] records in input order
   unsigned* tile_of; // [particles] first tile of each record (all ones: left out)
   uint4* sorted;     // [kPaintRecordsMax * particles] records in tile order

@@ -198,7 +198,7 @@ pspec_status build_plan(const pspec_params* p, int max_kbins, int nsm, Plan* pl,
   if (pl->max_particles > 0) {
     pl->o_tcnt = take((size_t)(pl->ntiles + 1) * sizeof(unsigned));
     pl->o_toff = take((size_t)pl->ntiles * sizeof(unsigned));
-    pl->o_tcur = take((size_t)pl->ntiles * sizeof(unsigned));
+    pl->o_tcur = take(2 * (size_t)pl->ntiles * sizeof(unsigned));
     pl->o_prec = take((size_t)pl->max_particles * 16);
     pl->o_ptile = take((size_t)pl->max_particles * sizeof(unsigned));
     pl->o_psort = take((size_t)pl->max_particles * kPaintRecordsMax * 16);
