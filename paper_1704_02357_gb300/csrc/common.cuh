@@ -323,4 +323,20 @@ template <> __device__ __forceinline__ float rsqrt_t<float>(float x) {
 template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return 1.0 / sqrt(x); }
 
 
+// 1/x and 1/sqrt(x) of a positive normal FP64 number: the hardware's approximation (about 20 bits) and
+// two Newton steps, within an ulp or two. (The divisions and square roots of the library take three
+// times the FP64 operations; the pipe runs two per clock and SM.)
+__device__ __forceinline__ double rcp_newton(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+__device__ __forceinline__ double rsqrt_newton(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(0.5 * y, fma(-(x * y), y, 1.0), y);
+  return fma(0.5 * y, fma(-(x * y), y, 1.0), y);
+}
+
 }  // namespace pspec

@@ -64,10 +64,11 @@ PSPEC_HD int ic_clz64(unsigned long long a) {
 // 1023 + max_log2.
 PSPEC_HD bool exp_below(double t, int max_log2) { return (int)((ic_bits(t) >> 52) & 0x7ff) < 1023 + max_log2; }
 
-// round to nearest, ties to even, of a finite double with |t| < 2^62
-PSPEC_HD long long d2ll_rn_int(double t) {
+// round to nearest, ties to even, of t 2^k for a finite double t with |t| 2^k < 2^62 (k >= 0): the
+// power of two is added to the exponent
+PSPEC_HD long long d2ll_rn_scaled(double t, int k) {
   const unsigned long long b = ic_bits(t);
-  const int e = (int)((b >> 52) & 0x7ff);
+  const int f = (int)((b >> 52) & 0x7ff), e = f ? f + k : 0;  // subnormal t: 0, as |t| 2^k < 1/2
   const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;  // 53 bits
   long long q;
   if (e >= 1075) {
@@ -80,6 +81,32 @@ PSPEC_HD long long d2ll_rn_int(double t) {
     q = (long long)(r + (unsigned long long)((rem > half) | ((rem == half) & (r & 1ull))));
   }
   return (b >> 63) ? -q : q;
+}
+
+// round to nearest, ties to even, of a finite double with |t| < 2^62
+PSPEC_HD long long d2ll_rn_int(double t) { return d2ll_rn_scaled(t, 0); }
+
+// The two floats around v and the chance of the upper-magnitude choice, from the bits of v: lo = v rounded to
+// the nearest float (ties to even), hi = the neighbouring float on the other side of v (lo itself when
+// v is a float), thr = |v - lo| / |hi - lo| 2^32. Needs a float exponent that is normal on both sides.
+struct FloatPair {
+  float lo, hi;
+  unsigned thr;
+};
+PSPEC_HD bool float_pair_ok(double v) {
+  const int e = (int)((ic_bits(v) >> 52) & 0x7ff) - 1023;
+  return e > -126 && e < 127;
+}
+PSPEC_HD FloatPair float_pair(double v) {
+  const unsigned long long b = ic_bits(v);
+  const unsigned t = ((unsigned)(b >> 63) << 31) | (unsigned)(((b & 0x7fffffffffffffffull) >> 29) - ((unsigned long long)896 << 23));
+  const unsigned f = (unsigned)(b & 0x1fffffffull);
+  const bool up = f > (1u << 28) || (f == (1u << 28) && (t & 1u));
+  FloatPair p;
+  p.lo = ic_float(up ? t + 1u : t);
+  p.hi = ic_float(up ? t : (f ? t + 1u : t));
+  p.thr = (up ? (1u << 29) - f : f) << 3;
+  return p;
 }
 
 // round to nearest, ties to even, of a finite float with |f| < 2^62

@@ -236,22 +236,6 @@ template <typename T, int N> __host__ __device__ constexpr size_t ylm_stage_byte
                                                                               : padded_len(N / 2) * sizeof(cx<T>));
 }
 
-// 1/x and 1/sqrt(x) of a positive normal FP64 number: the hardware's approximation (about 20 bits) and
-// two Newton steps, within an ulp or two. (The divisions and square roots of the library take three
-// times the FP64 operations; the pipe runs two per clock and SM.)
-__device__ __forceinline__ double rcp_newton(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
-}
-__device__ __forceinline__ double rsqrt_newton(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(0.5 * y, fma(-(x * y), y, 1.0), y);
-  return fma(0.5 * y, fma(-(x * y), y, 1.0), y);
-}
-
 // f Y_lm(rhat) of `rows` rows and M harmonics into the staging area (FP64 contexts): per row the
 // coefficients of the powers of z of each r^l Y_lm, then per node l/2 multiply-adds a harmonic at most and
 // one product with f / r^l (times z for odd powers). All threads of the block. 25 FP64 operations a

@@ -14,12 +14,12 @@ constexpr int kSumThreads = 256;
 // non-finite ones): beyond it the periodic reduction of the grid coordinate loses meaning.
 constexpr int kMaxCellsLog2 = 38;  // |u| < 2^38 cells for a valid particle
 
-// Grid coordinate of a position along one axis in units of 2^-24 cell, t = u 2^24 with
-// u = (x - corner) N/L in FP64 (the power-of-two scaling is exact). A particle is valid when every
-// |t| is below 2^62 (|u| < 2^kMaxCellsLog2 cells; NaN and infinities fail), tested on the exponent
+// Grid coordinate of a position along one axis, u = (x - corner) N/L in FP64; the paint takes it to
+// an integer in units of 2^-24 cell (grid_int, the power of two goes to the exponent). A particle is valid
+// when every |u| is below 2^kMaxCellsLog2 cells (NaN and infinities fail), tested on the exponent
 // bits. The test and the conversions (intconv.cuh) use integer instructions: GB300's FP64 pipe is
 // narrow, and FP64 compares and conversions between FP64 or FP32 and 64-bit integers all run on it. (One FMA,
-// x K - corner K with K = 2^24 N/L, gives the same t but for rare last-bit ties; measured over 30
+// x K - corner K with K = N/L, gives the same u but for rare last-bit ties; measured over 30
 // axis-permutation draws of the 512^3 survey catalogs, the FP32 results then came out with higher
 // median errors, so the two-operation form is kept.)
 struct GridMap {
@@ -29,9 +29,10 @@ struct GridMap {
     c[1] = a.corner[1];
     c[2] = a.corner[2];
   }
-  __device__ __forceinline__ double t(double x, int d) const { return ((x - c[d]) * inv) * 16777216.0; }
+  __device__ __forceinline__ double u(double x, int d) const { return (x - c[d]) * inv; }
 };
-__device__ __forceinline__ bool grid_ok(double t) { return exp_below(t, kMaxCellsLog2 + 24); }
+__device__ __forceinline__ bool grid_ok(double u) { return exp_below(u, kMaxCellsLog2); }
+__device__ __forceinline__ long long grid_int(double u) { return d2ll_rn_scaled(u, 24); }
 
 __device__ __forceinline__ void load_pos(const PaintArgs& a, int64_t p, double& x, double& y, double& z) {
   if (a.pos_f32) {
@@ -60,8 +61,13 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 }
 
 __device__ __forceinline__ double fkp_w(const PaintArgs& a, double nb) {
-  return a.nbar ? (a.P0 > 0.0 ? 1.0 / (1.0 + nb * a.P0) : 1.0) : a.wf_default;
+  if (!a.nbar) return a.wf_default;
+  if (!(a.P0 > 0.0)) return 1.0;
+  const double x = 1.0 + nb * a.P0;
+  const unsigned e = (unsigned)(__double2hiint(x) >> 20);  // sign and exponent
+  return e - 923u < 200u ? rcp_newton(x) : 1.0 / x;         // 2^-100 <= x < 2^100: the rule
 }
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
 // The FP32 mesh value of one particle: v rounded down or up to a neighbouring float, chosen
 // by a hash of (particle, catalog) with the probabilities that make its expectation v. All
@@ -71,11 +77,9 @@ __device__ __forceinline__ double fkp_w(const PaintArgs& a, double nb) {
 // the rounding errors are independent across particles and only add white noise ~1e-7 of the
 // shot noise. The hash is the 32-bit finaliser of MurmurHash3 (Appleby) applied to the
 // particle index mixed with a per-catalog salt.
-struct Dither {
-  float lo, hi;    // the two floats around v (equal when v is a float)
-  uint32_t thr;    // P(hi) * 2^32
-};
+using Dither = FloatPair;  // lo, hi: the two floats around v (equal when v is a float); thr: P(hi) 2^32
 __device__ __forceinline__ Dither dither_of(double v) {
+  if (float_pair_ok(v)) return float_pair(v);  // integer instructions, no FP64 division
   Dither d;
   d.lo = (float)v;
   const double r = v - (double)d.lo;
@@ -114,25 +118,59 @@ __device__ __forceinline__ PaintArgs resolve(const PaintArgs& in) {
 // Per-block partials: [0] sum w_c, [1] sum v^2 (v = w_c w_fkp), [2] sum nbar w_c w_fkp^2,
 // [3] sum |v| (bounds every mesh value, for the fixed-point scale of the exact paint).
 // Invalid particles are left out here and counted by the paint kernel.
+// A particle whose coordinates are all below 2^safe_log2 is valid without FP64 arithmetic; a
+// catalog without weights and n̄ is then only counted.
 __global__ void __launch_bounds__(kSumThreads) k_catalog_partials(PaintArgs a_in, double* out) {
   __shared__ double red[kSumThreads / 32];
   const PaintArgs a = resolve(a_in);
   const GridMap gm(a);
+  const bool uniform = (a.weight == nullptr) && (a.nbar == nullptr);
+  const int lim32 = a.safe_log2 > 126 ? 253 : a.safe_log2 + 127, lim64 = a.safe_log2 + 1023;
   double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.count;
-       p += (int64_t)gridDim.x * blockDim.x) {
+  int n = 0;
+  auto valid = [&](int64_t p) {
+    if (a.pos_f32) {
+      const unsigned* q = static_cast<const unsigned*>(a.pos) + 3 * p;
+      const int e0 = (q[0] >> 23) & 0xff, e1 = (q[1] >> 23) & 0xff, e2 = (q[2] >> 23) & 0xff;
+      if (max(e0, max(e1, e2)) < lim32) return true;
+    } else {
+      const double* q = static_cast<const double*>(a.pos) + 3 * p;
+      const int e0 = (__double2hiint(q[0]) >> 20) & 0x7ff, e1 = (__double2hiint(q[1]) >> 20) & 0x7ff,
+                e2 = (__double2hiint(q[2]) >> 20) & 0x7ff;
+      if (max(e0, max(e1, e2)) < lim64) return true;
+    }
     double x, y, z;
     load_pos(a, p, x, y, z);
+    return grid_ok(gm.u(x, 0)) && grid_ok(gm.u(y, 1)) && grid_ok(gm.u(z, 2));
+  };
+#pragma unroll 2
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.count;
+       p += (int64_t)gridDim.x * blockDim.x) {
+    if (uniform) {
+      n += valid(p) ? 1 : 0;
+      continue;
+    }
     const double wc = a.weight ? a.weight[p] : 1.0;
     const double nb = a.nbar ? a.nbar[p] : a.nbar_default;
-    if (!(grid_ok(gm.t(x, 0)) && grid_ok(gm.t(y, 1)) && grid_ok(gm.t(z, 2)) && isfinite(wc) && isfinite(nb)))
-      continue;
+    if (!(valid(p) && finite_bits(wc) && finite_bits(nb))) continue;
     const double wf = fkp_w(a, nb);
     const double v = wc * wf;
     s0 += wc;
     s1 += v * v;
-    s2 += nb * wc * wf * wf;
+    s2 += nb * v * wf;
     s3 += fabs(v);
+  }
+  if (uniform) {
+    const double m = block_sum((double)n, red);
+    if (threadIdx.x == 0) {
+      const double wf = a.wf_default;
+      double* o = out + (int64_t)blockIdx.x * kSumVals;
+      o[0] = m;
+      o[1] = m * (wf * wf);
+      o[2] = m * (a.nbar_default * wf * wf);
+      o[3] = m * fabs(wf);
+    }
+    return;
   }
   const double r0 = block_sum(s0, red);
   const double r1 = block_sum(s1, red);
@@ -349,8 +387,8 @@ __global__ void __launch_bounds__(256) k_paint(PaintArgs a_in, int is_randoms, d
       wc = a.weight ? a.weight[p] : 1.0;
       nb = a.nbar ? a.nbar[p] : a.nbar_default;
     }
-    const double tx = gm.t(x, 0), ty = gm.t(y, 1), tz = gm.t(z, 2);
-    if (!(grid_ok(tx) && grid_ok(ty) && grid_ok(tz) && (uniform || (isfinite(wc) && isfinite(nb))))) {
+    const double ux = gm.u(x, 0), uy = gm.u(y, 1), uz = gm.u(z, 2);
+    if (!(grid_ok(ux) && grid_ok(uy) && grid_ok(uz) && (uniform || (finite_bits(wc) && finite_bits(nb))))) {
       bad++;
       continue;
     }
@@ -362,7 +400,7 @@ __global__ void __launch_bounds__(256) k_paint(PaintArgs a_in, int is_randoms, d
     int ix[3], iy[3], iz[3];
     T wx[3], wy[3], wz[3];
     if constexpr (sizeof(T) == 4) {
-      const int64_t Ux = d2ll_rn_int(tx), Uy = d2ll_rn_int(ty), Uz = d2ll_rn_int(tz);
+      const int64_t Ux = grid_int(ux), Uy = grid_int(uy), Uz = grid_int(uz);
       if (Ux < 0 || Ux >= lim24 || Uy < 0 || Uy >= lim24 || Uz < 0 || Uz >= lim24) out++;
       Axis<float, WIN>::nodes(Ux, N, ix, wx);
       Axis<float, WIN>::nodes(Uy, N, iy, wy);
@@ -376,8 +414,6 @@ __global__ void __launch_bounds__(256) k_paint(PaintArgs a_in, int is_randoms, d
         scatter<T, WIN>(m2, N, ix, iy, iz, wx, wy, wz, v);
       }
     } else {
-      const double ux = tx * 5.9604644775390625e-8, uy = ty * 5.9604644775390625e-8,
-                   uz = tz * 5.9604644775390625e-8;  // 2^-24: exact
       const double lim = (double)N;
       if (ux < 0.0 || ux >= lim || uy < 0.0 || uy >= lim || uz < 0.0 || uz >= lim) out++;
       Axis<double, WIN>::nodes(ux, N, ix, wx);
@@ -460,17 +496,37 @@ __device__ __forceinline__ void footprint(int64_t U, int64_t& lo, int64_t& hi) {
   }
 }
 
-template <int WIN, bool INTER>
-__global__ void __launch_bounds__(256) k_ptile_prep(PaintArgs a_in, int is_randoms, double* __restrict__ derived,
-                                                    TileArgs ta, int64_t offset, int N) {
-  const PaintArgs a = resolve(a_in);
+// Catalogs of one prep launch (blockIdx.y): their records follow one another.
+struct PrepArgs {
+  PaintArgs a[2];
+  int kind[2];
+};
+// Meshes of up to this many tiles (256^3) count and place records per block in shared memory first: few
+// tiles mean many records each, and the global counter of a tile then takes one atomic add per block
+// instead of one per record (0.4 million galaxies on 128^3, whose densest tiles hold thousands:
+// prep 95 -> 12 us, scatter 94 -> 15 us).
+constexpr int kSharedTiles = 4096;
+
+template <int WIN, bool INTER, bool SHARED>
+__global__ void __launch_bounds__(512) k_ptile_prep(const __grid_constant__ PrepArgs pa, double* __restrict__ derived,
+                                                    TileArgs ta, int N) {
+  extern __shared__ __align__(16) unsigned hist[];  // SHARED: records per tile of this block
+  const PaintArgs a = resolve(pa.a[blockIdx.y]);
+  const int is_randoms = pa.kind[blockIdx.y];
+  const int64_t offset = blockIdx.y ? pa.a[0].count : 0;
   const double sign = is_randoms == 1 ? -derived[D_ALPHA] : 1.0;
   const bool uniform = (a.weight == nullptr) && (a.nbar == nullptr);
   const double v_uniform = sign * a.wf_default;
   const Dither d_uniform = dither_of(v_uniform);
   const GridMap gm(a);
   const int64_t lim24 = (int64_t)N << 24;
-  const int nts = N / kPT;
+  const int nts = N / kPT, ntiles = nts * nts * nts;
+  unsigned* cnt = SHARED ? hist : ta.cnt;
+  if (SHARED) {
+    if ((int64_t)blockIdx.x * blockDim.x >= a.count) return;  // uniform over the block
+    for (int i = threadIdx.x; i < ntiles; i += blockDim.x) hist[i] = 0u;
+    __syncthreads();
+  }
   unsigned bad = 0, out = 0;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.count;
        p += (int64_t)gridDim.x * blockDim.x) {
@@ -481,13 +537,13 @@ __global__ void __launch_bounds__(256) k_ptile_prep(PaintArgs a_in, int is_rando
       wc = a.weight ? a.weight[p] : 1.0;
       nb = a.nbar ? a.nbar[p] : a.nbar_default;
     }
-    const double tt[3] = {gm.t(x, 0), gm.t(y, 1), gm.t(z, 2)};
-    if (!(grid_ok(tt[0]) && grid_ok(tt[1]) && grid_ok(tt[2]) && (uniform || (isfinite(wc) && isfinite(nb))))) {
+    const double uu[3] = {gm.u(x, 0), gm.u(y, 1), gm.u(z, 2)};
+    if (!(grid_ok(uu[0]) && grid_ok(uu[1]) && grid_ok(uu[2]) && (uniform || (finite_bits(wc) && finite_bits(nb))))) {
       bad++;
       ta.tile_of[offset + p] = kNoTile;
       continue;
     }
-    const int64_t Ud[3] = {d2ll_rn_int(tt[0]), d2ll_rn_int(tt[1]), d2ll_rn_int(tt[2])};
+    const int64_t Ud[3] = {grid_int(uu[0]), grid_int(uu[1]), grid_int(uu[2])};
     if (Ud[0] < 0 || Ud[0] >= lim24 || Ud[1] < 0 || Ud[1] >= lim24 || Ud[2] < 0 || Ud[2] >= lim24) out++;
     const float v = dither_pick(uniform ? d_uniform : dither_of(sign * wc * fkp_w(a, nb)), p, is_randoms);
     unsigned packed[3];
@@ -509,8 +565,13 @@ __global__ void __launch_bounds__(256) k_ptile_prep(PaintArgs a_in, int is_rando
       for (int dy = 0; dy < span[1]; dy++)
         for (int dz = 0; dz < span[2]; dz++) {
           const int t = ((((tb[0] + dx) % nts) * nts + (tb[1] + dy) % nts) * nts) + (tb[2] + dz) % nts;
-          atomicAdd(&ta.cnt[t], 1u);
+          atomicAdd(&cnt[t], 1u);
         }
+  }
+  if (SHARED) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < ntiles; i += blockDim.x)
+      if (hist[i]) atomicAdd(&ta.cnt[i], hist[i]);
   }
   const unsigned nb_w = __reduce_add_sync(0xffffffffu, bad);
   const unsigned no_w = __reduce_add_sync(0xffffffffu, out);
@@ -579,6 +640,55 @@ __global__ void __launch_bounds__(256) k_ptile_scatter(TileArgs ta, int64_t tota
                                       (r.y & kCoordMask) | (dy ? kNextTile : 0u),
                                       (r.z & kCoordMask) | (dz ? kNextTile : 0u), r.w);
         }
+  }
+}
+
+// The same for meshes of few tiles: each block first counts its records per tile in shared memory,
+// reserves the block's share of every tile's range, front and back, with one atomic add each, and
+// then places its records with shared cursors.
+__global__ void __launch_bounds__(512) k_ptile_scatter_shared(TileArgs ta, int64_t total, const DevCat* dc, const int* cur,
+                                                              int N) {
+  extern __shared__ __align__(16) unsigned at[];  // [2][ntiles]: counts, then the next place
+  if (dc) total = dc[*cur].count;
+  const int nts = N / kPT, ntiles = nts * nts * nts;
+  const int64_t p0 = (int64_t)blockIdx.x * blockDim.x, step = (int64_t)gridDim.x * blockDim.x;
+  if (p0 >= total) return;  // uniform over the block
+  for (int i = threadIdx.x; i < 2 * ntiles; i += blockDim.x) at[i] = 0u;
+  __syncthreads();
+  // f(entry of `at`, copy) for each tile the record touches
+  auto each = [&](unsigned t, unsigned sx, unsigned sy, unsigned sz, auto&& f) {
+    if (!((sx | sy | sz) & kSpan2)) {
+      f((int)t, 0u, 0u, 0u);
+      return;
+    }
+    const int tb[3] = {(int)(t / (nts * nts)), (int)((t / nts) % nts), (int)(t % nts)};
+    const unsigned ex = sx >> 31, ey = sy >> 31, ez = sz >> 31;
+    for (unsigned dx = 0; dx <= ex; dx++)
+      for (unsigned dy = 0; dy <= ey; dy++)
+        for (unsigned dz = 0; dz <= ez; dz++)
+          f(ntiles + ((((tb[0] + (int)dx) % nts) * nts + (tb[1] + (int)dy) % nts) * nts) + (tb[2] + (int)dz) % nts, dx, dy, dz);
+  };
+  for (int64_t p = p0 + threadIdx.x; p < total; p += step) {
+    const unsigned t = ta.tile_of[p];
+    if (t == kNoTile) continue;
+    const uint4 r = ta.rec[p];
+    each(t, r.x, r.y, r.z, [&](int i, unsigned, unsigned, unsigned) { atomicAdd(&at[i], 1u); });
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < ntiles; i += blockDim.x) {
+    const unsigned nf = at[i], nb = at[ntiles + i];
+    if (nf) at[i] = atomicAdd(&ta.cursor[i], nf);
+    if (nb) at[ntiles + i] = atomicSub(&ta.cursor[ntiles + i], nb) - nb;
+  }
+  __syncthreads();
+  for (int64_t p = p0 + threadIdx.x; p < total; p += step) {
+    const unsigned t = ta.tile_of[p];
+    if (t == kNoTile) continue;
+    const uint4 r = ta.rec[p];
+    each(t, r.x, r.y, r.z, [&](int i, unsigned dx, unsigned dy, unsigned dz) {
+      ta.sorted[atomicAdd(&at[i], 1u)] = make_uint4((r.x & kCoordMask) | (dx ? kNextTile : 0u), (r.y & kCoordMask) | (dy ? kNextTile : 0u),
+                                                    (r.z & kCoordMask) | (dz ? kNextTile : 0u), r.w);
+    });
   }
 }
 
@@ -747,21 +857,47 @@ __global__ void __launch_bounds__(kTilePaintThreads, INTER ? 3 : 4) k_ptile_pain
   }
 }
 
-void launch_ptile_prep(const PaintArgs& a, int window, int interlaced, int is_randoms, double* derived,
-                       const TileArgs& ta, int64_t offset, int N, int nblocks, cudaStream_t s) {
-  if (!a.dc && a.count <= 0) return;
-  const int64_t need = a.dc ? nblocks : (a.count + 255) / 256;
-  const int nb = (int)(need < nblocks ? need : nblocks);
+namespace {
+bool shared_tiles(int N) { return (N / kPT) * (N / kPT) * (N / kPT) <= kSharedTiles; }
+// Blocks of 512 threads for `count` particles: with shared counts a few per SM, each with a long run of
+// particles to share them; else enough to fill the SMs several times over.
+int particle_blocks(int64_t count, bool shared, int nsm) {
+  const int64_t need = (count + 511) / 512, cap = (shared ? 4 : 8) * (int64_t)nsm;
+  return (int)(need < 1 ? 1 : (need < cap ? need : cap));
+}
+template <int WIN, bool INTER>
+void ptile_prep_v(const PrepArgs& pa, int ncat, int64_t most, double* derived, const TileArgs& ta, int N, int nsm, cudaStream_t s) {
+  const bool sh = shared_tiles(N);
+  const dim3 grid(particle_blocks(most, sh, nsm), ncat);
+  const size_t smem = sh ? (size_t)(N / kPT) * (N / kPT) * (N / kPT) * sizeof(unsigned) : 0;
+  if (sh)
+    k_ptile_prep<WIN, INTER, true><<<grid, 512, smem, s>>>(pa, derived, ta, N);
+  else
+    k_ptile_prep<WIN, INTER, false><<<grid, 512, 0, s>>>(pa, derived, ta, N);
+}
+}  // namespace
+
+void launch_ptile_prep(const PaintArgs& a, int kind_a, const PaintArgs* b, int kind_b, int window, int interlaced,
+                       double* derived, const TileArgs& ta, int N, int nsm, cudaStream_t s) {
+  PrepArgs pa;
+  pa.a[0] = a;
+  pa.kind[0] = kind_a;
+  pa.a[1] = b ? *b : a;
+  pa.kind[1] = kind_b;
+  // a catalog from a device descriptor (dc): its size is known on the device only
+  const int64_t most = a.dc ? INT64_MAX / 2 : (b && b->count > a.count ? b->count : a.count);
+  if (most <= 0) return;
+  const int ncat = b ? 2 : 1;
   if (window == PSPEC_WINDOW_CIC) {
     if (interlaced)
-      k_ptile_prep<PSPEC_WINDOW_CIC, true><<<nb, 256, 0, s>>>(a, is_randoms, derived, ta, offset, N);
+      ptile_prep_v<PSPEC_WINDOW_CIC, true>(pa, ncat, most, derived, ta, N, nsm, s);
     else
-      k_ptile_prep<PSPEC_WINDOW_CIC, false><<<nb, 256, 0, s>>>(a, is_randoms, derived, ta, offset, N);
+      ptile_prep_v<PSPEC_WINDOW_CIC, false>(pa, ncat, most, derived, ta, N, nsm, s);
   } else {
     if (interlaced)
-      k_ptile_prep<PSPEC_WINDOW_TSC, true><<<nb, 256, 0, s>>>(a, is_randoms, derived, ta, offset, N);
+      ptile_prep_v<PSPEC_WINDOW_TSC, true>(pa, ncat, most, derived, ta, N, nsm, s);
     else
-      k_ptile_prep<PSPEC_WINDOW_TSC, false><<<nb, 256, 0, s>>>(a, is_randoms, derived, ta, offset, N);
+      ptile_prep_v<PSPEC_WINDOW_TSC, false>(pa, ncat, most, derived, ta, N, nsm, s);
   }
 }
 
@@ -769,12 +905,15 @@ void launch_ptile_scan(const TileArgs& ta, int ntiles, cudaStream_t s) {
   k_ptile_scan<<<(ntiles + 1023) / 1024, 1024, 0, s>>>(ta, ntiles);
 }
 
-void launch_ptile_scatter(const TileArgs& ta, int64_t total, const DevCat* dc, const int* cur, int N, int nblocks,
+void launch_ptile_scatter(const TileArgs& ta, int64_t total, const DevCat* dc, const int* cur, int N, int nsm,
                           cudaStream_t s) {
   if (!dc && total <= 0) return;
-  const int64_t need = dc ? nblocks : (total + 255) / 256;
-  const int nb = (int)(need < nblocks ? need : nblocks);
-  k_ptile_scatter<<<nb, 256, 0, s>>>(ta, total, dc, cur, N);
+  const bool sh = shared_tiles(N);
+  const int nb = particle_blocks(dc ? INT64_MAX / 2 : total, sh, nsm);
+  if (sh)
+    k_ptile_scatter_shared<<<nb, 512, 2 * (size_t)(N / kPT) * (N / kPT) * (N / kPT) * sizeof(unsigned), s>>>(ta, total, dc, cur, N);
+  else
+    k_ptile_scatter<<<2 * nb, 256, 0, s>>>(ta, total, dc, cur, N);
 }
 
 template <typename K> static void set_smem_attr(K kernel, size_t bytes) {

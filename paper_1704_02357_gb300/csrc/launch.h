@@ -40,12 +40,29 @@ struct PaintArgs {
   int64_t count;
   double corner[3];
   double inv_cell;      // N / L
+  int safe_log2;        // positions below 2^safe_log2 in magnitude are valid (paint_safe_log2); -1000: test each
   double P0;
   double nbar_default;
   double wf_default;    // FKP weight for nbar_default
   const DevCat* dc;     // when set, pos/weight/nbar/count come from dc[*cur]
   const int* cur;
 };
+
+// The largest k for which |x| < 2^k implies a valid particle (grid coordinate below 2^62 in units of 2^-24
+// cell) on every axis, with a factor two of margin; -1000 when the corner itself is too far out.
+inline int paint_safe_log2(const double* corner, double inv_cell) {
+  double c = 0.0;
+  for (int d = 0; d < 3; d++) {
+    const double a = corner[d] < 0 ? -corner[d] : corner[d];
+    c = a > c ? a : c;
+  }
+  const double reach = 137438953472.0 / inv_cell - c;  // 2^37 cells from the corner
+  int k = -1000;
+  if (reach > 0.0)
+    for (k = -900; k < 900 && __builtin_ldexp(1.0, k + 1) <= reach; k++) {
+    }
+  return k;
+}
 
 struct BinArgs {
   const int32_t* bin_of_n2;  // bin index of |n|^2, or -1
@@ -105,10 +122,12 @@ struct TileArgs {
   unsigned* tile_of; // [particles] first tile of each record (all ones: left out)
   uint4* sorted;     // [kPaintRecordsMax * particles] records in tile order
 };
-void launch_ptile_prep(const PaintArgs& a, int window, int interlaced, int is_randoms, double* derived,
-                       const TileArgs& ta, int64_t offset, int N, int nblocks, cudaStream_t s);
+// Prep of one catalog, or of a second one in the same launch (b nullable): a's records first, then
+// b's. kind_a, kind_b as is_randoms above.
+void launch_ptile_prep(const PaintArgs& a, int kind_a, const PaintArgs* b, int kind_b, int window, int interlaced,
+                       double* derived, const TileArgs& ta, int N, int nsm, cudaStream_t s);
 void launch_ptile_scan(const TileArgs& ta, int ntiles, cudaStream_t s);
-void launch_ptile_scatter(const TileArgs& ta, int64_t total, const DevCat* dc, const int* cur, int N, int nblocks,
+void launch_ptile_scatter(const TileArgs& ta, int64_t total, const DevCat* dc, const int* cur, int N, int nsm,
                           cudaStream_t s);
 // r1, r2 (nullable, batched mocks): cached randoms meshes; mesh = painted - *alpha * randoms.
 void launch_ptile_paint(const TileArgs& ta, int window, int interlaced, float* m1, float* m2, int N,

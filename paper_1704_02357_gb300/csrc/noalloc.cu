@@ -58,6 +58,7 @@ PaintArgs args_for(const pspec_params* p, const pspec_catalog* c) {
   a.count = c->count;
   for (int d = 0; d < 3; d++) a.corner[d] = p->box_corner[d];
   a.inv_cell = (double)p->nmesh / p->box_size;
+  a.safe_log2 = paint_safe_log2(a.corner, a.inv_cell);
   a.P0 = p->P0;
   a.nbar_default = p->nbar;
   a.wf_default = p->P0 > 0 ? 1.0 / (1.0 + p->nbar * p->P0) : 1.0;

@@ -525,6 +525,7 @@ PaintArgs paint_args(Ctx* c, const pspec_catalog* cat) {
   a.count = cat->count;
   for (int d = 0; d < 3; d++) a.corner[d] = c->p.box_corner[d];
   a.inv_cell = (double)c->p.nmesh / c->p.box_size;
+  a.safe_log2 = paint_safe_log2(a.corner, a.inv_cell);
   a.P0 = c->p.P0;
   a.nbar_default = c->p.nbar;
   a.wf_default = fkp(c->p.nbar, c->p.P0);
@@ -588,14 +589,11 @@ pspec_status do_paint(Ctx* c, const pspec_catalog* d, const pspec_catalog* r) {
     if (e != cudaSuccess) return cuda_fail(c, e, "tile counts clear");
     float* f1 = reinterpret_cast<float*>(m1);
     float* f2 = reinterpret_cast<float*>(m2);
-    TRY(run(c, PSPEC_K_PAINT, cat_bytes(d), [&] {
-      launch_ptile_prep(ad, c->p.window, c->p.interlaced, 0, der, ta, 0, N, nb, c->stream);
-    }));
-    TRY(run(c, PSPEC_K_PAINT, cat_bytes(r), [&] {
-      launch_ptile_prep(ar, c->p.window, c->p.interlaced, 1, der, ta, d->count, N, nb, c->stream);
+    TRY(run(c, PSPEC_K_PAINT, cat_bytes(d) + cat_bytes(r), [&] {
+      launch_ptile_prep(ad, 0, &ar, 1, c->p.window, c->p.interlaced, der, ta, N, c->nsm, c->stream);
     }));
     TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scan(ta, pl.ntiles, c->stream); }));
-    TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scatter(ta, total, nullptr, nullptr, N, nb, c->stream); }));
+    TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scatter(ta, total, nullptr, nullptr, N, c->nsm, c->stream); }));
     TRY(run(c, PSPEC_K_PAINT, nmesh * pl.Sr, [&] {
       launch_ptile_paint(ta, c->p.window, c->p.interlaced, f1, f2, N, der + D_FIX, nullptr, nullptr, nullptr, c->stream);
     }));
@@ -810,10 +808,10 @@ pspec_status paint_one(Ctx* c, const PaintArgs& a, int is_randoms, bool binned, 
     e = cudaMemsetAsync(ta.cnt, 0, (size_t)(pl.ntiles + 1) * sizeof(unsigned), c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "tile counts clear");
     TRY(run(c, PSPEC_K_PAINT, pbytes, [&] {
-      launch_ptile_prep(a, c->p.window, c->p.interlaced, is_randoms, der, ta, 0, N, nb, c->stream);
+      launch_ptile_prep(a, is_randoms, nullptr, 0, c->p.window, c->p.interlaced, der, ta, N, c->nsm, c->stream);
     }));
     TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scan(ta, pl.ntiles, c->stream); }));
-    TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scatter(ta, a.count, a.dc, a.cur, N, nb, c->stream); }));
+    TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scatter(ta, a.count, a.dc, a.cur, N, c->nsm, c->stream); }));
     TRY(run(c, PSPEC_K_PAINT, (r1 ? 2.0 : 1.0) * nmesh * pl.Sr, [&] {
       launch_ptile_paint(ta, c->p.window, c->p.interlaced, reinterpret_cast<float*>(m1), reinterpret_cast<float*>(m2),
                          N, fix, reinterpret_cast<const float*>(r1), reinterpret_cast<const float*>(r2), der + D_ALPHA,

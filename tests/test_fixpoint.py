@@ -1,4 +1,5 @@
-"""The fixed-point arithmetic of the FP64 transforms (csrc/fixpoint.cuh), compiled for the host.
+"""The fixed-point arithmetic of the FP64 transforms (csrc/fixpoint.cuh) and the integer forms the
+paint uses (csrc/intconv.cuh), compiled for the host.
 
 Conversions are compared with exact integer arithmetic; products by a unit factor with exact integers
 (per real factor the term below one unit that they leave out, and one rounding: at most 1.5 units, 2.5
@@ -25,6 +26,8 @@ int main() {
   while (std::scanf(" %c", &op) == 1) {
     if (op == 'i') { double v; int c; std::scanf("%la %d", &v, &c); std::printf("%lld\n", fx_from_double(v, c)); }
     if (op == 'o') { long long q; int c; std::scanf("%lld %d", &q, &c); std::printf("%a\n", fx_to_double(q, c)); }
+    if (op == 'f') { double v; std::scanf("%la", &v); FloatPair p = float_pair(v); std::printf("%a %a %u %d\n", p.lo, p.hi, p.thr, (int)float_pair_ok(v)); }
+    if (op == 'd') { double v; int k; std::scanf("%la %d", &v, &k); std::printf("%lld\n", d2ll_rn_scaled(v, k)); }
     if (op == 'h') { long long q; std::scanf("%lld", &q); std::printf("%lld\n", fx_half(q)); }
     if (op == 'm') {
       lc a; int c, d, e, f; std::scanf("%lld %lld %d %d %d %d", &a.x, &a.y, &c, &d, &e, &f);
@@ -114,3 +117,27 @@ def test_scale_keeps_the_sum_below_2_62(ask, exponent):
             assert total > 2 ** 62 / Fraction(9, 4)  # the largest scale, up to the sum's own slack
     for v in ("inf", "nan"):
         assert ask([f"s 2 1 0 {v} 0x1p+0"])[0][1] == "1"
+
+
+def test_scaled_rounding_and_float_pairs(ask):
+    rng = random.Random(4)
+    vals = [(0.0, 24), (-0.0, 24), (5e-324, 24), (0.5 * 2.0 ** -24, 24), (1.5 * 2.0 ** -24, 24), (2.0 ** 37, 24)]
+    vals += [(math.ldexp(rng.uniform(-1, 1), rng.randint(-40, 38)), 24) for _ in range(20000)]
+    for (v, k), r in zip(vals, ask([f"d {v.hex()} {k}" for v, k in vals])):
+        assert int(r[0]) == round(Fraction(v) * 2 ** k), (v, r)  # ties to even
+    import struct
+    f32 = lambda x: struct.unpack("f", struct.pack("f", x))[0]
+    nxt = lambda x, up: struct.unpack("f", struct.pack("I", struct.unpack("I", struct.pack("f", x))[0] + (1 if up else -1)))[0]
+    vs = [0.25, -0.25, 1.0 - 2.0 ** -30, -(1.0 - 2.0 ** -30), 1.0 + 2.0 ** -25, 1.0 + 2.0 ** -24, 1.0 + 3 * 2.0 ** -24,
+          1.0 - 2.0 ** -25, -0.05]
+    vs += [rng.uniform(-1, 1) * 2.0 ** rng.randint(-100, 100) for _ in range(20000)]
+    for v, r in zip(vs, ask([f"f {v.hex()}" for v in vs])):
+        lo, hi, thr, ok = float.fromhex(r[0]), float.fromhex(r[1]), int(r[2]), r[3] == "1"
+        assert ok and lo == f32(v), (v, r)
+        if lo == v:
+            assert hi == lo and thr == 0
+            continue
+        assert hi == nxt(lo, abs(v) > abs(lo)) and min(lo, hi) < v < max(lo, hi), (v, r)
+        assert thr == Fraction(abs(v - lo)) / Fraction(abs(hi - lo)) * 2 ** 32, (v, r)
+    for v in (0.0, 1e-39, 3e38, float("inf"), float("nan")):
+        assert ask([f"f {v.hex()}"])[0][3] == "0", v
