@@ -25,11 +25,41 @@
 
 namespace pspec {
 
-struct xf {
-  float h, l;
-};
+// Packed FP32 pairs: one instruction adds, multiplies or multiply-adds both halves, each rounded as
+// the scalar instruction rounds it. The FMA pipe takes a pair no faster than two scalars (measured: 53
+// packed against 117 scalar results per clock and SM), but it takes one issue slot instead of two, and
+// these stages were bound by issue (85% of the slots in the z pass with the pipe 67% busy). Values
+// are complex numbers, so the pairs are (re, im): additions, splits and products by real constants are
+// packed; rotations by i and twiddle products, which mix the halves, stay scalar.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{.reg .b64 a, b, c; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; add.rn.f32x2 c, a, b; mov.b64 {%0, %1}, c;}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  float2 r;
+  asm("{.reg .b64 a, b, c; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; sub.rn.f32x2 c, a, b; mov.b64 {%0, %1}, c;}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float k) {
+  float2 r;
+  asm("{.reg .b64 a, b, c; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %4}; mul.rn.f32x2 c, a, b; mov.b64 {%0, %1}, c;}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(k));
+  return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float k, float2 d) {
+  float2 r;
+  asm("{.reg .b64 a, b, c, d; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %4}; mov.b64 d, {%5, %6}; fma.rn.f32x2 c, a, b, d; "
+      "mov.b64 {%0, %1}, c;}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(k), "f"(d.x), "f"(d.y));
+  return r;
+}
+
+// A complex value h + l; h = (re, im) on the quantum q.
 struct xc {
-  xf x, y;
+  float2 h, l;
 };
 
 __device__ __forceinline__ float xadd_(float a, float b) { return __fadd_rn(a, b); }
@@ -42,31 +72,30 @@ __device__ __forceinline__ float xmagic(float bound) {
   eb = eb > 240 ? 240 : eb;
   return __int_as_float(((eb + 13) << 23) | 0x400000);  // q = 2^(eb - 137), M = 1.5 * 2^(eb - 114)
 }
-__device__ __forceinline__ float xgrid(float p, float M) { return xsub_(xadd_(p, M), M); }
-
-__device__ __forceinline__ xf xsplit(float v, float M) {
-  const float g = xgrid(v, M);
-  return {g, xsub_(v, g)};
+__device__ __forceinline__ float2 xgrid(float2 p, float M) {
+  const float2 m = make_float2(M, M);
+  return sub2(add2(p, m), m);
 }
-__device__ __forceinline__ xc xsplit(float2 v, float M) { return {xsplit(v.x, M), xsplit(v.y, M)}; }
+__device__ __forceinline__ xc xsplit(float2 v, float M) {
+  const float2 g = xgrid(v, M);
+  return {g, sub2(v, g)};
+}
 // back onto the quantum q before another multiplication
-__device__ __forceinline__ xf xresplit(xf a, float M) {
-  const float g = xgrid(a.h, M);
-  return {g, xadd_(a.l, xsub_(a.h, g))};
+__device__ __forceinline__ xc xresplit(xc a, float M) {
+  const float2 g = xgrid(a.h, M);
+  return {g, add2(a.l, sub2(a.h, g))};
 }
-__device__ __forceinline__ xc xresplit(xc a, float M) { return {xresplit(a.x, M), xresplit(a.y, M)}; }
-__device__ __forceinline__ float xround(xf a) { return xadd_(a.h, a.l); }
-__device__ __forceinline__ float2 xround(xc a) { return make_float2(xround(a.x), xround(a.y)); }
+__device__ __forceinline__ float2 xround(xc a) { return add2(a.h, a.l); }
 
-__device__ __forceinline__ xf operator+(xf a, xf b) { return {xadd_(a.h, b.h), xadd_(a.l, b.l)}; }
-__device__ __forceinline__ xf operator-(xf a, xf b) { return {xsub_(a.h, b.h), xsub_(a.l, b.l)}; }
-__device__ __forceinline__ xf operator-(xf a) { return {-a.h, -a.l}; }
-__device__ __forceinline__ xc operator+(xc a, xc b) { return {a.x + b.x, a.y + b.y}; }
-__device__ __forceinline__ xc operator-(xc a, xc b) { return {a.x - b.x, a.y - b.y}; }
-// a * (i * sgn)
-__device__ __forceinline__ xc xmul_i(xc a, int sgn) { return sgn > 0 ? xc{-a.y, a.x} : xc{a.y, -a.x}; }
-__device__ __forceinline__ xc xconj(xc a) { return {a.x, -a.y}; }
-__device__ __forceinline__ xf xhalf(xf a) { return {0.5f * a.h, 0.5f * a.l}; }  // exact
+__device__ __forceinline__ xc operator+(xc a, xc b) { return {add2(a.h, b.h), add2(a.l, b.l)}; }
+__device__ __forceinline__ xc operator-(xc a, xc b) { return {sub2(a.h, b.h), sub2(a.l, b.l)}; }
+// a + i sgn b
+__device__ __forceinline__ float2 xadd_i(float2 a, float2 b, int sgn) {
+  return sgn > 0 ? make_float2(xsub_(a.x, b.y), xadd_(a.y, b.x)) : make_float2(xadd_(a.x, b.y), xsub_(a.y, b.x));
+}
+__device__ __forceinline__ xc xadd_i(xc a, xc b, int sgn) { return {xadd_i(a.h, b.h, sgn), xadd_i(a.l, b.l, sgn)}; }
+__device__ __forceinline__ float2 xconj(float2 a) { return make_float2(a.x, -a.y); }
+__device__ __forceinline__ xc xconj(xc a) { return {xconj(a.h), xconj(a.l)}; }
 
 // A constant |K| <= 1 as K12 (a multiple of 2^-12) + Kr, with kf = K rounded to FP32.
 struct K12 {
@@ -77,9 +106,7 @@ struct K12 {
         kf((float)k) {}
 };
 // a * K; a.h on the quantum q (at most 12 significant bits): a.h * K12 is exact.
-__device__ __forceinline__ xf xcm(xf a, const K12& k) {
-  return {xmul_(a.h, k.k12), fmaf(a.l, k.kf, a.h * k.kr)};
-}
+__device__ __forceinline__ xc xcm(xc a, const K12& k) { return {mul2(a.h, k.k12), fma2(a.l, k.kf, mul2(a.h, k.kr))}; }
 
 // a * w for a twiddle in the 12-bit form {c12, s12, cr, sr} (tables built on the host); a on the
 // quantum q. The h parts are exact: each product has at most 23 significant bits and the FMA's
@@ -87,15 +114,13 @@ __device__ __forceinline__ xf xcm(xf a, const K12& k) {
 __device__ __forceinline__ xc xtw(xc a, float4 w) {
   const float cf = xadd_(w.x, w.z), sf = xadd_(w.y, w.w);
   xc r;
-  r.x.h = fmaf(a.x.h, w.x, -xmul_(a.y.h, w.y));
-  r.y.h = fmaf(a.x.h, w.y, xmul_(a.y.h, w.x));
-  r.x.l = fmaf(a.x.l, cf, fmaf(-a.y.l, sf, fmaf(a.x.h, w.z, -(a.y.h * w.w))));
-  r.y.l = fmaf(a.x.l, sf, fmaf(a.y.l, cf, fmaf(a.x.h, w.w, a.y.h * w.z)));
+  r.h.x = fmaf(a.h.x, w.x, -xmul_(a.h.y, w.y));
+  r.h.y = fmaf(a.h.x, w.y, xmul_(a.h.y, w.x));
+  r.l.x = fmaf(a.l.x, cf, fmaf(-a.l.y, sf, fmaf(a.h.x, w.z, -xmul_(a.h.y, w.w))));
+  r.l.y = fmaf(a.l.x, sf, fmaf(a.l.y, cf, fmaf(a.h.x, w.w, xmul_(a.h.y, w.z))));
   return r;
 }
 __device__ __forceinline__ xc xtw(float2 a, float4 w, float M) { return xtw(xsplit(a, M), w); }
-// conjugate twiddle (inverse transforms)
-__device__ __forceinline__ float4 xconj_w(float4 w) { return make_float4(w.x, -w.y, w.z, -w.w); }
 
 // ------------------------------------------------------------------ butterflies
 // The radix-R DFTs of common.cuh (same decompositions and constants) on exact-add values. The
@@ -115,29 +140,32 @@ template <> struct XDft<4> {
   static __device__ __forceinline__ void run(xc* v, int dir, float) {
     const xc t0 = v[0] + v[2], t1 = v[0] - v[2];
     const xc t2 = v[1] + v[3], t3 = v[1] - v[3];
-    const xc it3 = xmul_i(t3, dir);
     v[0] = t0 + t2;
     v[2] = t0 - t2;
-    v[1] = t1 + it3;
-    v[3] = t1 - it3;
+    v[1] = xadd_i(t1, t3, dir);
+    v[3] = xadd_i(t1, t3, -dir);
   }
 };
 
 // z * (sr cr + i si ci) with sr, si = +-1
 __device__ __forceinline__ xc xrot(xc z, const K12& cr, const K12& ci, int sr, int si, float M) {
   z = xresplit(z, M);
-  const xf ax = xcm(z.x, cr), ay = xcm(z.y, ci);  // cr z.x, ci z.y
-  const xf bx = xcm(z.y, cr), by = xcm(z.x, ci);  // cr z.y, ci z.x
-  const xf p = sr > 0 ? ax : -ax, q = si > 0 ? ay : -ay;
-  const xf s = sr > 0 ? bx : -bx, u = si > 0 ? by : -by;
-  return {p - q, s + u};
+  const xc a = xcm(z, cr), b = xcm(z, ci);  // cr z, ci z
+  // sr a + i si b
+  auto mix = [&](float2 p, float2 q) {
+    const float2 u = sr > 0 ? p : make_float2(-p.x, -p.y);
+    return si > 0 ? make_float2(xsub_(u.x, q.y), xadd_(u.y, q.x)) : make_float2(xadd_(u.x, q.y), xsub_(u.y, q.x));
+  };
+  return {mix(a.h, b.h), mix(a.l, b.l)};
 }
 // z * (sgn + dir i) / sqrt2 (sgn = +-1)
 __device__ __forceinline__ xc xdiag(xc z, int sgn, int dir, const K12& h, float M) {
-  const xf zx = sgn > 0 ? z.x : -z.x, zy = sgn > 0 ? z.y : -z.y;
-  const xf re = dir > 0 ? zx - z.y : zx + z.y;  // sgn z.x - dir z.y
-  const xf im = dir > 0 ? zy + z.x : zy - z.x;  // sgn z.y + dir z.x
-  return {xcm(xresplit(re, M), h), xcm(xresplit(im, M), h)};
+  auto mix = [&](float2 p) {  // sgn p + i dir p
+    const float2 u = sgn > 0 ? p : make_float2(-p.x, -p.y);
+    return dir > 0 ? make_float2(xsub_(u.x, p.y), xadd_(u.y, p.x)) : make_float2(xadd_(u.x, p.y), xsub_(u.y, p.x));
+  };
+  const xc r = {mix(z.h), mix(z.l)};
+  return xcm(xresplit(r, M), h);
 }
 
 template <> struct XDft<8> {
@@ -148,14 +176,13 @@ template <> struct XDft<8> {
     XDft<4>::run(e, dir, M);
     XDft<4>::run(o, dir, M);
     const xc o1 = xdiag(o[1], 1, dir, h, M);
-    const xc o2 = xmul_i(o[2], dir);
     const xc o3 = xdiag(o[3], -1, dir, h, M);
     v[0] = e[0] + o[0];
     v[4] = e[0] - o[0];
     v[1] = e[1] + o1;
     v[5] = e[1] - o1;
-    v[2] = e[2] + o2;
-    v[6] = e[2] - o2;
+    v[2] = xadd_i(e[2], o[2], dir);
+    v[6] = xadd_i(e[2], o[2], -dir);
     v[3] = e[3] + o3;
     v[7] = e[3] - o3;
   }
@@ -177,7 +204,6 @@ template <> struct XDft<16> {
     a[1][2] = xdiag(a[1][2], 1, d, h, M);        // m = 2
     a[1][3] = xrot(a[1][3], s1, c1, 1, d, M);    // m = 3
     a[2][1] = xdiag(a[2][1], 1, d, h, M);        // m = 2
-    a[2][2] = xmul_i(a[2][2], d);                // m = 4
     a[2][3] = xdiag(a[2][3], -1, d, h, M);       // m = 6
     a[3][1] = xrot(a[3][1], s1, c1, 1, d, M);    // m = 3
     a[3][2] = xdiag(a[3][2], -1, d, h, M);       // m = 6
@@ -185,7 +211,16 @@ template <> struct XDft<16> {
 #pragma unroll
     for (int k1 = 0; k1 < 4; k1++) {
       xc t[4] = {a[0][k1], a[1][k1], a[2][k1], a[3][k1]};
-      XDft<4>::run(t, dir, M);
+      if (k1 == 2) {  // m = 4: a[2][2] times i d
+        const xc t0 = xadd_i(t[0], t[2], d), t1 = xadd_i(t[0], t[2], -d);
+        const xc t2 = t[1] + t[3], t3 = t[1] - t[3];
+        t[0] = t0 + t2;
+        t[2] = t0 - t2;
+        t[1] = xadd_i(t1, t3, d);
+        t[3] = xadd_i(t1, t3, -d);
+      } else {
+        XDft<4>::run(t, dir, M);
+      }
 #pragma unroll
       for (int k2 = 0; k2 < 4; k2++) v[k1 + 4 * k2] = t[k2];
     }
@@ -197,12 +232,11 @@ template <> struct XDft<3> {
     const K12 s3(0.86602540378443864676);
     const xc t = v[1] + v[2];
     const xc u = xresplit(v[1] - v[2], M);
-    const xc m = v[0] - xc{xhalf(t.x), xhalf(t.y)};
-    const xf sx = xcm(u.x, s3), sy = xcm(u.y, s3);
-    const xc isu = dir > 0 ? xc{-sy, sx} : xc{sy, -sx};  // i dir sin(2 pi/3) u
+    const xc m = v[0] - xc{mul2(t.h, 0.5f), mul2(t.l, 0.5f)};
+    const xc su = xcm(u, s3);  // sin(2 pi/3) u
     v[0] = v[0] + t;
-    v[1] = m + isu;
-    v[2] = m - isu;
+    v[1] = xadd_i(m, su, dir);
+    v[2] = xadd_i(m, su, -dir);
   }
 };
 
@@ -298,11 +332,10 @@ __device__ __forceinline__ void fft_any(C (&v)[E], C* sm, int t, int seq, const 
 __device__ __forceinline__ float2 r2c_unpack_xp(float2 zk, float2 zm, float4 w) {
   const float bound = fabsf(zk.x) + fabsf(zk.y) + fabsf(zm.x) + fabsf(zm.y);
   const float M = xmagic(4.f * bound);
-  const xc a = xsplit(zk, M), b = xconj(xsplit(zm, M));
+  const xc a = xsplit(zk, M), b = xsplit(xconj(zm), M);
   const xc s = a + b, d = a - b;
-  const xc o = xtw(xc{d.y, -d.x}, w);  // -i d w
-  const float2 r = xround(s + o);
-  return make_float2(0.5f * r.x, 0.5f * r.y);
+  const xc o = xtw(xc{make_float2(d.h.y, -d.h.x), make_float2(d.l.y, -d.l.x)}, w);  // -i d w
+  return mul2(xround(s + o), 0.5f);
 }
 
 // c2r pack (k_c2r_z) in exact-add arithmetic: with A = X[k] and B = conj(X[L-k]) (0 for k = 0),
@@ -310,10 +343,9 @@ __device__ __forceinline__ float2 r2c_unpack_xp(float2 zk, float2 zm, float4 w) 
 __device__ __forceinline__ float2 c2r_pack_xp(float2 xk, float2 xm, float4 wc) {
   const float bound = fabsf(xk.x) + fabsf(xk.y) + fabsf(xm.x) + fabsf(xm.y);
   const float M = xmagic(4.f * bound);
-  const xc a = xsplit(xk, M), b = xconj(xsplit(xm, M));
+  const xc a = xsplit(xk, M), b = xsplit(xconj(xm), M);
   const xc ev = a + b, od = xtw(a - b, wc);
-  const float2 r = xround(xc{ev.x - od.y, ev.y + od.x});  // 2E + i 2O'
-  return make_float2(0.5f * r.x, 0.5f * r.y);
+  return mul2(xround(xadd_i(ev, od, 1)), 0.5f);  // (2E + i 2O') / 2
 }
 
 }  // namespace pspec
