@@ -80,6 +80,23 @@ __host__ __device__ constexpr CtPlan ct_plan(int L, int E = 8) {
   return p;
 }
 
+// Twiddle tables: the entries of each stage after the first lie together, [r - 1][k] for r < R and k < Ns
+// (w_L^{r k L/(Ns R)}), so that a warp's loads of one r are contiguous. From one table of w_L^t they
+// were r k L/(Ns R) entries apart and spread over up to 12 lines a load; the z pass was bound by
+// its L1 wavefronts. A buffer holds the tables of every plan of a length one after another: E = 8
+// (or 24 for lengths with a factor 3), then 16 and 32.
+constexpr int tw_stage_off(int L, int E, int stage) {
+  const CtPlan p = ct_plan(L, E);
+  int o = 0;
+  for (int s = 1; s < stage; s++) o += (p.rad[s] - 1) * p.ns[s];
+  return o;
+}
+constexpr int tw_len(int L, int E) { return tw_stage_off(L, E, ct_plan(L, E).nst); }
+constexpr int tw_base(int L, int E) {
+  return E == 32 ? tw_len(L, 8) + tw_len(L, 16) : (E == 16 ? tw_len(L, 8) : 0);
+}
+constexpr int tw_total(int L) { return L % 3 == 0 ? tw_len(L, 24) : tw_base(L, 32) + tw_len(L, 32); }
+
 template <int B, int E, typename F> __device__ __forceinline__ void static_for(F&& f) {
   if constexpr (B < E) {
     f(std::integral_constant<int, B>{});
@@ -87,29 +104,50 @@ template <int B, int E, typename F> __device__ __forceinline__ void static_for(F
   }
 }
 
-// Shared-memory layouts of the exchange buffer.
-//   kInterleaved: [pos][NSEQ], sequence fastest (columns of a tile; lanes run across seqs)
-//   kPaddedRows:  [seq][L + L/16], position fastest with one pad slot per 16 (rows)
+// Shared-memory layouts of the exchange buffer (elements of 8 or 16 bytes).
+//   kInterleaved: [pos][NSEQ], sequence fastest (columns of a tile; lanes run across seqs). A position's
+//     elements fill 1/CPR of the 32 banks; its log2(CPR) low bits take in (^) the bits that threads'
+//     stores in a radix 8, 16 or 32 stage step by, so that stores of a first stage (R positions apart)
+//     use all banks as loads of consecutive positions do.
+//   kPaddedRows:  [seq][padded_len], position fastest with one pad slot per 16 (8 for 16-byte elements);
+//     rows of fewer than 16 threads are spaced so that the rows of a half warp use different banks.
 enum { kInterleaved = 0, kPaddedRows = 1 };
 
-__host__ __device__ constexpr int padded_len(int L) { return L + (L >> 4); }
+__host__ __device__ constexpr int padded_len(int L, int Tc, int bytes) {
+  if (bytes == 16) return L + (L >> 3);
+  int s = L + (L >> 4);
+  if (Tc < 16)
+    while (s % 16 != Tc) s++;
+  return s;
+}
 
-template <int LAYOUT, int L, int NSEQ>
-__device__ __forceinline__ int sidx(int seq, int pos) {
-  if constexpr (LAYOUT == kInterleaved)
-    return pos * NSEQ + seq;
-  else
-    return seq * padded_len(L) + pos + (pos >> 4);
+// Slot of position a + b of a sequence; b is a multiple of a power of two above every bit of a (or,
+// in a first stage, below them), known at compile time after unrolling, so that the slots of a
+// thread are one of CPR bases plus a constant.
+template <int LAYOUT, int L, int NSEQ, int BYTES, int Tc>
+__device__ __forceinline__ int sidx(int seq, int a, int b) {
+  if constexpr (LAYOUT == kInterleaved) {
+    constexpr int CPR = 128 / (NSEQ * BYTES);
+    if constexpr (CPR > 1 && CPR <= 4) {
+      auto f = [](int p) { return ((p >> 3) ^ (p >> 4) ^ (p >> 5)) & (CPR - 1); };
+      const int low = b & (CPR - 1);
+      return ((a ^ f(a) ^ (low ^ f(b))) + (b - low)) * NSEQ + seq;
+    }
+    return (a + b) * NSEQ + seq;
+  } else {
+    constexpr int SH = BYTES == 16 ? 3 : 4;
+    return seq * padded_len(L, Tc, BYTES) + a + b + ((a + b) >> SH);
+  }
 }
 
 template <typename C> __device__ __forceinline__ C ldg_c(const C* p) { return __ldg(p); }
 
-template <typename C, int E, int L, int R, int NS, bool LAST, int LAYOUT, int NSEQ, int DIR>
+template <typename C, int E, int L, int R, int NS, int OFF, bool LAST, int LAYOUT, int NSEQ, int DIR>
 __device__ __forceinline__ void stage_ct(C (&v)[E], C* sm, int t, int seq, const ux_of<C>* __restrict__ tw) {
   using U = ux_of<C>;
   constexpr int Q = E / R;
   constexpr int Tc = L / E;
-  constexpr int TSTEP = L / (NS * R);
+  tw += OFF - NS;  // entry r of k at r NS + k
   // With NS | Tc every butterfly of this thread has k = t mod NS: load its twiddles once.
   constexpr bool kShared = (Q > 1) && (NS > 1) && !LAST && (NS <= Tc);
   U ws[kShared ? R : 1];
@@ -117,7 +155,7 @@ __device__ __forceinline__ void stage_ct(C (&v)[E], C* sm, int t, int seq, const
     const int k = t & (NS - 1);
 #pragma unroll
     for (int r = 1; r < R; r++) {
-      ws[r] = ldg_u(tw + r * k * TSTEP);
+      ws[r] = ldg_u(tw + r * NS + k);
       if (DIR > 0) ws[r] = uconj(ws[r]);
     }
   }
@@ -135,7 +173,7 @@ __device__ __forceinline__ void stage_ct(C (&v)[E], C* sm, int t, int seq, const
         if constexpr (kShared) {
           w = ws[r];
         } else {
-          w = ldg_u(tw + r * k * TSTEP);
+          w = ldg_u(tw + r * NS + k);
           if (DIR > 0) w = uconj(w);
         }
         u[r] = umul(u[r], w);
@@ -148,7 +186,7 @@ __device__ __forceinline__ void stage_ct(C (&v)[E], C* sm, int t, int seq, const
     } else {
       const int base = (j - k) * R + k;
 #pragma unroll
-      for (int r = 0; r < R; r++) sm[sidx<LAYOUT, L, NSEQ>(seq, base + r * NS)] = u[r];
+      for (int r = 0; r < R; r++) sm[sidx<LAYOUT, L, NSEQ, sizeof(C), Tc>(seq, base, r * NS)] = u[r];
     }
   }
 }
@@ -174,11 +212,11 @@ __device__ __forceinline__ void fft_ct(C (&v)[E], C* sm, int t, int seq, const u
   static_for<0, P.nst>([&](auto s_) {
     constexpr int s = decltype(s_)::value;
     constexpr bool last = (s == P.nst - 1);
-    stage_ct<C, E, L, P.rad[s], P.ns[s], last, LAYOUT, NSEQ, DIR>(v, sm, t, seq, tw);
+    stage_ct<C, E, L, P.rad[s], P.ns[s], tw_base(L, E) + tw_stage_off(L, E, s), last, LAYOUT, NSEQ, DIR>(v, sm, t, seq, tw);
     if constexpr (!last) {
       fft_sync<WARP>();
 #pragma unroll
-      for (int e = 0; e < E; e++) v[e] = sm[sidx<LAYOUT, L, NSEQ>(seq, t + Tc * e)];
+      for (int e = 0; e < E; e++) v[e] = sm[sidx<LAYOUT, L, NSEQ, sizeof(C), Tc>(seq, t, Tc * e)];
       fft_sync<WARP>();
     }
   });

@@ -161,12 +161,12 @@ __device__ __forceinline__ void fx_row_r2c(double2 (&v)[E], double2* smd, int t,
   for (int e = 0; e < E; e++) u[e] = fx_in(v[e], 1084 - sc.S);
   fft_ct<lc, E, L, kPaddedRows, 1, -1, WARP>(u, sm, t, seq, reinterpret_cast<const int4*>(twh));
 #pragma unroll
-  for (int e = 0; e < E; e++) sm[sidx<kPaddedRows, L, 1>(seq, t + Tc * e)] = u[e];
+  for (int e = 0; e < E; e++) sm[sidx<kPaddedRows, L, 1, 16, Tc>(seq, t, Tc * e)] = u[e];
   fft_sync<WARP>();
 #pragma unroll
   for (int e = 0; e < E; e++) {
     const int k = t + Tc * e;
-    const lc m = sm[sidx<kPaddedRows, L, 1>(seq, k ? L - k : 0)];
+    const lc m = sm[sidx<kPaddedRows, L, 1, 16, Tc>(seq, k ? L - k : 0, 0)];
     const lc s = lc{u[e].x + m.x, u[e].y - m.y}, d = lc{u[e].x - m.x, u[e].y + m.y};
     const lc o = umul(lc{d.y, -d.x}, ldg_u(reinterpret_cast<const int4*>(twr) + k));
     v[e] = fx_out(cadd(s, o), 1085 - sc.S - 1, sc.bad);

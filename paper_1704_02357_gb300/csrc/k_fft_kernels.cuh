@@ -15,6 +15,7 @@
 //      combine (F0 and the l = 0 sums) or with the Y_lm(khat) accumulate-and-bin.
 // Every pass keeps its elements in registers (fft_engine.cuh).
 #pragma once
+#include <algorithm>
 #include <cmath>
 #include "launch.h"
 #include "fft_engine.cuh"
@@ -162,12 +163,12 @@ __global__ void __launch_bounds__(ZRow<T, N, false>::ZT, min_blocks<T, ZRow<T, N
       row_mirrors<C, E, Tc>(v, zm, t);
     } else {
 #pragma unroll
-      for (int e = 0; e < E; e++) sm[sidx<kPaddedRows, L, 1>(r, t + Tc * e)] = v[e];
+      for (int e = 0; e < E; e++) sm[sidx<kPaddedRows, L, 1, sizeof(C), Tc>(r, t, Tc * e)] = v[e];
       __syncthreads();
 #pragma unroll
       for (int e = 0; e < E; e++) {
         const int k = t + Tc * e;
-        zm[e] = sm[sidx<kPaddedRows, L, 1>(r, k ? L - k : 0)];
+        zm[e] = sm[sidx<kPaddedRows, L, 1, sizeof(C), Tc>(r, k ? L - k : 0, 0)];
       }
     }
 #pragma unroll
@@ -231,9 +232,12 @@ __global__ void __launch_bounds__(ZRow<T, N, XP>::ZT, min_blocks<T, ZRow<T, N, X
 // into the M spectra. With the Y_lm(rhat) table and sequences within one warp, each thread loads
 // its own slots of f and of the table and multiplies them in registers: no staging, and no block
 // barrier.
-template <typename T, int N> __host__ __device__ constexpr size_t ylm_stage_bytes(int M, int rows) {
-  return (size_t)M * rows * (N * sizeof(T) > padded_len(N / 2) * sizeof(cx<T>) ? N * sizeof(T)
-                                                                              : padded_len(N / 2) * sizeof(cx<T>));
+// Bytes of a row's exchange buffer in the z passes.
+template <typename T, int N, bool XP> __host__ __device__ constexpr size_t row_bytes() {
+  return padded_len(N / 2, ZRow<T, N, XP>::Tz, sizeof(cx<T>)) * sizeof(cx<T>);
+}
+template <typename T, int N, bool XP> __host__ __device__ constexpr size_t ylm_stage_bytes(int M, int rows) {
+  return (size_t)M * rows * (N * sizeof(T) > row_bytes<T, N, XP>() ? N * sizeof(T) : row_bytes<T, N, XP>());
 }
 
 // f Y_lm(rhat) of `rows` rows and M harmonics into the staging area (FP64 contexts): per row the
@@ -357,7 +361,7 @@ __global__ void __launch_bounds__(ylm_thread_cap(LT), sizeof(T) == 4 ? ylm_min_b
   }
   if constexpr (sizeof(T) == 8 && LT >= 0) {
     if (poly) {
-      T* cf = reinterpret_cast<T*>(smraw + ylm_stage_bytes<T, N>(M, rows));
+      T* cf = reinterpret_cast<T*>(smraw + ylm_stage_bytes<T, N, XP>(M, rows));
       poly_weights<N, LT>(f, axis, poly, LT > 0 ? LT : ell, h0, M, row0, rows, cf, stage);
     }
   }
@@ -450,12 +454,12 @@ __global__ void __launch_bounds__(ylm_thread_cap(LT), sizeof(T) == 4 ? ylm_min_b
     fft_any<XP, C, E, L, kPaddedRows, 1, -1, S::ZW>(v, xb, t, sq, twh);
     // mirrors through shared memory (shuffles would raise this kernel's register count, measured slower)
 #pragma unroll
-    for (int e = 0; e < E; e++) xb[sidx<kPaddedRows, L, 1>(sq, t + Tc * e)] = v[e];
+    for (int e = 0; e < E; e++) xb[sidx<kPaddedRows, L, 1, sizeof(C), Tc>(sq, t, Tc * e)] = v[e];
     fft_sync<S::ZW>();
 #pragma unroll
     for (int e = 0; e < E; e++) {
       const int k = t + Tc * e;
-      const C zm = xb[sidx<kPaddedRows, L, 1>(sq, k ? L - k : 0)];
+      const C zm = xb[sidx<kPaddedRows, L, 1, sizeof(C), Tc>(sq, k ? L - k : 0, 0)];
       if constexpr (XP)
         dst[Lay<N>::row(grow, k)] = r2c_unpack_xp(v[e], zm, ldg_u(twr + k));
       else
@@ -973,14 +977,14 @@ template <typename T, int N> struct Passes {
 
   static void r2c_z(const T* in, C* out, const U* twh, const U* twr, cudaStream_t s) {
     using Z = ZRow<T, N, false>;
-    const size_t smem = (size_t)Z::ROWS * padded_len(S::NH) * sizeof(C);
+    const size_t smem = (size_t)Z::ROWS * row_bytes<T, N, false>();
     set_smem(k_r2c_z<T, N>, smem);
     k_r2c_z<T, N><<<N * N / Z::ROWS, Z::ZT, smem, s>>>(in, out, twh, twr);
   }
   // Launchers taking `xp` run the exact-add variant of their kernel when it is set (FP32 only).
   template <bool XP> static void c2r_z_v(const C* in, T* out, const U* twh, const U* twr, T scale, cudaStream_t s) {
     using Z = ZRow<T, N, XP>;
-    const size_t smem = (size_t)Z::ROWS * padded_len(S::NH) * sizeof(C);
+    const size_t smem = (size_t)Z::ROWS * row_bytes<T, N, XP>();
     set_smem(k_c2r_z<T, N, XP>, smem);
     k_c2r_z<T, N, XP><<<N * N / Z::ROWS, Z::ZT, smem, s>>>(in, out, twh, twr, scale);
   }
@@ -992,7 +996,9 @@ template <typename T, int N> struct Passes {
   }
   // staging area or exchange buffer, and in FP64 the coefficients of the rows' polynomials
   static size_t smem_ylm(int M, int rows) {
-    return ylm_stage_bytes<T, N>(M, rows) + (sizeof(T) == 8 ? (size_t)M * rows * poly_np(kPolyLmax) * sizeof(T) : 0);
+    // the larger of the two transform modes' spacings
+    const size_t st = std::max(ylm_stage_bytes<T, N, false>(M, rows), ylm_stage_bytes<T, N, sizeof(T) == 4>(M, rows));
+    return st + (sizeof(T) == 8 ? (size_t)M * rows * poly_np(kPolyLmax) * sizeof(T) : 0);
   }
   template <int LT, bool XP>
   static void ylm_z_v(const T* f, C* out, int64_t stride, int ell, int h0, int M, const U* twh, const U* twr,

@@ -9,6 +9,7 @@
 #include <algorithm>
 #include "pspec.h"
 #include "launch.h"
+#include "fft_engine.cuh"
 
 using namespace pspec;
 
@@ -161,12 +162,12 @@ pspec_status build_plan(const pspec_params* p, int max_kbins, int nsm, Plan* pl,
   pl->o_f = pl->roundtrip ? take(pl->Sr) : 0;
   pl->o_g = pl->group_max ? take(pl->Sc * pl->group_max) : 0;
   const size_t usz = 16;  // one table factor: float4 or double2
-  pl->o_twh = take(NH * usz);
-  pl->o_twf = take(N * usz);
+  pl->o_twh = take(tw_total(NH) * usz);
+  pl->o_twf = take(tw_total(N) * usz);
   pl->o_twr = take(NH * usz);
   if (pl->xp) {
-    pl->o_twh12 = take(NH * sizeof(float4));
-    pl->o_twf12 = take(N * sizeof(float4));
+    pl->o_twh12 = take(tw_total(NH) * sizeof(float4));
+    pl->o_twf12 = take(tw_total(N) * sizeof(float4));
     pl->o_twr12 = take(NH * sizeof(float4));
   }
   if (f64) {
@@ -345,20 +346,34 @@ template <> ux<double> twiddle<double>(int t, int n) {
   return u;
 }
 
+// The stage tables of every plan of length L (layout: fft_engine.cuh) from w[t] = w_L^t.
+template <typename U> std::vector<U> stage_twiddles(const std::vector<U>& w, int L) {
+  std::vector<U> out;
+  out.reserve(tw_total(L));
+  for (int E : L % 3 == 0 ? std::vector<int>{24} : std::vector<int>{8, 16, 32}) {
+    const CtPlan p = ct_plan(L, E);
+    for (int s = 1; s < p.nst; s++)
+      for (int r = 1; r < p.rad[s]; r++)
+        for (int k = 0; k < p.ns[s]; k++) out.push_back(w[r * k * (L / (p.ns[s] * p.rad[s]))]);
+  }
+  return out;
+}
+
 template <typename T>
 pspec_status upload_tables(Ctx* c) {
   const Plan& pl = c->pl;
   const int N = pl.g.N, NH = pl.g.NH;
   using C = cx<T>;
   using U = ux<T>;
-  std::vector<U> twh(NH), twf(N), twr(NH), phase(3 * N);
+  std::vector<U> wf(N), wh(NH), twr(NH), phase(3 * N);
   std::vector<C> invw(N + NH);
   std::vector<T> axis(3 * N);
-  for (int t = 0; t < N; t++) twf[t] = twiddle<T>(t, N);
+  for (int t = 0; t < N; t++) wf[t] = twiddle<T>(t, N);
   for (int t = 0; t < NH; t++) {
-    twh[t] = twf[2 * t];
-    twr[t] = twf[t];
+    wh[t] = wf[2 * t];
+    twr[t] = wf[t];
   }
+  const std::vector<U> twf = stage_twiddles(wf, N), twh = stage_twiddles(wh, NH);
   const double H = c->p.box_size / N;
   for (int d = 0; d < 3; d++)
     for (int i = 0; i < N; i++) axis[d * N + i] = T(c->p.box_corner[d] + i * H - c->p.observer[d]);
@@ -384,18 +399,21 @@ pspec_status upload_tables(Ctx* c) {
     invw[i] = mk(hi, T(w / (double)hi - 1.0));
   }
   cudaError_t e;
-  e = cudaMemcpyAsync(c->at<U>(pl.o_twh), twh.data(), NH * sizeof(U), cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<U>(pl.o_twf), twf.data(), N * sizeof(U), cudaMemcpyHostToDevice, c->stream);
+  e = cudaMemcpyAsync(c->at<U>(pl.o_twh), twh.data(), twh.size() * sizeof(U), cudaMemcpyHostToDevice, c->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<U>(pl.o_twf), twf.data(), twf.size() * sizeof(U), cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<U>(pl.o_twr), twr.data(), NH * sizeof(U), cudaMemcpyHostToDevice, c->stream);
-  std::vector<float4> twh12(NH), twf12(N), twr12(NH);
+  std::vector<float4> twh12, twf12, twr12(NH);
   if (pl.xp) {
+    std::vector<float4> wf12(N), wh12(NH);
+    for (int t = 0; t < N; t++) wf12[t] = unit_factor12(-2.0 * M_PI * t / N);
     for (int t = 0; t < NH; t++) {
-      twh12[t] = unit_factor12(-2.0 * M_PI * t / NH);
-      twr12[t] = unit_factor12(-2.0 * M_PI * t / N);
+      wh12[t] = wf12[2 * t];
+      twr12[t] = wf12[t];
     }
-    for (int t = 0; t < N; t++) twf12[t] = unit_factor12(-2.0 * M_PI * t / N);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<float4>(pl.o_twh12), twh12.data(), NH * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<float4>(pl.o_twf12), twf12.data(), N * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
+    twf12 = stage_twiddles(wf12, N);
+    twh12 = stage_twiddles(wh12, NH);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<float4>(pl.o_twh12), twh12.data(), twh12.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<float4>(pl.o_twf12), twf12.data(), twf12.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<float4>(pl.o_twr12), twr12.data(), NH * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
   }
   std::vector<double> rinv;

@@ -245,18 +245,18 @@ template <> struct XDft<3> {
 // exact-add arithmetic. The quantum is chosen from the thread's E inputs: every intermediate of
 // a butterfly is a sum of its inputs times factors of modulus <= 1, so each component stays below
 // sqrt(2) times the sum of the inputs' |re| + |im|; the bound passed is twice that sum.
-template <int E, int L, int R, int NS, bool LAST, int LAYOUT, int NSEQ, int DIR>
+template <int E, int L, int R, int NS, int OFF, bool LAST, int LAYOUT, int NSEQ, int DIR>
 __device__ __forceinline__ void stage_xp(float2 (&v)[E], float2* sm, int t, int seq, const float4* __restrict__ tw) {
   constexpr int Q = E / R;
   constexpr int Tc = L / E;
-  constexpr int TSTEP = L / (NS * R);
+  tw += OFF - NS;  // entry r of k at r NS + k
   constexpr bool kShared = (Q > 1) && (NS > 1) && !LAST && (NS <= Tc);
   float4 ws[kShared ? R : 1];
   if constexpr (kShared) {
     const int k = t & (NS - 1);
 #pragma unroll
     for (int r = 1; r < R; r++) {
-      ws[r] = ldg_u(tw + r * k * TSTEP);
+      ws[r] = ldg_u(tw + r * NS + k);
       if (DIR > 0) ws[r] = uconj(ws[r]);
     }
   }
@@ -276,7 +276,7 @@ __device__ __forceinline__ void stage_xp(float2 (&v)[E], float2* sm, int t, int 
         if constexpr (kShared) {
           w = ws[r];
         } else {
-          w = ldg_u(tw + r * k * TSTEP);
+          w = ldg_u(tw + r * NS + k);
           if (DIR > 0) w = uconj(w);
         }
         u[r] = xtw(v[q + r * Q], w, M);  // the 12-bit twiddle table
@@ -291,7 +291,7 @@ __device__ __forceinline__ void stage_xp(float2 (&v)[E], float2* sm, int t, int 
     } else {
       const int base = (j - k) * R + k;
 #pragma unroll
-      for (int r = 0; r < R; r++) sm[sidx<LAYOUT, L, NSEQ>(seq, base + r * NS)] = xround(u[r]);
+      for (int r = 0; r < R; r++) sm[sidx<LAYOUT, L, NSEQ, 8, Tc>(seq, base, r * NS)] = xround(u[r]);
     }
   }
 }
@@ -305,11 +305,11 @@ __device__ __forceinline__ void fft_xp(float2 (&v)[E], float2* sm, int t, int se
   static_for<0, P.nst>([&](auto s_) {
     constexpr int s = decltype(s_)::value;
     constexpr bool last = (s == P.nst - 1);
-    stage_xp<E, L, P.rad[s], P.ns[s], last, LAYOUT, NSEQ, DIR>(v, sm, t, seq, tw);
+    stage_xp<E, L, P.rad[s], P.ns[s], tw_base(L, E) + tw_stage_off(L, E, s), last, LAYOUT, NSEQ, DIR>(v, sm, t, seq, tw);
     if constexpr (!last) {
       fft_sync<WARP>();
 #pragma unroll
-      for (int e = 0; e < E; e++) v[e] = sm[sidx<LAYOUT, L, NSEQ>(seq, t + Tc * e)];
+      for (int e = 0; e < E; e++) v[e] = sm[sidx<LAYOUT, L, NSEQ, 8, Tc>(seq, t, Tc * e)];
       fft_sync<WARP>();
     }
   });
