@@ -538,6 +538,9 @@ __global__ void __launch_bounds__(col_block_tile<T, N>() * (N / col_elems<T, N, 
 // X = (F1 + exp(-i k.s) F2)/2 (interlaced) or F1; divided by W(k) when compensating; zeroed
 // where some n_d = -N/2 when the inverse transform follows; stored as F0.
 // Binned: sum over modes of mult |X|^2 (slot SLOT_P0). Persistent over tiles.
+// F0 is read and written in place, so the loads of one element would wait for the store of the one
+// before (long-scoreboard stalls at 15-20% of the DRAM rate): all of a thread's loads of F0 and of the bin
+// table come first, then the arithmetic and the stores, then the bins.
 template <typename T, int N>
 __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E>(col_threads<T, N>()))
     k_combine_x(const cx<T>* B, cx<T>* F0, const ux<T>* __restrict__ twf, int interlaced, int compensate,
@@ -570,15 +573,23 @@ __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E
     const T wyz = iwy.x * iwz.x, lyz = iwy.y + iwz.y;
     const int syz = sfreq<N>(j) + kz + 3 * N / 2;  // index of exp(-i pi (nx + ny + nz) / N) less nx
     const T mult = kz ? T(2) : T(1);
+    C A[E];
+    int bin[E];
+    if (interlaced) {
+#pragma unroll
+      for (int e = 0; e < E; e++) A[e] = F0[off + (t + Tc * e) * si];
+    }
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+      const int ii = t + Tc * e, nx = sfreq<N>(ii), n2 = nx * nx + ny * ny + kz * kz;
+      bin[e] = j == N / 2 || ii == N / 2 || n2 == 0 ? -1 : __ldg(ba.bin_of_n2 + n2);
+    }
 #pragma unroll
     for (int e = 0; e < E; e++) {
       const int ii = t + Tc * e;
       const int64_t addr = off + ii * si;
       C X = v[e];
-      if (interlaced) {
-        const C A = F0[addr];
-        X = cscale(cadd(A, umul(X, ldg_u(phase + syz + sfreq<N>(ii)))), T(0.5));
-      }
+      if (interlaced) X = cscale(cadd(A[e], umul(X, ldg_u(phase + syz + sfreq<N>(ii)))), T(0.5));
       if (compensate == 1 || compensate == 2) {
         // 1/W = prod_d hi_d (1 + lo_d): the relative rounding errors lo_d of the per-axis
         // factors enter the roundings of the products X * w3, so that no per-axis
@@ -590,16 +601,14 @@ __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E
       const bool nyq = (ii == N / 2) || (j == N / 2);
       if (roundtrip && nyq) X = mk(T(0), T(0));
       F0[addr] = X;
-      if (!nyq) {
-        const int nx = sfreq<N>(ii);
-        const int n2 = nx * nx + ny * ny + kz * kz;
-        const int b = ba.bin_of_n2[n2];
-        if (b >= 0 && n2 > 0) {
-          T x2 = X.x * X.x + X.y * X.y;
-          if (compensate == 3) x2 = per_mode_w2<T, N>(x2, invw, ii, j, kz);  // compensation per mode
-          wb.add(b, mult * x2);
-        }
-      }
+      v[e] = X;
+    }
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+      if (bin[e] < 0) continue;
+      T x2 = fma_t(v[e].y, v[e].y, v[e].x * v[e].x);
+      if (compensate == 3) x2 = per_mode_w2<T, N>(x2, invw, t + Tc * e, j, kz);  // compensation per mode
+      wb.add(bin[e], mult * x2);
     }
     __syncthreads();
     wb.fold();
@@ -613,6 +622,7 @@ __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E
 // of the group, the x-pass of G_h and acc += Y_{l,m(h)}(khat) Re[G_h conj(F0)] per mode;
 // then mult * acc into the bins of `slot`. For odd l, F0 is stored times i, so the same
 // product gives Re[G conj(i F0)] = Im[G conj(F0)].
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 template <typename C> __device__ __forceinline__ C f0_for(C f, int odd) { return odd ? mk(-f.y, f.x) : f; }
 
 template <typename T, int N, bool YT, bool XP>
@@ -634,6 +644,9 @@ __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E
   wb.init();
   const int c = threadIdx.x % TW, t = threadIdx.x / TW;
   constexpr int64_t si = Lay<N>::XI, modes = (int64_t)N * N * NH;
+  // 24 elements (radix 3): the table values are loaded after the transform, which needs the registers
+  // (spills otherwise), and the next tile is fetched into L2 meanwhile
+  constexpr bool kLateY = E > 8;
   __syncthreads();
   for (int q = blockIdx.x; q < ba.n_xtiles * SUB; q += gridDim.x) {
     const int tile = ba.xtiles[q / SUB];
@@ -659,9 +672,27 @@ __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E
 #pragma unroll
       for (int e = 0; e < E; e++) {
         v[e] = Gs[off + (t + Tc * e) * si];
-        if constexpr (YT) yv[e] = __ldg(Ys + (t + Tc * e) * TW);
+        if constexpr (YT && !kLateY) yv[e] = __ldg(Ys + (t + Tc * e) * TW);
+      }
+      if constexpr (YT && kLateY) {
+        // the next stage of copies: this tile's next harmonic, or the next tile's F0 and first harmonic
+        const int nq = s + 1 < M ? q : q + (int)gridDim.x;
+        if (nq < ba.n_xtiles * SUB) {
+          const int nt = ba.xtiles[nq / SUB], nkt = nt / N, nj = nt - nkt * N;
+          const int64_t at = Lay<N>::at(0, nj, nkt * Lay<N>::TW + (nq % SUB) * TW);
+          const C* Gn = G + (s + 1 < M ? (int64_t)(s + 1) * spec_stride : 0) + at;
+          const float* Yn = ytab + (s + 1 < M ? (int64_t)(s + 1) * modes : 0) + Lay<N>::table_tile(nkt, nj);
+          for (int i = threadIdx.x; i < N; i += TW * Tc) prefetch_l2(Gn + i * si);
+          for (int i = threadIdx.x; i < N * TW / 32; i += TW * Tc) prefetch_l2(Yn + i * 32);
+          if (s + 1 == M)
+            for (int i = threadIdx.x; i < N; i += TW * Tc) prefetch_l2(F0 + at + i * si);
+        }
       }
       fft_any<XP, C, E, N, kInterleaved, TW, -1>(v, sm, t, c, twf);
+      if constexpr (YT && kLateY) {
+#pragma unroll
+        for (int e = 0; e < E; e++) yv[e] = __ldg(Ys + (t + Tc * e) * TW);
+      }
 #pragma unroll
       for (int e = 0; e < E; e++) {
         const T fx = T(sfreq<N>(t + Tc * e));
