@@ -139,10 +139,12 @@ __device__ __forceinline__ T per_mode_w2(T v, const cx<T>* __restrict__ iw, int 
 // ------------------------------------------------------------------ pass z: r2c of plain rows
 template <typename T, int N>
 __global__ void __launch_bounds__(ZRow<T, N, false>::ZT, min_blocks<T, ZRow<T, N, false>::E>(ZRow<T, N, false>::ZT))
-    k_r2c_z(const T* __restrict__ in, cx<T>* __restrict__ out, const ux<T>* __restrict__ twh,
-            const ux<T>* __restrict__ twr) {
+    k_r2c_z(const T* __restrict__ in, cx<T>* __restrict__ out, int64_t in_stride, int64_t out_stride,
+            const ux<T>* __restrict__ twh, const ux<T>* __restrict__ twr) {
   using C = cx<T>;
   using S = ZRow<T, N, false>;
+  in += blockIdx.y * in_stride;  // the interlaced mesh
+  out += blockIdx.y * out_stride;
   constexpr int L = N / 2, E = S::E, Tc = S::Tz;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
@@ -267,38 +269,38 @@ __device__ __forceinline__ void poly_weights(const double* __restrict__ f, const
     cf[q] = acc;
   }
   __syncthreads();
-  for (int r = 0; r < rows; r++) {
+  // every node of the block's rows (rows of a small mesh are shorter than the block)
+  for (int q = threadIdx.x; q < rows * N; q += blockDim.x) {
+    const int r = q / N, kk = q - r * N;
     const int grow = row0 + r, i = grow / N, j = grow - i * N;
     const double vx = axis[i], vy = axis[N + j], rho2 = vx * vx + vy * vy;
     const double* cr = cf + r * M * NP;
-    for (int kk = threadIdx.x; kk < N; kk += blockDim.x) {
-      const double z = axis[2 * N + kk], z2 = z * z, r2 = rho2 + z2;
-      double g = f[(int64_t)grow * N + kk];
-      if (ell & 1) {
-        const double inv = rsqrt_newton(r2), inv2 = inv * inv;
-        g *= inv;
-        for (int p = 1; p < ell; p += 2) g *= inv2;
-      } else {
-        const double inv2 = rcp_newton(r2);
-        for (int p = 0; p < ell; p += 2) g *= inv2;
-      }
-      if (r2 == 0.0) g = 0.0;  // the node at the observer
-      const double gz = g * z;
-      double* st = stage + r * N + kk;
-      auto one = [&](int s, int a) {
-        const double* c = cr + s * NP;
-        const int deg = (ell - a) >> 1;
-        double v = c[deg];
+    const double z = axis[2 * N + kk], z2 = z * z, r2 = rho2 + z2;
+    double g = f[(int64_t)grow * N + kk];
+    if (ell & 1) {
+      const double inv = rsqrt_newton(r2), inv2 = inv * inv;
+      g *= inv;
+      for (int p = 1; p < ell; p += 2) g *= inv2;
+    } else {
+      const double inv2 = rcp_newton(r2);
+      for (int p = 0; p < ell; p += 2) g *= inv2;
+    }
+    if (r2 == 0.0) g = 0.0;  // the node at the observer
+    const double gz = g * z;
+    double* st = stage + r * N + kk;
+    auto one = [&](int s, int a) {
+      const double* c = cr + s * NP;
+      const int deg = (ell - a) >> 1;
+      double v = c[deg];
 #pragma unroll
-        for (int p = deg - 1; p >= 0; p--) v = fma(v, z2, c[p]);
-        st[s * rows * N] = v * (((ell - a) & 1) ? gz : g);
-      };
-      if (LT > 0 && h0 == 0 && M == 2 * LT + 1) {
+      for (int p = deg - 1; p >= 0; p--) v = fma(v, z2, c[p]);
+      st[s * rows * N] = v * (((ell - a) & 1) ? gz : g);
+    };
+    if (LT > 0 && h0 == 0 && M == 2 * LT + 1) {
 #pragma unroll
-        for (int s = 0; s < 2 * LT + 1; s++) one(s, harm_a(s));
-      } else {
-        for (int s = 0; s < M; s++) one(s, harm_a(h0 + s));
-      }
+      for (int s = 0; s < 2 * LT + 1; s++) one(s, harm_a(s));
+    } else {
+      for (int s = 0; s < M; s++) one(s, harm_a(h0 + s));
     }
   }
 }
@@ -541,6 +543,24 @@ __global__ void __launch_bounds__(col_block_tile<T, N>() * (N / col_elems<T, N, 
 // F0 is read and written in place, so the loads of one element would wait for the store of the one
 // before (long-scoreboard stalls at 15-20% of the DRAM rate): all of a thread's loads of F0 and of the bin
 // table come first, then the arithmetic and the stores, then the bins.
+// FP64: a thread's values and bins go through its own slots of shared memory and are added in an order
+// rotated by the lane, so that the lanes of a warp add modes of different |n| (their own order puts
+// neighbouring modes, and up to 13 lanes of one bin, into one instruction: each retry of the shared
+// compare-and-swap is another FP64 addition of the whole warp).
+template <int E> __device__ __forceinline__ void rotated_add(const WarpBins<double>& wb, const double (&a)[E], const int (&bin)[E],
+                                                             double2* slots) {
+  static_assert((E & (E - 1)) == 0, "rotation by a mask");
+  // value and bin of element e as one 16-byte slot, at [e][thread]
+#pragma unroll
+  for (int e = 0; e < E; e++) slots[e * blockDim.x + threadIdx.x] = make_double2(a[e], __hiloint2double(0, bin[e]));
+#pragma unroll
+  for (int e = 0; e < E; e++) {
+    const double2 s = slots[((e + threadIdx.x + (threadIdx.x >> 3)) & (E - 1)) * blockDim.x + threadIdx.x];
+    const int b = __double2loint(s.y);
+    if (b >= 0) wb.add(b, s.x);
+  }
+}
+
 template <typename T, int N>
 __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E>(col_threads<T, N>()))
     k_combine_x(const cx<T>* B, cx<T>* F0, const ux<T>* __restrict__ twf, int interlaced, int compensate,
@@ -603,6 +623,16 @@ __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E
       F0[addr] = X;
       v[e] = X;
     }
+    if constexpr (sizeof(T) == 8 && (E & (E - 1)) == 0) {
+      T a[E];
+#pragma unroll
+      for (int e = 0; e < E; e++) {
+        T x2 = fma_t(v[e].y, v[e].y, v[e].x * v[e].x);
+        if (compensate == 3) x2 = per_mode_w2<T, N>(x2, invw, t + Tc * e, j, kz);
+        a[e] = mult * x2;
+      }
+      rotated_add(wb, a, bin, sm);  // the exchange buffer is free: N * TW slots of 16 bytes
+    } else
 #pragma unroll
     for (int e = 0; e < E; e++) {
       if (bin[e] < 0) continue;
@@ -770,6 +800,11 @@ __global__ void __launch_bounds__(col_threads<double, N>(), Shape<N>::E == 8 && 
   wb.w = wb.b + ba.nk;
   wb.init();
   const int NP = poly_np(ell), NI = ell + 1;
+  // this block's share of the group's harmonics (gridDim.y > 1 on small meshes: the bins are sums over them)
+  const int share = (M + gridDim.y - 1) / gridDim.y;
+  G += (int64_t)(blockIdx.y * share) * spec_stride;
+  h0 += blockIdx.y * share;
+  M = min(share, M - (int)blockIdx.y * share);
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
     const double x = (double)sfreq<N>(i);
     xs[i] = x;
@@ -831,23 +866,30 @@ __global__ void __launch_bounds__(col_threads<double, N>(), Shape<N>::E == 8 && 
     if (j != N / 2) {
       const double mult = kz ? 2.0 : 1.0;
       const int ny = sfreq<N>(j);
+      double val[E];
+      int bin[E];
 #pragma unroll
       for (int e = 0; e < E; e++) {
-        const int ii = t + Tc * e;
-        if (ii == N / 2) continue;
-        const int nx = sfreq<N>(ii);
-        const int n2 = nx * nx + ny * ny + kz * kz;
-        const int b = ba.bin_of_n2[n2];
-        if (b >= 0 && n2 > 0) {
+        const int ii = t + Tc * e, nx = sfreq<N>(ii), n2 = nx * nx + ny * ny + kz * kz;
+        bin[e] = ii == N / 2 || n2 == 0 ? -1 : __ldg(ba.bin_of_n2 + n2);
+        val[e] = 0.0;
+        if (bin[e] >= 0) {
           const double2 f0 = f0_for(F0[off + ii * si], ba.odd);
           double a = S[e].x * f0.x + S[e].y * f0.y;
-          const double ri = kp.rinv[n2];
+          const double ri = __ldg(kp.rinv + n2);
           if (ell & 1) a *= ri;
           const double ri2 = ri * ri;
           for (int p = 1; p < ell; p += 2) a *= ri2;
           if (ba.permode_w) a = per_mode_w2<double, N>(a, static_cast<const double2*>(ba.permode_w), ii, j, kz);
-          wb.add(b, mult * a);
+          val[e] = mult * a;
         }
+      }
+      if constexpr ((E & (E - 1)) == 0) {
+        rotated_add(wb, val, bin, sm);
+      } else {
+#pragma unroll
+        for (int e = 0; e < E; e++)
+          if (bin[e] >= 0) wb.add(bin[e], val[e]);
       }
     }
     __syncthreads();
@@ -1006,11 +1048,12 @@ template <typename T, int N> struct Passes {
            (size_t)((S::CT + 31) / 32) * nk * sizeof(float);
   }
 
-  static void r2c_z(const T* in, C* out, const U* twh, const U* twr, cudaStream_t s) {
+  static void r2c_z(const T* in, C* out, int64_t in_stride, int64_t out_stride, int nmesh, const U* twh, const U* twr,
+                    cudaStream_t s) {
     using Z = ZRow<T, N, false>;
     const size_t smem = (size_t)Z::ROWS * row_bytes<T, N, false>();
     set_smem(k_r2c_z<T, N>, smem);
-    k_r2c_z<T, N><<<N * N / Z::ROWS, Z::ZT, smem, s>>>(in, out, twh, twr);
+    k_r2c_z<T, N><<<dim3(N * N / Z::ROWS, nmesh), Z::ZT, smem, s>>>(in, out, in_stride, out_stride, twh, twr);
   }
   // Launchers taking `xp` run the exact-add variant of their kernel when it is set (FP32 only).
   template <bool XP> static void c2r_z_v(const C* in, T* out, const U* twh, const U* twr, T scale, cudaStream_t s) {
@@ -1123,7 +1166,12 @@ template <typename T, int N> struct Passes {
                        const BinArgs& ba, int ctas, const KPoly& kp, cudaStream_t s) {
     const size_t smem = smem_bin_fx(ba.nk);
     set_smem(k_bin_fx<N, LT>, smem);
-    k_bin_fx<N, LT><<<ctas, col_threads<T, N>(), smem, s>>>(G, stride, ell, h0, M, F0, twf, slot, ba, kp);
+    // a mesh with fewer tiles than four blocks per SM splits the harmonics over blocks (64^3, l = 4: 64 us
+    // with 128 blocks)
+    const int tiles = ba.n_xtiles * (Lay<N>::TW / TWB);
+    const int share = (M + std::max(1, 4 * ba.nsm / std::max(1, tiles)) - 1) / std::max(1, 4 * ba.nsm / std::max(1, tiles));
+    const dim3 grid(ctas, (M + share - 1) / share);
+    k_bin_fx<N, LT><<<grid, col_threads<T, N>(), smem, s>>>(G, stride, ell, h0, M, F0, twf, slot, ba, kp);
   }
   template <bool XP>
   static void bin_x_v(const C* G, int64_t stride, int ell, int h0, int M, const C* F0, const U* twf, int slot,

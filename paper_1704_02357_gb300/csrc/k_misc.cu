@@ -4,6 +4,7 @@
 //   a6 finalise:     Sec. 2.1 eq. Pell-ours (4 pi / (I N_b) for l >= 2; noise for l = 0).
 //   a7 wedges:       Sec. 2.2 eqs. wedge-est and Lbar.
 #include <cmath>
+#include <type_traits>
 #include "launch.h"
 #include "intconv.cuh"
 
@@ -793,8 +794,9 @@ __device__ __forceinline__ void tile_record(unsigned* acc, const uint4 r, float 
 }
 
 // Threads of a tile's block: three blocks' accumulators (64 KB each with interlacing) fit an SM, and the
-// shared atomics need the warps: 512 threads keep 48 warps resident, 256 kept 24.
-constexpr int kTilePaintThreads = 512;
+// shared atomics need the warps: 512 threads keep 48 warps resident, 256 kept 24. Meshes of at most
+// kFewTiles tiles (96^3) leave SMs idle or with one block: 1024 threads shorten each tile's chain of records.
+constexpr int kTilePaintThreads = 512, kFewTilesThreads = 1024, kFewTiles = 216;
 
 // One block per tile (every tile, so that empty tiles store their zeros): sums its records into
 // shared 64-bit accumulators (lo words of both meshes, then hi words), then stores each cell of
@@ -802,8 +804,8 @@ constexpr int kTilePaintThreads = 512;
 // skips the accumulators. With cached randoms meshes r1, r2 (batched mocks; r1 null: none) it stores
 // cell - alpha * randoms cell instead: the same FMA as a pass of its own over the meshes, which
 // would read and write each once more (135 us a mesh at 384^3).
-template <int WIN, bool INTER>
-__global__ void __launch_bounds__(kTilePaintThreads, INTER ? 3 : 4) k_ptile_paint(TileArgs ta, float* __restrict__ m1, float* __restrict__ m2,
+template <int WIN, bool INTER, int NT>
+__global__ void __launch_bounds__(NT, NT <= 512 ? 3 : 1) k_ptile_paint(TileArgs ta, float* __restrict__ m1, float* __restrict__ m2,
                                                      int N, const double* __restrict__ fix,
                                                      const float* __restrict__ r1, const float* __restrict__ r2,
                                                      const double* __restrict__ alpha) {
@@ -920,24 +922,34 @@ template <typename K> static void set_smem_attr(K kernel, size_t bytes) {
   if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+template <int WIN, bool INTER>
+static void ptile_paint_v(const TileArgs& ta, float* m1, float* m2, int N, const double* fix, const float* r1,
+                          const float* r2, const double* alpha, cudaStream_t s) {
+  const int ntiles = (N / kPT) * (N / kPT) * (N / kPT);
+  const size_t smem = (size_t)(INTER ? 2 : 1) * kPT3 * sizeof(unsigned long long);
+  auto go = [&](auto nt) {
+    constexpr int NT = decltype(nt)::value;
+    set_smem_attr(k_ptile_paint<WIN, INTER, NT>, smem);
+    k_ptile_paint<WIN, INTER, NT><<<ntiles, NT, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
+  };
+  if (ntiles <= kFewTiles)
+    go(std::integral_constant<int, kFewTilesThreads>{});
+  else
+    go(std::integral_constant<int, kTilePaintThreads>{});
+}
+
 void launch_ptile_paint(const TileArgs& ta, int window, int interlaced, float* m1, float* m2, int N,
                         const double* fix, const float* r1, const float* r2, const double* alpha, cudaStream_t s) {
-  const int ntiles = (N / kPT) * (N / kPT) * (N / kPT);
-  const size_t smem = (size_t)(interlaced ? 2 : 1) * kPT3 * sizeof(unsigned long long);
   if (window == PSPEC_WINDOW_CIC) {
-    if (interlaced) {
-      set_smem_attr(k_ptile_paint<PSPEC_WINDOW_CIC, true>, smem);
-      k_ptile_paint<PSPEC_WINDOW_CIC, true><<<ntiles, kTilePaintThreads, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
-    } else {
-      k_ptile_paint<PSPEC_WINDOW_CIC, false><<<ntiles, kTilePaintThreads, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
-    }
+    if (interlaced)
+      ptile_paint_v<PSPEC_WINDOW_CIC, true>(ta, m1, m2, N, fix, r1, r2, alpha, s);
+    else
+      ptile_paint_v<PSPEC_WINDOW_CIC, false>(ta, m1, m2, N, fix, r1, r2, alpha, s);
   } else {
-    if (interlaced) {
-      set_smem_attr(k_ptile_paint<PSPEC_WINDOW_TSC, true>, smem);
-      k_ptile_paint<PSPEC_WINDOW_TSC, true><<<ntiles, kTilePaintThreads, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
-    } else {
-      k_ptile_paint<PSPEC_WINDOW_TSC, false><<<ntiles, kTilePaintThreads, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
-    }
+    if (interlaced)
+      ptile_paint_v<PSPEC_WINDOW_TSC, true>(ta, m1, m2, N, fix, r1, r2, alpha, s);
+    else
+      ptile_paint_v<PSPEC_WINDOW_TSC, false>(ta, m1, m2, N, fix, r1, r2, alpha, s);
   }
 }
 
@@ -1028,28 +1040,30 @@ struct EllList {
 __global__ void k_finalize(const double* __restrict__ bins, const double* __restrict__ nmodes_in,
                            const double* __restrict__ ksum, int nk, EllList el, const double* __restrict__ derived,
                            double* P, double* kmean, double* nmodes, int cart) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  // row 0: n_modes and k_mean; row 1 + i: P of ell[i] (FP64 divisions are long chains: one or two per thread)
+  const int b = blockIdx.x * blockDim.x + threadIdx.x, i = (int)blockIdx.y - 1;
   if (b >= nk) return;
   const double n = nmodes_in[b];
-  const double I = derived[D_I], S = derived[D_S];
   const double nan = __longlong_as_double(0x7ff8000000000000ULL);
-  nmodes[b] = n;
-  kmean[b] = n > 0.0 ? ksum[b] / n : nan;
-  for (int i = 0; i < el.n; i++) {
-    const int ell = el.ell[i];
-    double v;
-    const double B0 = bins[SLOT_P0 * nk + b];
-    if (ell == 0)
-      v = (B0 / n - S) / I;
-    else if (!cart)
-      v = 4.0 * M_PI * bins[(SLOT_ELL0 + i) * nk + b] / (I * n);
-    else {
-      // Cartesian: A2, A4 = sum mult (khat . rhat)^2, ^4 terms; L_2 = (3mu^2-1)/2, L_4 = (35mu^4-30mu^2+3)/8
-      const double A2 = bins[SLOT_ELL0 * nk + b], A4 = bins[(SLOT_ELL0 + 1) * nk + b];
-      v = ell == 2 ? 2.5 * (3.0 * A2 - B0) / (I * n) : 1.125 * (35.0 * A4 - 30.0 * A2 + 3.0 * B0) / (I * n);
-    }
-    P[(int64_t)i * nk + b] = n > 0.0 ? v : nan;
+  if (i < 0) {
+    nmodes[b] = n;
+    kmean[b] = n > 0.0 ? ksum[b] / n : nan;
+    return;
   }
+  const double I = derived[D_I], S = derived[D_S];
+  const int ell = el.ell[i];
+  double v;
+  const double B0 = bins[SLOT_P0 * nk + b];
+  if (ell == 0)
+    v = (B0 / n - S) / I;
+  else if (!cart)
+    v = 4.0 * M_PI * bins[(SLOT_ELL0 + i) * nk + b] / (I * n);
+  else {
+    // Cartesian: A2, A4 = sum mult (khat . rhat)^2, ^4 terms; L_2 = (3mu^2-1)/2, L_4 = (35mu^4-30mu^2+3)/8
+    const double A2 = bins[SLOT_ELL0 * nk + b], A4 = bins[(SLOT_ELL0 + 1) * nk + b];
+    v = ell == 2 ? 2.5 * (3.0 * A2 - B0) / (I * n) : 1.125 * (35.0 * A4 - 30.0 * A2 + 3.0 * B0) / (I * n);
+  }
+  P[(int64_t)i * nk + b] = n > 0.0 ? v : nan;
 }
 
 void launch_finalize(const double* bins, const double* nmodes_in, const double* ksum, int nk, const int32_t* ells,
@@ -1058,7 +1072,7 @@ void launch_finalize(const double* bins, const double* nmodes_in, const double* 
   EllList el;
   el.n = n_ells;
   for (int i = 0; i < n_ells; i++) el.ell[i] = ells[i];
-  k_finalize<<<(nk + 127) / 128, 128, 0, s>>>(bins, nmodes_in, ksum, nk, el, derived, P, k_mean, n_modes, cartesian);
+  k_finalize<<<dim3((nk + 127) / 128, n_ells + 1), 128, 0, s>>>(bins, nmodes_in, ksum, nk, el, derived, P, k_mean, n_modes, cartesian);
 }
 
 // ------------------------------------------------------------------ a7: wedges

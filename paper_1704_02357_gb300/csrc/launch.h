@@ -74,6 +74,7 @@ struct BinArgs {
   // (a tile whose columns all have ny^2 + kz^2 beyond the last bin is left out)
   const int32_t* xtiles;
   int n_xtiles;
+  int nsm;
 };
 
 // a1: per-block partial sums of one weighted catalog; final combine into `derived`.
@@ -139,7 +140,8 @@ void launch_ptile_paint(const TileArgs& ta, int window, int interlaced, float* m
 //   col_tile(N): kz columns per y/x tile, a power of two dividing N/2 with at most 512
 //                threads (N/E per column) and at most 16 columns;
 //   z_rows(N):   rows per block of the plain z passes, a power of two dividing N^2 with at
-//                most 512 threads (N/(2E) per row).
+//                most 512 threads (N/(2E) per row), 128 up to 128^3 so that the blocks of a small
+//                mesh spread over the SMs.
 constexpr int elems_per_thread(int N) { return N % 3 == 0 ? 24 : 8; }
 constexpr int col_tile(int N) {
   const int tc = N / elems_per_thread(N);
@@ -153,7 +155,7 @@ constexpr int col_tile(int N) {
 constexpr int z_elems(int N) { return N % 3 == 0 ? 24 : (N / 2 >= 128 ? 16 : 8); }
 constexpr int z_rows(int N) {
   const int tz = (N / 2) / z_elems(N);
-  int cap = 512 / tz, r = 1;
+  int cap = (N <= 128 ? 128 : 512) / tz, r = 1;
   while (r * 2 <= cap && ((long long)N * N) % (r * 2) == 0) r *= 2;
   return r;
 }
@@ -225,7 +227,8 @@ struct KPoly {
 template <typename T> struct PassTable {
   int N, E, tw, rows_z, tz;
   int tz_xp;  // threads per row of the exact-add z passes
-  void (*r2c_z)(const T*, cx<T>*, const ux<T>*, const ux<T>*, cudaStream_t);
+  // in, out, strides to the second mesh and spectrum, meshes (1 or 2), ...
+  void (*r2c_z)(const T*, cx<T>*, int64_t, int64_t, int, const ux<T>*, const ux<T>*, cudaStream_t);
   void (*c2r_z)(const cx<T>*, T*, const ux<T>*, const ux<T>*, T, int, cudaStream_t);
   // ..., rows, Y_lm(rhat) table slot of the group's first harmonic (FP32) or nullptr, real-space
   // polynomials (FP64), xp

@@ -328,22 +328,42 @@ float4 unit_factor12(double a) {
   return make_float4((float)c12, (float)s12, (float)(c - c12), (float)(s - s12));
 }
 
-// Twiddle exp(-2 pi i t/n) as the transform stages take it: unit_factor in FP32; in FP64 contexts four
-// integers {c_h, c_l, s_h, s_l} of the fixed-point stages, each component h 2^-30 + l 2^-62.
-template <typename T> ux<T> twiddle(int t, int n) { return unit_factor<T>(-2.0 * M_PI * t / n); }
-template <> ux<double> twiddle<double>(int t, int n) {
-  const long double a = -2.0L * std::acos(-1.0L) * t / n;
-  int32_t w[4];
-  for (int i = 0; i < 2; i++) {
-    const int64_t q = (int64_t)std::llrint((i ? std::sin(a) : std::cos(a)) * 4611686018427387904.0L);  // 2^62
-    const int64_t h = (q + (1ll << 31)) >> 32;
-    w[2 * i] = (int32_t)h;
-    w[2 * i + 1] = (int32_t)std::max<int64_t>(q - h * (1ll << 32), INT_MIN + 1);  // its negative is needed too
+// Twiddles exp(-2 pi i t/n), t < n, as the transform stages take them: unit_factor in FP32; in FP64 contexts
+// four integers {c_h, c_l, s_h, s_l} of the fixed-point stages, each component h 2^-30 + l 2^-62, from
+// one octant in extended precision (n is a multiple of 8).
+template <typename T> std::vector<ux<T>> twiddles(int n) {
+  std::vector<ux<T>> w(n);
+  for (int t = 0; t < n; t++) w[t] = unit_factor<T>(-2.0 * M_PI * t / n);
+  return w;
+}
+template <> std::vector<ux<double>> twiddles<double>(int n) {
+  std::vector<int64_t> c(n / 8 + 1), s(n / 8 + 1);  // cos, sin(2 pi t/n) 2^62
+  for (int t = 0; t <= n / 8; t++) {
+    const long double a = 2.0L * std::acos(-1.0L) * t / n;
+    c[t] = (int64_t)std::llrint(std::cos(a) * 4611686018427387904.0L);
+    s[t] = (int64_t)std::llrint(std::sin(a) * 4611686018427387904.0L);
   }
-  ux<double> u;
-  static_assert(sizeof u == sizeof w, "one table entry");
-  std::memcpy(&u, w, sizeof u);
-  return u;
+  std::vector<ux<double>> w(n);
+  for (int t = 0; t < n; t++) {
+    const int quarter = 4 * t / n, r = t - quarter * (n / 4);
+    const bool low = r <= n / 8;
+    int64_t x = low ? c[r] : s[n / 4 - r], y = low ? s[r] : c[n / 4 - r];
+    for (int q = 0; q < quarter; q++) {  // times i
+      const int64_t nx = -y;
+      y = x;
+      x = nx;
+    }
+    const int64_t v[2] = {x, -y};
+    int32_t e[4];
+    for (int i = 0; i < 2; i++) {
+      const int64_t h = (v[i] + (1ll << 31)) >> 32;
+      e[2 * i] = (int32_t)h;
+      e[2 * i + 1] = (int32_t)std::max<int64_t>(v[i] - h * (1ll << 32), INT_MIN + 1);  // its negative is needed too
+    }
+    static_assert(sizeof(ux<double>) == sizeof e, "one table entry");
+    std::memcpy(&w[t], e, sizeof e);
+  }
+  return w;
 }
 
 // The stage tables of every plan of length L (layout: fft_engine.cuh) from w[t] = w_L^t.
@@ -365,10 +385,10 @@ pspec_status upload_tables(Ctx* c) {
   const int N = pl.g.N, NH = pl.g.NH;
   using C = cx<T>;
   using U = ux<T>;
-  std::vector<U> wf(N), wh(NH), twr(NH), phase(3 * N);
+  const std::vector<U> wf = twiddles<T>(N);
+  std::vector<U> wh(NH), twr(NH), phase(3 * N);
   std::vector<C> invw(N + NH);
   std::vector<T> axis(3 * N);
-  for (int t = 0; t < N; t++) wf[t] = twiddle<T>(t, N);
   for (int t = 0; t < NH; t++) {
     wh[t] = wf[2 * t];
     twr[t] = wf[t];
@@ -677,6 +697,7 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
   ba.odd = 0;
   ba.xtiles = c->at<int32_t>(pl.o_xtiles);
   ba.n_xtiles = c->n_xtiles;
+  ba.nsm = c->nsm;
   cudaError_t e = cudaMemsetAsync(ba.bins, 0, (size_t)(SLOT_ELL0 + std::max(n_ells, 2)) * nk * sizeof(double), s);
   if (e != cudaSuccess) return cuda_fail(c, e, "bins clear");
   int64_t transforms = 0;
@@ -695,14 +716,14 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
   };
 
   // a3: F1 (and F2), combine + compensate -> F0 with the l = 0 sums; round trip -> f
-  TRY(run(c, PSPEC_K_FFT_Z, acc(Sr + Sc), [&] { PT->r2c_z(m1, F0, twh, twr, s); }));
-  TRY(run(c, PSPEC_K_FFT_Y, acc(2 * Sc), [&] { PT->fft_y(F0, 0, 1, twf, -1, c->tune.tile_y, INT_MAX, 0, s); }));
-  transforms++;
+  // both meshes of an interlaced pair in one launch per pass
+  const int nm_in = c->p.interlaced ? 2 : 1;
+  TRY(run(c, PSPEC_K_FFT_Z, acc(nm_in * (Sr + Sc)), [&] { PT->r2c_z(m1, F0, m2 - m1, W - F0, nm_in, twh, twr, s); }));
+  TRY(run(c, PSPEC_K_FFT_Y, acc(2 * nm_in * Sc),
+          [&] { PT->fft_y(F0, W - F0, nm_in, twf, -1, c->tune.tile_y, INT_MAX, 0, s); }));
+  transforms += nm_in;
   if (c->p.interlaced) {
     TRY(run(c, PSPEC_K_FFT_X, acc(2 * Sc), [&] { PT->fft_x(F0, F0, twf, -1, 0, s); }));
-    TRY(run(c, PSPEC_K_FFT_Z, acc(Sr + Sc), [&] { PT->r2c_z(m2, W, twh, twr, s); }));
-    TRY(run(c, PSPEC_K_FFT_Y, acc(2 * Sc), [&] { PT->fft_y(W, 0, 1, twf, -1, c->tune.tile_y, INT_MAX, 0, s); }));
-    transforms++;
     TRY(run(c, PSPEC_K_COMBINE, acc(3 * Sc), [&] {
       PT->combine_x(W, F0, twf, 1, c->p.compensate, pl.roundtrip, phase, invw, ba, ctas_comb, s);
     }));
