@@ -83,10 +83,11 @@ template <int N> struct Lay {
 // kz columns per block of the y and x passes: the storage tile's, but at most 256 threads in FP64, whose
 // fixed-point stages take 72 registers a thread and more: three blocks of 256 threads share an SM where
 // one of 512 would run alone, and each covers the others' barriers (512^3, per spectrum: y pass
-// 1.08 -> 0.72 ms).
+// 1.08 -> 0.72 ms). N * TW <= 4096 keeps two FP64 tiles (binning pass) plus the bins within shared
+// memory: a 768^3 storage tile of 8 columns is worked on by two neighbouring blocks.
 template <typename T, int N> constexpr int col_block_tile() {
   int tw = Shape<N>::TW;
-  while (sizeof(T) == 8 && tw > 1 && tw * Shape<N>::Tc > 256) tw /= 2;
+  while (tw > 1 && ((sizeof(T) == 8 && tw * Shape<N>::Tc > 256) || N * tw > 4096)) tw /= 2;
   return tw;
 }
 
@@ -696,13 +697,13 @@ __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E
       const int a = harm_a(h), sg = harm_sign(h);
       const C* Gs = G + (int64_t)s * spec_stride;
       // FP32 with a table: Y_lm(khat) of this harmonic, one contiguous block per x tile
-      const float* Ys = YT ? ytab + (int64_t)s * modes + Lay<N>::table_tile(kt, j) + c : nullptr;
+      const float* Ys = YT ? ytab + (int64_t)s * modes + Lay<N>::table_tile(kt, j) + (q % SUB) * TW + c : nullptr;
       C v[E];
       float yv[YT ? E : 1];  // table values, loaded with the spectrum so that the FFT hides their latency
 #pragma unroll
       for (int e = 0; e < E; e++) {
         v[e] = Gs[off + (t + Tc * e) * si];
-        if constexpr (YT && !kLateY) yv[e] = __ldg(Ys + (t + Tc * e) * TW);
+        if constexpr (YT && !kLateY) yv[e] = __ldg(Ys + (t + Tc * e) * Lay<N>::TW);
       }
       if constexpr (YT && kLateY) {
         // the next stage of copies: this tile's next harmonic, or the next tile's F0 and first harmonic
@@ -713,7 +714,7 @@ __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E
           const C* Gn = G + (s + 1 < M ? (int64_t)(s + 1) * spec_stride : 0) + at;
           const float* Yn = ytab + (s + 1 < M ? (int64_t)(s + 1) * modes : 0) + Lay<N>::table_tile(nkt, nj);
           for (int i = threadIdx.x; i < N; i += TW * Tc) prefetch_l2(Gn + i * si);
-          for (int i = threadIdx.x; i < N * TW / 32; i += TW * Tc) prefetch_l2(Yn + i * 32);
+          for (int i = threadIdx.x; i < N * Lay<N>::TW / 32; i += TW * Tc) prefetch_l2(Yn + i * 32);
           if (s + 1 == M)
             for (int i = threadIdx.x; i < N; i += TW * Tc) prefetch_l2(F0 + at + i * si);
         }
@@ -721,7 +722,7 @@ __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E
       fft_any<XP, C, E, N, kInterleaved, TW, -1>(v, sm, t, c, twf);
       if constexpr (YT && kLateY) {
 #pragma unroll
-        for (int e = 0; e < E; e++) yv[e] = __ldg(Ys + (t + Tc * e) * TW);
+        for (int e = 0; e < E; e++) yv[e] = __ldg(Ys + (t + Tc * e) * Lay<N>::TW);
       }
 #pragma unroll
       for (int e = 0; e < E; e++) {
@@ -1044,6 +1045,7 @@ template <typename T, int N> struct Passes {
   static size_t smem_bin_fx(int nk) { return smem_col() + (2 * N + kPolyMaxCoef * TWB) * sizeof(double) + smem_bins(nk); }
   // pipelined FP32 pass: two G tiles and two Y tiles (float), then the bins
   static size_t smem_bin_pipe(int nk) {
+    if (S::E != 8) return 0;  // not used
     return 2 * (size_t)N * S::TW * (sizeof(float2) + sizeof(float)) + (size_t)nk * sizeof(double) +
            (size_t)((S::CT + 31) / 32) * nk * sizeof(float);
   }

@@ -789,16 +789,21 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
       const int M = std::min(pl.group_max, hhi - h0);
       // z pass with the Y_lm weights: one block holds Ms harmonics x rows rows, tz threads each
       const int tz = pl.xp ? PT->tz_xp : PT->tz;
-      const int cap = ylm_thread_cap(ell);
-      const int ms_max = std::max(1, std::min(c->tune.ylm_harmonics, cap / tz));
+      // With the table a block's rows are independent of each other: eight harmonics at most a launch leave
+      // blocks of close to 512 threads (of 24 elements: 16 warps an SM where the 33 harmonics of l = 16 in one
+      // block of 264 left 9). 384^3 l <= 16: 31.8 -> 28.1 ms a set, 512^3 plain l <= 4: 3.19 -> 3.06 ms.
+      const bool tab = pl.has_rtab && ell > 0 && !(ell & 1);
+      const int cap = ylm_thread_cap(tab && N % 3 == 0 ? 0 : ell);
+      const int ms_max = std::max(1, std::min({c->tune.ylm_harmonics, cap / tz, tab ? 8 : INT_MAX}));
       const double* rpoly = f64 && ell <= kPolyLmax ? c->at<PolyTab>(pl.o_poly)->rz + poly_base(ell) : nullptr;
-      for (int hs = 0; hs < M; hs += ms_max) {
-        const int Ms = std::min(ms_max, M - hs);
-        int rows = std::max(1, pow2_floor(std::max(1, cap / (Ms * tz))));
-        while (rows > 1 && (((int64_t)N * N) % rows || PT->smem_ylm(Ms, rows) > kSmemBudget)) rows >>= 1;
+      const int nlaunch = (M + ms_max - 1) / ms_max, ms = (M + nlaunch - 1) / nlaunch;  // of nearly equal size
+      for (int hs = 0; hs < M; hs += ms) {
+        const int Ms = std::min(ms, M - hs);
+        // the most rows that fit (any divisor of N^2: 6 and 12 on radix-3 meshes)
+        int rows = std::max(1, cap / (Ms * tz));
+        while (rows > 1 && (((int64_t)N * N) % rows || PT->smem_ylm(Ms, rows) > kSmemBudget)) rows--;
         // even l of the SH route read their weights from the Y_lm(rhat) table when the plan holds it
-        const float* rt = pl.has_rtab && ell > 0 && !(ell & 1)
-                              ? c->at<float>(pl.o_rtab) + (int64_t)(ytab_base(ell) + h0 + hs) * N * N * N
+        const float* rt = tab ? c->at<float>(pl.o_rtab) + (int64_t)(ytab_base(ell) + h0 + hs) * N * N * N
                               : nullptr;
         TRY(run(c, PSPEC_K_YLM_Z, acc(Sr + Ms * Sc + (rt ? Ms * (double)N * N * N * sizeof(float) : 0.0)), [&] {
           PT->ylm_z(f, G + hs * stride, stride, ell, h0 + hs, Ms, twh_x, twr_x, axis, rows, rt, rpoly, pl.xp, s);
