@@ -123,6 +123,28 @@ __device__ __forceinline__ double2 fx_out(lc v, int c2, bool bad) {
   return make_double2(fx_to_double(v.x, c2), fx_to_double(v.y, c2));
 }
 
+// The same by two FP64 additions in place of some 25 integer instructions: hi and lo words pasted into the
+// mantissas of 2^84 and 2^52 (times 2^-S), their offsets taken off, one rounding (ties to even). The
+// integer pipe bounds the column passes (64% busy) while the FP64 pipe idles, so they convert the real
+// parts this way and the imaginary parts in integers.
+struct FxPaste {
+  int hi, lo;     // upper words of 2^(84-S), 2^(52-S)
+  double off;     // (2^84 + 2^63 + 2^52) 2^-S
+};
+__device__ __forceinline__ FxPaste fx_paste(int S) {
+  FxPaste p;
+  p.hi = (1023 + 84 - S) << 20;
+  p.lo = (1023 + 52 - S) << 20;
+  p.off = __hiloint2double(((1023 + 84 - S) << 20), 0) + __hiloint2double((1023 + 63 - S) << 20, 0) +
+          __hiloint2double((1023 + 52 - S) << 20, 0);
+  return p;
+}
+__device__ __forceinline__ bool fx_paste_ok(int S) { return S > -800 && S < 900; }
+__device__ __forceinline__ double fx_pasted(long long q, const FxPaste& p) {
+  const int hi = (int)(q >> 32) ^ 0x80000000, lo = (int)q;
+  return (__hiloint2double(p.hi, hi) - p.off) + __hiloint2double(p.lo, lo);
+}
+
 // The scale of the sequence of E values per thread, with 2^extra of headroom.
 template <int E, int L, int LAYOUT, int NSEQ, bool WARP>
 __device__ __forceinline__ FxScale fx_sequence_scale(const double2 (&v)[E], void* sm, int t, int seq, int extra) {
@@ -135,16 +157,23 @@ __device__ __forceinline__ FxScale fx_sequence_scale(const double2 (&v)[E], void
   return fx_scale(fx_sequence_bound<L / E, LAYOUT, NSEQ, WARP>(b, sm, t, seq), log2_ceil(L), extra);
 }
 
-// fft_ct of FP64 values through fixed point; `tw` holds int4 entries.
-template <int E, int L, int LAYOUT, int NSEQ, int DIR, bool WARP = false>
+// fft_ct of FP64 values through fixed point; `tw` holds int4 entries. PASTE: passes that leave the FP64
+// pipe idle otherwise.
+template <int E, int L, int LAYOUT, int NSEQ, int DIR, bool WARP = false, bool PASTE = false>
 __device__ __forceinline__ void fft_fx(double2 (&v)[E], double2* sm, int t, int seq, const double2* __restrict__ tw) {
   const FxScale sc = fx_sequence_scale<E, L, LAYOUT, NSEQ, WARP>(v, sm, t, seq, 0);
   lc u[E];
 #pragma unroll
   for (int e = 0; e < E; e++) u[e] = fx_in(v[e], 1084 - sc.S);
   fft_ct<lc, E, L, LAYOUT, NSEQ, DIR, WARP>(u, reinterpret_cast<lc*>(sm), t, seq, reinterpret_cast<const int4*>(tw));
+  if (PASTE && fx_paste_ok(sc.S) && !sc.bad) {
+    const FxPaste p = fx_paste(sc.S);
 #pragma unroll
-  for (int e = 0; e < E; e++) v[e] = fx_out(u[e], 1085 - sc.S, sc.bad);
+    for (int e = 0; e < E; e++) v[e] = make_double2(fx_pasted(u[e].x, p), fx_to_double(u[e].y, 1085 - sc.S));
+  } else {
+#pragma unroll
+    for (int e = 0; e < E; e++) v[e] = fx_out(u[e], 1085 - sc.S, sc.bad);
+  }
 }
 
 // A row of 2L reals as L packed pairs -> its L modes: the transform, then

@@ -507,7 +507,10 @@ __global__ void __launch_bounds__(TW * (N / col_elems<T, N, XP>()),
   C v[E];
 #pragma unroll
   for (int e = 0; e < E; e++) v[e] = base[(int64_t)(t + Tc * e) * Lay<N>::YJ];
-  fft_any<XP, C, E, N, kInterleaved, TW, DIR>(v, sm, t, c, twf);
+  if constexpr (sizeof(T) == 8)
+    fft_fx<E, N, kInterleaved, TW, DIR, false, true>(v, sm, t, c, twf);
+  else
+    fft_any<XP, C, E, N, kInterleaved, TW, DIR>(v, sm, t, c, twf);
 #pragma unroll
   for (int e = 0; e < E; e++) {
     const int ny = sfreq<N>(t + Tc * e);
@@ -532,7 +535,10 @@ __global__ void __launch_bounds__(col_block_tile<T, N>() * (N / col_elems<T, N, 
   C v[E];
 #pragma unroll
   for (int e = 0; e < E; e++) v[e] = in[off + (t + Tc * e) * si];
-  fft_any<XP, C, E, N, kInterleaved, TW, DIR>(v, sm, t, c, twf);
+  if constexpr (sizeof(T) == 8)
+    fft_fx<E, N, kInterleaved, TW, DIR, false, true>(v, sm, t, c, twf);
+  else
+    fft_any<XP, C, E, N, kInterleaved, TW, DIR>(v, sm, t, c, twf);
 #pragma unroll
   for (int e = 0; e < E; e++) out[off + (t + Tc * e) * si] = v[e];
 }
