@@ -66,7 +66,8 @@ enum { PSPEC_WINDOW_CIC = 2, PSPEC_WINDOW_TSC = 3 };   /* value = order p of sin
  * remainder) and round once per shared-memory exchange and pass, which keeps the multipoles
  * within 1e-5 (l <= 4) / 1e-4 (l <= 16) of an FP64 evaluation at 512^3.
  * PSPEC_FP32_PLAIN: every transform a plain FP32 radix tree (faster; rounds at every add level).
- * PSPEC_FP64: FP64 throughout. */
+ * PSPEC_FP64: FP64 meshes, sums and bins; each row or column of a transform runs in 62-bit fixed point
+ * on a scale of its own (more accurate than an FP64 radix tree) and is rounded to FP64 once per pass. */
 enum { PSPEC_FP32 = 0, PSPEC_FP64 = 1, PSPEC_FP32_PLAIN = 2 };
 enum { PSPEC_POS_F64 = 0, PSPEC_POS_F32 = 1 };
 #define PSPEC_MAX_ELL 16
