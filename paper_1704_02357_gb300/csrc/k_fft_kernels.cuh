@@ -247,6 +247,34 @@ template <typename T, int N, bool XP> __host__ __device__ constexpr size_t ylm_s
 // coefficients of the powers of z of each r^l Y_lm, then per node l/2 multiply-adds a harmonic at most and
 // one product with f / r^l (times z for odd powers). All threads of the block. 25 FP64 operations a
 // node for the nine harmonics of l = 4, 16 for l = 2, where the recurrence took about 90 and 55.
+// The axis table of FP64 contexts is in units of a power of two above its largest entry (upload_tables):
+// Y_lm has no scale, and r^l and its inverse stay within FP64's range whatever the box's unit. What is left is a node
+// that nearly coincides with the observer, r below 2^-85 of the largest distance: node_near_observer takes
+// its coordinates to a scale of their own (once in a mesh at most, so a call of its own).
+constexpr double kNearR2 = 0x1p-170;
+static __device__ __noinline__ void node_near_observer(double x, double y, double z, double f, const double* __restrict__ poly,
+                                                       int ell, int h0, int M, double* st, int stride) {
+  const double m = fmax(fabs(x), fmax(fabs(y), fabs(z)));
+  const int e = m > 0.0 ? -ilogb(m) : 0;  // the node at the observer: 0, below
+  x = scalbn(x, e);
+  y = scalbn(y, e);
+  z = scalbn(z, e);
+  const double inv = m > 0.0 ? rsqrt_t<double>(x * x + y * y + z * z) : 0.0;
+  const int NP = poly_np(ell), NI = ell + 1;
+  for (int s = 0; s < M; s++) {
+    const int par = poly_par_z(ell, h0 + s);
+    double v = 0.0;
+    for (int k = 0; par + 2 * k <= ell; k++) {
+      const int n = ell - par - 2 * k;  // degree in x and y
+      const double* c = poly + ((h0 + s) * NP + k) * NI;
+      double a = 0.0;
+      for (int i = 0; i <= n; i++) a += c[i] * ipow(x, i) * ipow(y, n - i);
+      v += a * ipow(z, par + 2 * k);
+    }
+    st[s * stride] = f * (v * ipow(inv, ell));
+  }
+}
+
 template <int N, int LT>
 __device__ __forceinline__ void poly_weights(const double* __restrict__ f, const double* __restrict__ axis,
                                              const double* __restrict__ poly, int ell, int h0, int M, int row0, int rows,
@@ -278,6 +306,10 @@ __device__ __forceinline__ void poly_weights(const double* __restrict__ f, const
     const double* cr = cf + r * M * NP;
     const double z = axis[2 * N + kk], z2 = z * z, r2 = rho2 + z2;
     double g = f[(int64_t)grow * N + kk];
+    if (r2 < kNearR2) {
+      node_near_observer(vx, vy, z, g, poly, ell, h0, M, stage + r * N + kk, rows * N);
+      continue;
+    }
     if (ell & 1) {
       const double inv = rsqrt_newton(r2), inv2 = inv * inv;
       g *= inv;
@@ -286,7 +318,6 @@ __device__ __forceinline__ void poly_weights(const double* __restrict__ f, const
       const double inv2 = rcp_newton(r2);
       for (int p = 0; p < ell; p += 2) g *= inv2;
     }
-    if (r2 == 0.0) g = 0.0;  // the node at the observer
     const double gz = g * z;
     double* st = stage + r * N + kk;
     auto one = [&](int s, int a) {

@@ -407,6 +407,13 @@ pspec_status upload_tables(Ctx* c) {
   const double H = c->p.box_size / N;
   for (int d = 0; d < 3; d++)
     for (int i = 0; i < N; i++) axis[d * N + i] = T(c->p.box_corner[d] + i * H - c->p.observer[d]);
+  if (sizeof(T) == 8) {
+    // in units of a power of two, exact, for the powers of the polynomials' weights (poly_weights)
+    double m = 0.0;
+    for (const T a : axis) m = std::max(m, std::fabs((double)a));
+    const int e = m > 0.0 ? std::ilogb(m) + 1 : 0;
+    for (T& a : axis) a = (T)std::scalbn((double)a, -e);
+  }
   const int p = c->p.window;  // order of sinc^p
   // compensation divisor per axis: sinc^p(pi n/N), or (compensate = 2) the square root of its
   // alias sum sum_m sinc^{2p}(pi (n/N + m)) in closed form (Jing 2005): 1 - 2/3 s^2 (CIC),
