@@ -40,7 +40,7 @@ struct PaintArgs {
   int64_t count;
   double corner[3];
   double inv_cell;      // N / L
-  int safe_log2;        // positions below 2^safe_log2 in magnitude are valid (paint_safe_log2); -1000: test each
+  int safe_log2;        // positions below 2^safe_log2 in magnitude are valid (paint_safe_log2); kNoSafeLog2: test each
   double P0;
   double nbar_default;
   double wf_default;    // FKP weight for nbar_default
@@ -49,15 +49,18 @@ struct PaintArgs {
 };
 
 // The largest k for which |x| < 2^k implies a valid particle (grid coordinate below 2^62 in units of 2^-24
-// cell) on every axis, with a factor two of margin; -1000 when the corner itself is too far out.
+// cell) on every axis, with a factor two of margin; kNoSafeLog2, below every exponent, when the corner is too
+// far out or not a number: each position is then tested.
+constexpr int kNoSafeLog2 = -5000;
 inline int paint_safe_log2(const double* corner, double inv_cell) {
   double c = 0.0;
   for (int d = 0; d < 3; d++) {
     const double a = corner[d] < 0 ? -corner[d] : corner[d];
+    if (!(a >= 0.0)) return kNoSafeLog2;
     c = a > c ? a : c;
   }
   const double reach = 137438953472.0 / inv_cell - c;  // 2^37 cells from the corner
-  int k = -1000;
+  int k = kNoSafeLog2;
   if (reach > 0.0)
     for (k = -900; k < 900 && __builtin_ldexp(1.0, k + 1) <= reach; k++) {
     }
