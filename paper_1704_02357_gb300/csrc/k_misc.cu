@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(kSumThreads) k_catalog_partials(PaintArgs a_in
   const bool uniform = (a.weight == nullptr) && (a.nbar == nullptr);
   const int lim32 = a.safe_log2 > 126 ? 253 : a.safe_log2 + 127, lim64 = a.safe_log2 + 1023;
   double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+  const bool nb_ok = finite_bits(a.nbar_default);  // a default n̄ that is not a number leaves every particle out
   int n = 0;
   auto valid = [&](int64_t p) {
     if (a.pos_f32) {
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(kSumThreads) k_catalog_partials(PaintArgs a_in
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.count;
        p += (int64_t)gridDim.x * blockDim.x) {
     if (uniform) {
-      n += valid(p) ? 1 : 0;
+      n += nb_ok && valid(p) ? 1 : 0;
       continue;
     }
     const double wc = a.weight ? a.weight[p] : 1.0;
@@ -167,9 +168,9 @@ __global__ void __launch_bounds__(kSumThreads) k_catalog_partials(PaintArgs a_in
       const double wf = a.wf_default;
       double* o = out + (int64_t)blockIdx.x * kSumVals;
       o[0] = m;
-      o[1] = m * (wf * wf);
-      o[2] = m * (a.nbar_default * wf * wf);
-      o[3] = m * fabs(wf);
+      o[1] = nb_ok ? m * (wf * wf) : 0.0;
+      o[2] = nb_ok ? m * (a.nbar_default * wf * wf) : 0.0;
+      o[3] = nb_ok ? m * fabs(wf) : 0.0;
     }
     return;
   }

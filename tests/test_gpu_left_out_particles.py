@@ -47,3 +47,8 @@ def test_far_corner(pos, weights):
 def test_corner_that_is_not_a_number(corner, weights):
     import torch
     assert _sums(corner, torch.float64, weights=weights) == (0.0, 0.0)
+
+
+def test_default_density_that_is_not_a_number():
+    import torch
+    assert _sums((500.0, 400.0, 300.0), torch.float64, nbar=float("nan")) == (0.0, 0.0)
