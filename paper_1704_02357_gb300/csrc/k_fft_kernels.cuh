@@ -1064,10 +1064,6 @@ __global__ void __launch_bounds__(Shape<N>::CT, min_blocks<float, Shape<N>::E>(S
 }
 
 // ------------------------------------------------------------------ launchers of one size
-template <typename K> static void set_smem(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <typename T, int N> struct Passes {
   using C = cx<T>;
   using U = ux<T>;
@@ -1091,14 +1087,14 @@ template <typename T, int N> struct Passes {
                     cudaStream_t s) {
     using Z = ZRow<T, N, false>;
     const size_t smem = (size_t)Z::ROWS * row_bytes<T, N, false>();
-    set_smem(k_r2c_z<T, N>, smem);
+    allow_smem(k_r2c_z<T, N>, smem);
     k_r2c_z<T, N><<<dim3(N * N / Z::ROWS, nmesh), Z::ZT, smem, s>>>(in, out, in_stride, out_stride, twh, twr);
   }
   // Launchers taking `xp` run the exact-add variant of their kernel when it is set (FP32 only).
   template <bool XP> static void c2r_z_v(const C* in, T* out, const U* twh, const U* twr, T scale, cudaStream_t s) {
     using Z = ZRow<T, N, XP>;
     const size_t smem = (size_t)Z::ROWS * row_bytes<T, N, XP>();
-    set_smem(k_c2r_z<T, N, XP>, smem);
+    allow_smem(k_c2r_z<T, N, XP>, smem);
     k_c2r_z<T, N, XP><<<N * N / Z::ROWS, Z::ZT, smem, s>>>(in, out, twh, twr, scale);
   }
   static void c2r_z(const C* in, T* out, const U* twh, const U* twr, T scale, int xp, cudaStream_t s) {
@@ -1118,7 +1114,7 @@ template <typename T, int N> struct Passes {
                       const T* axis, int rows, const float* rtab, const double* poly, cudaStream_t s) {
     const size_t smem = smem_ylm(M, rows);
     const dim3 grid(N * N / rows), block(M * rows * ZRow<T, N, XP>::Tz);
-    set_smem(k_ylm_r2c_z<T, N, LT, XP>, smem);
+    allow_smem(k_ylm_r2c_z<T, N, LT, XP>, smem);
     k_ylm_r2c_z<T, N, LT, XP><<<grid, block, smem, s>>>(f, out, stride, ell, h0, M, twh, twr, axis, rows, rtab,
                                                          poly, host_ytab<T>());
   }
@@ -1153,10 +1149,10 @@ template <typename T, int N> struct Passes {
     const int threads = TWV * (N / col_elems<T, N, XP>());
     dim3 grid(N * (S::NH / TWV), nspec);
     if (dir < 0) {
-      set_smem(k_fft_y<T, N, -1, TWV, XP>, smem);
+      allow_smem(k_fft_y<T, N, -1, TWV, XP>, smem);
       k_fft_y<T, N, -1, TWV, XP><<<grid, threads, smem, s>>>(data, stride, twf, n2_cut);
     } else {
-      set_smem(k_fft_y<T, N, 1, TWV, XP>, smem);
+      allow_smem(k_fft_y<T, N, 1, TWV, XP>, smem);
       k_fft_y<T, N, 1, TWV, XP><<<grid, threads, smem, s>>>(data, stride, twf, n2_cut);
     }
   }
@@ -1181,10 +1177,10 @@ template <typename T, int N> struct Passes {
     const unsigned grid = N * (S::NH / TWB);
     const int threads = TWB * (N / col_elems<T, N, XP>());
     if (dir < 0) {
-      set_smem(k_fft_x<T, N, -1, XP>, smem);
+      allow_smem(k_fft_x<T, N, -1, XP>, smem);
       k_fft_x<T, N, -1, XP><<<grid, threads, smem, s>>>(in, out, twf);
     } else {
-      set_smem(k_fft_x<T, N, 1, XP>, smem);
+      allow_smem(k_fft_x<T, N, 1, XP>, smem);
       k_fft_x<T, N, 1, XP><<<grid, threads, smem, s>>>(in, out, twf);
     }
   }
@@ -1197,14 +1193,14 @@ template <typename T, int N> struct Passes {
   static void combine_x(const C* B, C* F0, const U* twf, int interlaced, int compensate, int roundtrip,
                         const U* phase, const C* invw, const BinArgs& ba, int ctas, cudaStream_t s) {
     const size_t smem = smem_combine(ba.nk);
-    set_smem(k_combine_x<T, N>, smem);
+    allow_smem(k_combine_x<T, N>, smem);
     k_combine_x<T, N><<<ctas, col_threads<T, N>(), smem, s>>>(B, F0, twf, interlaced, compensate, roundtrip, phase, invw, ba);
   }
   template <int LT>
   static void bin_fx_v(const C* G, int64_t stride, int ell, int h0, int M, const C* F0, const U* twf, int slot,
                        const BinArgs& ba, int ctas, const KPoly& kp, cudaStream_t s) {
     const size_t smem = smem_bin_fx(ba.nk);
-    set_smem(k_bin_fx<N, LT>, smem);
+    allow_smem(k_bin_fx<N, LT>, smem);
     // a mesh with fewer tiles than four blocks per SM splits the harmonics over blocks (64^3, l = 4: 64 us
     // with 128 blocks)
     const int tiles = ba.n_xtiles * (Lay<N>::TW / TWB);
@@ -1219,16 +1215,16 @@ template <typename T, int N> struct Passes {
     if constexpr (sizeof(T) == 4 && S::E == 8) {
       if (ytab) {
         const size_t sp = smem_bin_pipe(ba.nk);
-        set_smem(k_bin_x_pipe<N, XP>, sp);
+        allow_smem(k_bin_x_pipe<N, XP>, sp);
         k_bin_x_pipe<N, XP><<<ctas, S::CT, sp, s>>>(G, stride, ell, h0, M, F0, twf, slot, ba, ytab);
         return;
       }
     }
     if (ytab && sizeof(T) == 4) {
-      set_smem(k_bin_x<T, N, true, XP>, smem);
+      allow_smem(k_bin_x<T, N, true, XP>, smem);
       k_bin_x<T, N, true, XP><<<ctas, col_threads<T, N>(), smem, s>>>(G, stride, ell, h0, M, F0, twf, slot, ba, ytab, host_ytab<T>());
     } else {
-      set_smem(k_bin_x<T, N, false, XP>, smem);
+      allow_smem(k_bin_x<T, N, false, XP>, smem);
       k_bin_x<T, N, false, XP><<<ctas, col_threads<T, N>(), smem, s>>>(G, stride, ell, h0, M, F0, twf, slot, ba, ytab, host_ytab<T>());
     }
   }
@@ -1255,27 +1251,27 @@ template <typename T, int N> struct Passes {
     int per = 0;
     if (which == 0) {
       const size_t smem = smem_combine(nk);
-      set_smem(k_combine_x<T, N>, smem);
+      allow_smem(k_combine_x<T, N>, smem);
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_combine_x<T, N>, col_threads<T, N>(), smem);
     } else if (which == 2 && sizeof(T) == 4 && S::E == 8) {
       if constexpr (sizeof(T) == 4 && S::E == 8) {
         const size_t smem = smem_bin_pipe(nk);
-        set_smem(k_bin_x_pipe<N, XP>, smem);
+        allow_smem(k_bin_x_pipe<N, XP>, smem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_x_pipe<N, XP>, S::CT, smem);
       }
     } else if (which == 3) {
       if constexpr (sizeof(T) == 8) {
         const size_t smem = smem_bin_fx(nk);
-        set_smem(k_bin_fx<N, 4>, smem);
+        allow_smem(k_bin_fx<N, 4>, smem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_fx<N, 4>, col_threads<T, N>(), smem);
       }
     } else if (which == 2) {
       const size_t smem = smem_bin(nk);
-      set_smem(k_bin_x<T, N, true, XP>, smem);
+      allow_smem(k_bin_x<T, N, true, XP>, smem);
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_x<T, N, true, XP>, col_threads<T, N>(), smem);
     } else {
       const size_t smem = smem_bin(nk);
-      set_smem(k_bin_x<T, N, false, XP>, smem);
+      allow_smem(k_bin_x<T, N, false, XP>, smem);
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_x<T, N, false, XP>, col_threads<T, N>(), smem);
     }
     if (per < 1) per = 1;

@@ -919,10 +919,6 @@ void launch_ptile_scatter(const TileArgs& ta, int64_t total, const DevCat* dc, c
     k_ptile_scatter<<<2 * nb, 256, 0, s>>>(ta, total, dc, cur, N);
 }
 
-template <typename K> static void set_smem_attr(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <int WIN, bool INTER>
 static void ptile_paint_v(const TileArgs& ta, float* m1, float* m2, int N, const double* fix, const float* r1,
                           const float* r2, const double* alpha, cudaStream_t s) {
@@ -930,7 +926,7 @@ static void ptile_paint_v(const TileArgs& ta, float* m1, float* m2, int N, const
   const size_t smem = (size_t)(INTER ? 2 : 1) * kPT3 * sizeof(unsigned long long);
   auto go = [&](auto nt) {
     constexpr int NT = decltype(nt)::value;
-    set_smem_attr(k_ptile_paint<WIN, INTER, NT>, smem);
+    allow_smem(k_ptile_paint<WIN, INTER, NT>, smem);
     k_ptile_paint<WIN, INTER, NT><<<ntiles, NT, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
   };
   if (ntiles <= kFewTiles)

@@ -67,6 +67,15 @@ inline int paint_safe_log2(const double* corner, double inv_cell) {
   return k;
 }
 
+constexpr size_t kSmemMaxBlock = 227 * 1024;  // per-block limit of the device
+// Lets a kernel be launched with `bytes` of dynamic shared memory. The allowance belongs to the kernel on its
+// device, not to a context: set to the bytes of one call, another host thread's smaller call could
+// lower it again before the launch. It is only ever set to the limit (these kernels have no static
+// shared memory); launches and occupancy queries take the bytes they need.
+template <typename K> void allow_smem(K kernel, size_t bytes) {
+  if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMaxBlock);
+}
+
 struct BinArgs {
   const int32_t* bin_of_n2;  // bin index of |n|^2, or -1
   int nk;

@@ -17,7 +17,6 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr size_t kSmemBudget = 200 * 1024;   // one block
-constexpr size_t kSmemMaxBlock = 227 * 1024; // per-block limit of the device
 constexpr int kMaxElls = PSPEC_MAX_ELL / 2 + 1;
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
