@@ -416,23 +416,26 @@ pspec_status upload_tables(Ctx* c) {
   const int p = c->p.window;  // order of sinc^p
   // compensation divisor per axis: sinc^p(pi n/N), or (compensate = 2) the square root of its
   // alias sum sum_m sinc^{2p}(pi (n/N + m)) in closed form (Jing 2005): 1 - 2/3 s^2 (CIC),
-  // 1 - s^2 + 2/15 s^4 (TSC), s = sin(pi n/N)
+  // 1 - s^2 + 2/15 s^4 (TSC), s = sin(pi n/N). FP64 contexts take it in extended precision: its rounding
+  // to FP64, the same for all modes of a plane, put the power off by 2e-16 to 5e-16 of itself.
+  using A = std::conditional_t<sizeof(T) == 8, long double, double>;
+  const A pi = sizeof(T) == 8 ? std::acos(A(-1)) : A(M_PI);
   auto sincp = [&](int n) {
-    const double x = M_PI * n / N;
+    const A x = pi * n / N;
     if (c->p.compensate == 2) {
-      const double s2 = std::sin(x) * std::sin(x);
-      return std::sqrt(p == PSPEC_WINDOW_CIC ? 1.0 - 2.0 / 3.0 * s2 : 1.0 - s2 + 2.0 / 15.0 * s2 * s2);
+      const A s2 = std::sin(x) * std::sin(x);
+      return std::sqrt(p == PSPEC_WINDOW_CIC ? A(1) - A(2) / A(3) * s2 : A(1) - s2 + A(2) / A(15) * s2 * s2);
     }
-    if (n == 0) return 1.0;
-    return std::pow(std::sin(x) / x, p);
+    if (n == 0) return A(1);
+    return std::pow(std::sin(x) / x, A(p));
   };
   // exp(-i pi s / N), s = nx + ny + nz in [-3N/2, 3N/2): the H/2 shift of the second mesh
   for (int i = 0; i < 3 * N; i++) phase[i] = unit_factor<T>(-M_PI * (i - 3 * N / 2) / N);
   for (int i = 0; i < N + NH; i++) {
     const int n = i < N ? (i < NH ? i : i - N) : (i - N);
-    const double w = 1.0 / sincp(n);
+    const A w = A(1) / sincp(n);
     const T hi = T(w);
-    invw[i] = mk(hi, T(w / (double)hi - 1.0));
+    invw[i] = mk(hi, T(w / A(hi) - A(1)));
   }
   cudaError_t e;
   e = cudaMemcpyAsync(c->at<U>(pl.o_twh), twh.data(), twh.size() * sizeof(U), cudaMemcpyHostToDevice, c->stream);
