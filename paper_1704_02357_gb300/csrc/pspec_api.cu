@@ -18,6 +18,7 @@ namespace {
 constexpr size_t kAlign = 256;
 constexpr size_t kSmemBudget = 200 * 1024;   // one block
 constexpr int kMaxElls = PSPEC_MAX_ELL / 2 + 1;
+constexpr int kYlmHarmonicsAuto = 64;  // tuning value (the default) from which the z pass chooses itself
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -255,7 +256,7 @@ struct Ctx {
   std::vector<DevCat> desc_host;
   BatchOut bout_host{};  // this batch's output buffers, uploaded to o_bout
   pspec_catalog batch_proto{};  // dtype of the mocks' positions (pointers come from the table)
-  pspec_tuning tune{1, 64, 0, 0};
+  pspec_tuning tune{1, kYlmHarmonicsAuto, 0, 0};
   std::string err;
   int64_t launches = 0;
   int64_t transforms_last = 0;
@@ -803,7 +804,8 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
       // block of 264 left 9). 384^3 l <= 16: 31.8 -> 28.1 ms a set, 512^3 plain l <= 4: 3.19 -> 3.06 ms.
       const bool tab = pl.has_rtab && ell > 0 && !(ell & 1);
       const int cap = ylm_thread_cap(tab && N % 3 == 0 ? 0 : ell);
-      const int ms_max = std::max(1, std::min({c->tune.ylm_harmonics, cap / tz, tab ? 8 : INT_MAX}));
+      const int most = c->tune.ylm_harmonics < kYlmHarmonicsAuto ? c->tune.ylm_harmonics : (tab ? 8 : INT_MAX);
+      const int ms_max = std::max(1, std::min(most, cap / tz));
       const double* rpoly = f64 && ell <= kPolyLmax ? c->at<PolyTab>(pl.o_poly)->rz + poly_base(ell) : nullptr;
       const int nlaunch = (M + ms_max - 1) / ms_max, ms = (M + nlaunch - 1) / nlaunch;  // of nearly equal size
       for (int hs = 0; hs < M; hs += ms) {

@@ -1,9 +1,10 @@
-"""Contexts next to each other."""
+"""Contexts next to each other, and the knobs of one context."""
 import threading
 
 import numpy as np
 import pytest
 
+import synth
 from oracle import estimator as E
 from tests._parity import gpu_estimator
 
@@ -47,3 +48,26 @@ def test_contexts_of_two_threads_with_other_bins():
     for t in threads:
         t.join()
     assert res == {512: "ok", 64: "ok"}
+
+
+@pytest.mark.parametrize("ylm_table", [True, False])
+@pytest.mark.parametrize("knob", [1, 3, 9, 16, 17])
+def test_ylm_harmonics_is_the_most_a_block_takes(knob, ylm_table):
+    """17 harmonics of l = 8 in ceil(17 / knob) launches of the Y-weighted z pass."""
+    L, corner = 900.0, (300.0, 350.0, 320.0)
+    d, r = synth.uniform_box(3000, L, corner, 7), synth.uniform_box(9000, L, corner, 8)
+    p = E.Params(nmesh=32, box_size=L, box_corner=corner, window="cic", interlaced=False, compensate=True, P0=1e4,
+                 nbar=3000 / L ** 3)
+    est = gpu_estimator(p, precision="fp32_plain", ell_max=8, ylm_table=ylm_table, max_particles=12000)
+    assert est.tuning()["ylm_harmonics"] == 64
+    edges = np.linspace(0.0, np.pi * 32 / L, 7)
+    est.paint(d.pos, r.pos)
+    want = est.multipoles([0, 8], edges)
+    est.set_tuning(ylm_harmonics=knob)
+    est.set_profiling(True)
+    est.kernel_times()
+    got = est.multipoles([0, 8], edges)
+    launches = est.kernel_times()["ylm_r2c_z"]["launches"]
+    assert launches == -(-17 // knob)
+    np.testing.assert_allclose(got["P"], want["P"], rtol=0, atol=1e-9 * np.abs(want["P"]).max())
+    est.close()
