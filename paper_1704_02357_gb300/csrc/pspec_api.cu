@@ -19,6 +19,7 @@ constexpr size_t kAlign = 256;
 constexpr size_t kSmemBudget = 200 * 1024;   // one block
 constexpr int kMaxElls = PSPEC_MAX_ELL / 2 + 1;
 constexpr int kYlmHarmonicsAuto = 64;  // tuning value (the default) from which the z pass chooses itself
+constexpr int kYlmGroupsMesh = 384;   // ... groups of eight harmonics with the table (do_multipoles)
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -799,12 +800,16 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
       const int M = std::min(pl.group_max, hhi - h0);
       // z pass with the Y_lm weights: one block holds Ms harmonics x rows rows, tz threads each
       const int tz = pl.xp ? PT->tz_xp : PT->tz;
-      // With the table a block's rows are independent of each other: eight harmonics at most a launch leave
-      // blocks of close to 512 threads (of 24 elements: 16 warps an SM where the 33 harmonics of l = 16 in one
-      // block of 264 left 9). 384^3 l <= 16: 31.8 -> 28.1 ms a set, 512^3 plain l <= 4: 3.19 -> 3.06 ms.
+      // With the table a block's rows are independent of each other. Large meshes take eight harmonics at most a
+      // launch: blocks of close to 512 threads (of 24 elements: 16 warps an SM where the 33 harmonics of l = 16
+      // in one block of 264 left 9). z pass of a set, all that fit -> eight: 384^3 l <= 16 31.6 -> 28.3 ms (plain 21.1 ->
+      // 20.4), 512^3 l <= 4 4.83 -> 4.79 (plain 3.18 -> 3.03), 768^3 l <= 4 23.8 -> 22.4 ms (plain 17.0 -> 17.1). Smaller ones
+      // take all that fit, f and the launches are what counts: 32^3 l <= 16 74 against 232 us, 128^3 768 against
+      // 872 us, 192^3 4.20 against 4.19 ms (plain 3.17 against 3.29), 256^3 6.37 against 6.31 (plain 4.73 against 4.99).
       const bool tab = pl.has_rtab && ell > 0 && !(ell & 1);
       const int cap = ylm_thread_cap(tab && N % 3 == 0 ? 0 : ell);
-      const int most = c->tune.ylm_harmonics < kYlmHarmonicsAuto ? c->tune.ylm_harmonics : (tab ? 8 : INT_MAX);
+      const int most = c->tune.ylm_harmonics < kYlmHarmonicsAuto ? c->tune.ylm_harmonics
+                                                                 : (tab && N >= kYlmGroupsMesh ? 8 : INT_MAX);
       const int ms_max = std::max(1, std::min(most, cap / tz));
       const double* rpoly = f64 && ell <= kPolyLmax ? c->at<PolyTab>(pl.o_poly)->rz + poly_base(ell) : nullptr;
       const int nlaunch = (M + ms_max - 1) / ms_max, ms = (M + nlaunch - 1) / nlaunch;  // of nearly equal size

@@ -71,3 +71,18 @@ def test_ylm_harmonics_is_the_most_a_block_takes(knob, ylm_table):
     assert launches == -(-17 // knob)
     np.testing.assert_allclose(got["P"], want["P"], rtol=0, atol=1e-9 * np.abs(want["P"]).max())
     est.close()
+
+
+@pytest.mark.parametrize("nmesh,table,launches", [(32, True, 1), (32, False, 1), (256, True, 1), (384, True, 3)])
+def test_groups_of_harmonics_by_mesh(nmesh, table, launches):
+    """The default: the 17 harmonics of l = 8 in one launch on small meshes, in groups of eight at most from 384 on."""
+    L, corner = 900.0, (300.0, 350.0, 320.0)
+    d, r = synth.uniform_box(3000, L, corner, 7), synth.uniform_box(9000, L, corner, 8)
+    p = E.Params(nmesh=nmesh, box_size=L, box_corner=corner, window="cic", interlaced=False, compensate=True, P0=1e4,
+                 nbar=3000 / L ** 3)
+    est = gpu_estimator(p, precision="fp32_plain", ell_max=8, ylm_table=table, max_particles=12000)
+    est.paint(d.pos, r.pos)
+    est.set_profiling(True)
+    est.multipoles([0, 8], np.linspace(0.0, np.pi * nmesh / L, 7))
+    assert est.kernel_times()["ylm_r2c_z"]["launches"] == launches
+    est.close()
