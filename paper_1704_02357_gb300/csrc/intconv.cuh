@@ -150,4 +150,24 @@ PSPEC_HD float ll2f_rn_int(long long x) {
   return ic_float(sgn | ((unsigned)(e + 127) << 23) | ((unsigned)r & 0x7fffffu));
 }
 
+// A k for which |x| < 2^k implies a valid particle of the paint (grid coordinate below 2^62 in units of 2^-24
+// cell) on every axis: the largest one that stays within 2^37 cells of the corner, a factor two of margin, and at most
+// 900; kNoSafeLog2, below every exponent, when the corner is too far out or not a number: each position is
+// then tested. Host code, for every paint call: one frexp (a search upwards from 2^-900 took 8 us).
+constexpr int kNoSafeLog2 = -5000;
+inline int paint_safe_log2(const double* corner, double inv_cell) {
+  double c = 0.0;
+  for (int d = 0; d < 3; d++) {
+    const double a = corner[d] < 0 ? -corner[d] : corner[d];
+    if (!(a >= 0.0)) return kNoSafeLog2;
+    c = a > c ? a : c;
+  }
+  const double reach = 137438953472.0 / inv_cell - c;  // 2^37 cells from the corner
+  if (!(reach > 0.0)) return kNoSafeLog2;
+  if (reach >= 0x1p900) return 900;
+  int e;
+  __builtin_frexp(reach, &e);  // 2^(e-1) <= reach < 2^e
+  return e - 1 < -900 ? kNoSafeLog2 : e - 1;
+}
+
 }  // namespace pspec

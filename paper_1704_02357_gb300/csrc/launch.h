@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include "common.cuh"
+#include "intconv.cuh"
 #include "pspec.h"
 
 namespace pspec {
@@ -47,25 +48,6 @@ struct PaintArgs {
   const DevCat* dc;     // when set, pos/weight/nbar/count come from dc[*cur]
   const int* cur;
 };
-
-// The largest k for which |x| < 2^k implies a valid particle (grid coordinate below 2^62 in units of 2^-24
-// cell) on every axis, with a factor two of margin; kNoSafeLog2, below every exponent, when the corner is too
-// far out or not a number: each position is then tested.
-constexpr int kNoSafeLog2 = -5000;
-inline int paint_safe_log2(const double* corner, double inv_cell) {
-  double c = 0.0;
-  for (int d = 0; d < 3; d++) {
-    const double a = corner[d] < 0 ? -corner[d] : corner[d];
-    if (!(a >= 0.0)) return kNoSafeLog2;
-    c = a > c ? a : c;
-  }
-  const double reach = 137438953472.0 / inv_cell - c;  // 2^37 cells from the corner
-  int k = kNoSafeLog2;
-  if (reach > 0.0)
-    for (k = -900; k < 900 && __builtin_ldexp(1.0, k + 1) <= reach; k++) {
-    }
-  return k;
-}
 
 constexpr size_t kSmemMaxBlock = 227 * 1024;  // per-block limit of the device
 // Lets a kernel be launched with `bytes` of dynamic shared memory. The allowance belongs to the kernel on its
