@@ -132,8 +132,9 @@ void launch_ptile_paint(const TileArgs& ta, int window, int interlaced, float* m
 // Tables: tw_half (L = N/2), tw_full (L = N), twr (exp(-2 pi i k/N), k < N/2).
 // Shapes fixed per N at compile time:
 //   col_tile(N): kz columns per storage tile, a power of two dividing N/2 with at most 512
-//                threads (N/E per column) and at most 16 columns, at least 8 up to 768 (rows of 64 bytes
-//                in FP32: with rows of 32 the x passes of a 768^3 mesh ran at half the rate per mode);
+//                threads (N/E per column) and at most 16 columns: 8 where that fits (rows of 64 bytes in
+//                FP32; with rows of 32 the x passes of a 768^3 mesh ran at half the rate per mode), 16 while
+//                N * TW <= 4096. 1024^3 stays at 4, its 128 threads a column leave no more;
 //   z_rows(N):   rows per block of the plain z passes, a power of two dividing N^2 with at
 //                most 512 threads (N/(2E) per row), 128 up to 128^3 so that the blocks of a small
 //                mesh spread over the SMs.
@@ -141,7 +142,7 @@ constexpr int elems_per_thread(int N) { return N % 3 == 0 ? 24 : 8; }
 constexpr int col_tile(int N) {
   const int tc = N / elems_per_thread(N);
   int cap = 512 / tc < 16 ? 512 / tc : 16, tw = 1;
-  while (tw * 2 <= cap && (N / 2) % (tw * 2) == 0 && N * tw * 2 <= (N == 768 ? 8192 : 4096)) tw *= 2;
+  while (tw * 2 <= cap && (N / 2) % (tw * 2) == 0 && (tw * 2 <= 8 || N * tw * 2 <= 4096)) tw *= 2;
   return tw;
 }
 // Elements per thread in the z passes (rows of N/2 complex points): 16 where a row splits into
