@@ -30,7 +30,10 @@
  *     names a status; pspec_last_error() gives the detail of the last failure on a context.
  *   - The caller owns every pointer it passes. Device memory for meshes, spectra and
  *     tables is one caller-provided workspace (size from pspec_workspace_size) that must
- *     stay allocated until pspec_destroy; the library allocates no device memory itself.
+ *     stay allocated until pspec_destroy; the library allocates no device memory itself. The
+ *     CUDA driver keeps memory of its own for launch graphs: one of pspec_run_batch with
+ *     use_graph = 1, and one that pspec_multipoles captures when the same ells, k_edges and
+ *     tuning come a third time in a row (see there). Both are freed by pspec_destroy.
  *   - All device work is enqueued on the stream given to pspec_create, in call order.
  *     Calls on one context are not thread-safe; distinct contexts are independent.
  *   - Host output pointers are written before the call returns (the call synchronises
@@ -163,7 +166,10 @@ pspec_status pspec_paint(void* ctx, const pspec_catalog* data, const pspec_catal
  * Odd l: the shell average of eq. Pell-yama (Sec. 2.1) is purely imaginary for odd l with
  * the end-point line of sight; P holds its imaginary part,
  *   4 pi/(I N_b) sum_b mult sum_m Y_lm(khat) Im[G_lm conj(F0)],
- * with Y_lm(khat) evaluated in the binning kernel (the Y table holds even l only). */
+ * with Y_lm(khat) evaluated in the binning kernel (the Y table holds even l only).
+ * The launches of a call are replayed as a CUDA graph from the third call in a row on with the
+ * same ells, k_edges and tuning; that third call
+ * also captures it. pspec_multipoles_replays counts the replays of a context. */
 pspec_status pspec_multipoles(void* ctx, const int32_t* ells, int32_t n_ells,
                               const double* k_edges, int32_t n_kbins,
                               double* P, double* k_mean, double* n_modes);
@@ -312,6 +318,9 @@ typedef struct {
   int64_t ylm_rtable_bytes;                   /* Y_lm(rhat) table held (0: evaluated per node) */
 } pspec_plan_info;
 pspec_status pspec_get_plan_info(void* ctx, pspec_plan_info* info);
+
+/* Calls of pspec_multipoles that replayed its launch graph so far (for tests and reports). */
+pspec_status pspec_multipoles_replays(void* ctx, int64_t* n);
 
 /* Per-kernel-class timing with CUDA events on the context's stream, for the benchmark.
  * While enabled, each launch is bracketed by events; pspec_kernel_times returns, per

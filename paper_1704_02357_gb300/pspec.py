@@ -79,6 +79,7 @@ SIGNATURES = [
     ("pspec_wedges", C.c_int32, [C.c_void_p, C.POINTER(C.c_int32), C.c_int32, C.c_int32,
                                  C.POINTER(C.c_double), C.c_int32, C.c_void_p, C.c_void_p]),
     ("pspec_get_plan_info", C.c_int32, [C.c_void_p, C.POINTER(PlanInfo)]),
+    ("pspec_multipoles_replays", C.c_int32, [C.c_void_p, C.POINTER(C.c_int64)]),
     ("pspec_set_profiling", C.c_int32, [C.c_void_p, C.c_int32]),
     ("pspec_kernel_times", C.c_int32, [C.c_void_p, C.POINTER(C.c_int64), C.POINTER(C.c_double),
                                        C.POINTER(C.c_double)]),
@@ -364,6 +365,12 @@ class Estimator:
         info = PlanInfo()
         _check(load().pspec_get_plan_info(self._ctx, C.byref(info)), self._ctx)
         return {f: getattr(info, f) for f, _ in PlanInfo._fields_}
+
+    def multipoles_replays(self) -> int:
+        """Calls of multipoles() that replayed its launch graph so far."""
+        n = C.c_int64(0)
+        _check(load().pspec_multipoles_replays(self._ctx, C.byref(n)), self._ctx)
+        return int(n.value)
 
     def set_profiling(self, on: bool):
         _check(load().pspec_set_profiling(self._ctx, int(bool(on))), self._ctx)
