@@ -168,8 +168,8 @@ pspec_status pspec_paint(void* ctx, const pspec_catalog* data, const pspec_catal
  *   4 pi/(I N_b) sum_b mult sum_m Y_lm(khat) Im[G_lm conj(F0)],
  * with Y_lm(khat) evaluated in the binning kernel (the Y table holds even l only).
  * The launches of a call are replayed as a CUDA graph from the third call in a row on with the
- * same ells, k_edges and tuning; that third call
- * also captures it. pspec_multipoles_replays counts the replays of a context. */
+ * same ells, k_edges and tuning (later for callers that change them again before two replays);
+ * that third call also captures it. pspec_multipoles_replays counts the replays of a context. */
 pspec_status pspec_multipoles(void* ctx, const int32_t* ells, int32_t n_ells,
                               const double* k_edges, int32_t n_kbins,
                               double* P, double* k_mean, double* n_modes);

@@ -249,6 +249,7 @@ struct Ctx {
   // launch sequence of pspec_multipoles as a graph, and what it was captured for (multipoles_graph)
   struct MultGraph {
     cudaGraphExec_t exec = nullptr;
+    int64_t launched = 0;  // of exec
     std::vector<int32_t> ells;
     std::vector<double> edges;
     pspec_tuning tune{};
@@ -261,6 +262,7 @@ struct Ctx {
   pspec_catalog batch_proto{};  // dtype of the mocks' positions (pointers come from the table)
   pspec_tuning tune{1, kYlmHarmonicsAuto, 0, 0};
   std::string err;
+  int graph_after = kGraphAfter;  // plain calls of the same arguments before a capture
   int64_t replays = 0;            // pspec_multipoles calls that launched the graph
   int64_t launches = 0;
   int64_t transforms_last = 0;
@@ -976,7 +978,8 @@ pspec_status multipoles_common(Ctx* c, const int32_t* ells, int n_ells, const do
 // takes the host 72 us, about as long as a 32^3 mesh's kernels run. The kernels read everything that
 // changes from one call to the next (meshes, catalog sums) from the workspace. Other arguments, another
 // tuning or profiling take the plain path; a capture that fails leaves it in place. Calls 1 to 5 of a 32^3 box: 174
-// (with the bin tables' upload), 130, 163 (capture), 93, 87 us.
+// (with the bin tables' upload), 130, 163 (capture), 93, 87 us. A caller that changes its arguments before a
+// second replay has repaid the capture is asked for twice as many calls from then on.
 pspec_status multipoles_graph(Ctx* c, const int32_t* ells, int n_ells, const double* k_edges, int nk) {
   double* out = c->at<double>(c->pl.o_out);
   auto plain = [&] { return multipoles_common(c, ells, n_ells, k_edges, nk, out + 2 * (size_t)nk, out, out + nk); };
@@ -987,13 +990,16 @@ pspec_status multipoles_graph(Ctx* c, const int32_t* ells, int n_ells, const dou
                     std::equal(k_edges, k_edges + nk + 1, m.edges.begin()) &&
                     std::memcmp(&m.tune, &c->tune, sizeof m.tune) == 0;
   if (!same) {
-    if (m.exec) cudaGraphExecDestroy(m.exec);
+    if (m.exec) {
+      cudaGraphExecDestroy(m.exec);
+      if (m.launched < 2 && c->graph_after < (1 << 20)) c->graph_after *= 2;
+    }
     m = Ctx::MultGraph();
     m.ells.assign(ells, ells + n_ells);
     m.edges.assign(k_edges, k_edges + nk + 1);
     m.tune = c->tune;
   }
-  if (c->prof || m.seen < kGraphAfter) {
+  if (c->prof || m.seen < c->graph_after) {
     m.seen++;
     return plain();
   }
@@ -1033,6 +1039,7 @@ pspec_status multipoles_graph(Ctx* c, const int32_t* ells, int n_ells, const dou
   }
   e = cudaGraphLaunch(m.exec, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "graph launch");
+  m.launched++;
   c->replays++;
   c->launches += m.kernels;
   c->transforms_last = m.transforms;

@@ -68,3 +68,18 @@ def test_replays_between_other_calls():
     for n in range(4):
         call(n % 2, 9 + max(0, n - 1))
     est.close()
+
+
+def test_arguments_that_change_every_third_call():
+    """A graph that was not replayed a second time is not worth its capture: the next ones wait longer."""
+    est = gpu_estimator(_params(), max_particles=20000)
+    est.paint(_cats(0)[0].pos, _cats(0)[1].pos)
+    for _ in range(3):
+        for edges in (E1, E2):
+            for _ in range(3):
+                est.multipoles([0, 2], edges)
+    assert est.multipoles_replays() == 1
+    for _ in range(8):  # a caller that stays with its arguments gets one again
+        est.multipoles([0, 2], E1)
+    assert est.multipoles_replays() == 1 + 8 - 4
+    est.close()
