@@ -33,12 +33,6 @@ bool good_nmesh(int n) {
   return x == 3 && n >= 48;
 }
 
-int pow2_floor(int v) {
-  int p = 1;
-  while (p * 2 <= v) p *= 2;
-  return p;
-}
-
 struct Plan {
   Geo g;
   int E;
