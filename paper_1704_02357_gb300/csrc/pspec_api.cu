@@ -421,20 +421,23 @@ pspec_status upload_tables(Ctx* c) {
   // to FP64, the same for all modes of a plane, put the power off by 2e-16 to 5e-16 of itself.
   using A = std::conditional_t<sizeof(T) == 8, long double, double>;
   const A pi = sizeof(T) == 8 ? std::acos(A(-1)) : A(M_PI);
-  auto sincp = [&](int n) {
+  std::vector<A> winv(NH + 1);  // 1 / divisor, the same for n and -n
+  for (int n = 0; n <= NH; n++) {
     const A x = pi * n / N;
+    A w = A(1);
     if (c->p.compensate == 2) {
       const A s2 = std::sin(x) * std::sin(x);
-      return std::sqrt(p == PSPEC_WINDOW_CIC ? A(1) - A(2) / A(3) * s2 : A(1) - s2 + A(2) / A(15) * s2 * s2);
+      w = std::sqrt(p == PSPEC_WINDOW_CIC ? A(1) - A(2) / A(3) * s2 : A(1) - s2 + A(2) / A(15) * s2 * s2);
+    } else if (n > 0) {
+      const A v = std::sin(x) / x;
+      w = sizeof(T) == 4 ? std::pow(v, A(p)) : (p == 2 ? v * v : v * v * v);
     }
-    if (n == 0) return A(1);
-    return std::pow(std::sin(x) / x, A(p));
-  };
+    winv[n] = A(1) / w;
+  }
   // exp(-i pi s / N), s = nx + ny + nz in [-3N/2, 3N/2): the H/2 shift of the second mesh
   for (int i = 0; i < 3 * N; i++) phase[i] = unit_factor<T>(-M_PI * (i - 3 * N / 2) / N);
   for (int i = 0; i < N + NH; i++) {
-    const int n = i < N ? (i < NH ? i : i - N) : (i - N);
-    const A w = A(1) / sincp(n);
+    const A w = winv[i < N ? (i < NH ? i : N - i) : i - N];
     const T hi = T(w);
     invw[i] = mk(hi, T(w / A(hi) - A(1)));
   }
