@@ -70,7 +70,11 @@ enum { PSPEC_WINDOW_CIC = 2, PSPEC_WINDOW_TSC = 3 };   /* value = order p of sin
  * within 1e-5 (l <= 4) / 1e-4 (l <= 16) of an FP64 evaluation at 512^3.
  * PSPEC_FP32_PLAIN: every transform a plain FP32 radix tree (faster; rounds at every add level).
  * PSPEC_FP64: FP64 meshes, sums and bins; each row or column of a transform runs in 62-bit fixed point
- * on a scale of its own (more accurate than an FP64 radix tree) and is rounded to FP64 once per pass. */
+ * on a scale of its own and is rounded to FP64 once per pass. (A 512-point transform of noise is off by
+ * 1.0e-16 rms, an FP64 radix tree by 2.1e-16; P at 32^3 for l = 0, 2, 4 by 1.6, 2.0 and 3.0e-16 |P_0|
+ * rms against binary128, with radix trees 2.4, 2.2 and 3.3e-16.) A row or column that holds an infinity, a
+ * NaN or a value of 2^1004 and more becomes NaN, one that is below 2^-895 throughout becomes zero: the
+ * powers of such modes are no FP64 numbers either way. */
 enum { PSPEC_FP32 = 0, PSPEC_FP64 = 1, PSPEC_FP32_PLAIN = 2 };
 enum { PSPEC_POS_F64 = 0, PSPEC_POS_F32 = 1 };
 #define PSPEC_MAX_ELL 16
@@ -134,7 +138,7 @@ typedef struct {
   double alpha, I, S;      /* as defined above */
   double W_d, W_r;         /* sums of completeness weights */
   int64_t n_nonfinite;     /* particles with a non-finite weight or nbar, or a position non-finite or
-                              more than 2^40 cells from the corner (an error) */
+                              more than 2^38 cells from the corner (an error) */
   int64_t n_wrapped;       /* particles outside [corner, corner + L)^3, painted periodically */
 } pspec_stats;
 
