@@ -796,10 +796,21 @@ __device__ __forceinline__ void tile_record(unsigned* acc, const uint4 r, float 
   }
 }
 
-// Threads of a tile's block: three blocks' accumulators (64 KB each with interlacing) fit an SM, and the
-// shared atomics need the warps: 512 threads keep 48 warps resident, 256 kept 24. Meshes of at most
-// kFewTiles tiles (96^3) leave SMs idle or with one block: 1024 threads shorten each tile's chain of records.
-constexpr int kTilePaintThreads = 512, kFewTilesThreads = 1024, kFewTiles = 216;
+// Threads of a tile's block. Interlaced, three blocks' accumulators (64 KB each) fit an SM, and the shared atomics
+// need the warps: 512 threads keep 48 warps resident, 256 kept 24. Tiles of few particles (below 64 on average) have more
+// to clear and to store than to add and run better with blocks of 256 (512^3, 16 a tile: TSC paint 1161 -> 1099 us; 64 a tile
+// box 1397 -> 1319 but survey 821 -> 845). Without interlacing (32 KB) 256 threads keep as many warps in twice the blocks,
+// whose clearing, adding and storing overlap (512^3 box: 4 a tile 337 -> 214 us, 64 587 -> 478, 1024 2416 -> 2300); meshes of
+// up to 192^3 keep 512 for crowded tiles, whose few long chains of records decide (192^3 survey, TSC, 512 a tile 147 against
+// 155 us, 1024 237 against 263). Meshes of at most kFewTiles tiles (96^3) leave SMs idle or with one block:
+// 1024 threads shorten each tile's chain of records.
+constexpr int kFewTiles = 216, kSmallTiles = 1728;
+constexpr int kSparseTile = 64, kCrowdedTile = 512;  // particles per tile
+template <bool INTER> int tile_paint_threads(int ntiles, int64_t count) {
+  if (ntiles <= kFewTiles) return 1024;
+  if (INTER) return count < (int64_t)kSparseTile * ntiles ? 256 : 512;
+  return ntiles <= kSmallTiles && count >= (int64_t)kCrowdedTile * ntiles ? 512 : 256;
+}
 
 // One block per tile (every tile, so that empty tiles store their zeros): sums its records into
 // shared 64-bit accumulators (lo words of both meshes, then hi words), then stores each cell of
@@ -808,7 +819,7 @@ constexpr int kTilePaintThreads = 512, kFewTilesThreads = 1024, kFewTiles = 216;
 // cell - alpha * randoms cell instead: the same FMA as a pass of its own over the meshes, which
 // would read and write each once more (135 us a mesh at 384^3).
 template <int WIN, bool INTER, int NT>
-__global__ void __launch_bounds__(NT, NT <= 512 ? 3 : 1) k_ptile_paint(TileArgs ta, float* __restrict__ m1, float* __restrict__ m2,
+__global__ void __launch_bounds__(NT, NT == 256 && !INTER ? 6 : (NT <= 512 ? 3 : 1)) k_ptile_paint(TileArgs ta, float* __restrict__ m1, float* __restrict__ m2,
                                                      int N, const double* __restrict__ fix,
                                                      const float* __restrict__ r1, const float* __restrict__ r2,
                                                      const double* __restrict__ alpha) {
@@ -818,6 +829,7 @@ __global__ void __launch_bounds__(NT, NT <= 512 ? 3 : 1) k_ptile_paint(TileArgs 
   const int tile = blockIdx.x;
   const unsigned n = ta.cnt[tile];
   const unsigned o = ta.off[tile];
+  const unsigned nf = ta.cursor[tile] - o;  // records that touch this tile only
   const int nts = N / kPT;
   const int tz = tile % nts, ty = (tile / nts) % nts, tx = tile / (nts * nts);
   // 16-byte group i of the tile: mesh, then cells (lx, ly, lz..lz+3); its mesh address
@@ -847,9 +859,9 @@ __global__ void __launch_bounds__(NT, NT <= 512 ? 3 : 1) k_ptile_paint(TileArgs 
   const float scale = (float)sc, inv = (float)(1.0 / sc);  // powers of two: exact
   for (int i = threadIdx.x; i < 2 * NM * kPT3 / 4; i += blockDim.x) reinterpret_cast<uint4*>(acc)[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
-  const unsigned nf = ta.cursor[tile] - o;  // records that touch this tile only
-  for (unsigned q = threadIdx.x; q < nf; q += blockDim.x) tile_record<WIN, INTER, true>(acc, ta.sorted[o + q], scale);
-  for (unsigned q = nf + threadIdx.x; q < n; q += blockDim.x) tile_record<WIN, INTER, false>(acc, ta.sorted[o + q], scale);
+  // the others from the last warp on: a sparse tile's two short runs go to different warps
+  for (unsigned q = threadIdx.x; q < nf; q += NT) tile_record<WIN, INTER, true>(acc, ta.sorted[o + q], scale);
+  for (unsigned q = nf + (NT - 1 - threadIdx.x); q < n; q += NT) tile_record<WIN, INTER, false>(acc, ta.sorted[o + q], scale);
   __syncthreads();
   for (int i = threadIdx.x; i < NM * kPT3 / 4; i += blockDim.x) {
     int mesh;
@@ -922,7 +934,7 @@ void launch_ptile_scatter(const TileArgs& ta, int64_t total, const DevCat* dc, c
 }
 
 template <int WIN, bool INTER>
-static void ptile_paint_v(const TileArgs& ta, float* m1, float* m2, int N, const double* fix, const float* r1,
+static void ptile_paint_v(const TileArgs& ta, int64_t count, float* m1, float* m2, int N, const double* fix, const float* r1,
                           const float* r2, const double* alpha, cudaStream_t s) {
   const int ntiles = (N / kPT) * (N / kPT) * (N / kPT);
   const size_t smem = (size_t)(INTER ? 2 : 1) * kPT3 * sizeof(unsigned long long);
@@ -931,24 +943,25 @@ static void ptile_paint_v(const TileArgs& ta, float* m1, float* m2, int N, const
     allow_smem(k_ptile_paint<WIN, INTER, NT>, smem);
     k_ptile_paint<WIN, INTER, NT><<<ntiles, NT, smem, s>>>(ta, m1, m2, N, fix, r1, r2, alpha);
   };
-  if (ntiles <= kFewTiles)
-    go(std::integral_constant<int, kFewTilesThreads>{});
-  else
-    go(std::integral_constant<int, kTilePaintThreads>{});
+  switch (tile_paint_threads<INTER>(ntiles, count)) {
+    case 256: go(std::integral_constant<int, 256>{}); break;
+    case 512: go(std::integral_constant<int, 512>{}); break;
+    default: go(std::integral_constant<int, 1024>{});
+  }
 }
 
-void launch_ptile_paint(const TileArgs& ta, int window, int interlaced, float* m1, float* m2, int N,
+void launch_ptile_paint(const TileArgs& ta, int64_t count, int window, int interlaced, float* m1, float* m2, int N,
                         const double* fix, const float* r1, const float* r2, const double* alpha, cudaStream_t s) {
   if (window == PSPEC_WINDOW_CIC) {
     if (interlaced)
-      ptile_paint_v<PSPEC_WINDOW_CIC, true>(ta, m1, m2, N, fix, r1, r2, alpha, s);
+      ptile_paint_v<PSPEC_WINDOW_CIC, true>(ta, count, m1, m2, N, fix, r1, r2, alpha, s);
     else
-      ptile_paint_v<PSPEC_WINDOW_CIC, false>(ta, m1, m2, N, fix, r1, r2, alpha, s);
+      ptile_paint_v<PSPEC_WINDOW_CIC, false>(ta, count, m1, m2, N, fix, r1, r2, alpha, s);
   } else {
     if (interlaced)
-      ptile_paint_v<PSPEC_WINDOW_TSC, true>(ta, m1, m2, N, fix, r1, r2, alpha, s);
+      ptile_paint_v<PSPEC_WINDOW_TSC, true>(ta, count, m1, m2, N, fix, r1, r2, alpha, s);
     else
-      ptile_paint_v<PSPEC_WINDOW_TSC, false>(ta, m1, m2, N, fix, r1, r2, alpha, s);
+      ptile_paint_v<PSPEC_WINDOW_TSC, false>(ta, count, m1, m2, N, fix, r1, r2, alpha, s);
   }
 }
 

@@ -124,8 +124,9 @@ void launch_ptile_prep(const PaintArgs& a, int kind_a, const PaintArgs* b, int k
 void launch_ptile_scan(const TileArgs& ta, int ntiles, cudaStream_t s);
 void launch_ptile_scatter(const TileArgs& ta, int64_t total, const DevCat* dc, const int* cur, int N, int nsm,
                           cudaStream_t s);
-// r1, r2 (nullable, batched mocks): cached randoms meshes; mesh = painted - *alpha * randoms.
-void launch_ptile_paint(const TileArgs& ta, int window, int interlaced, float* m1, float* m2, int N,
+// count: the particles, or a bound on them (it chooses the blocks). r1, r2 (nullable, batched mocks): cached randoms
+// meshes; mesh = painted - *alpha * randoms.
+void launch_ptile_paint(const TileArgs& ta, int64_t count, int window, int interlaced, float* m1, float* m2, int N,
                         const double* fix, const float* r1, const float* r2, const double* alpha, cudaStream_t s);
 
 // Transform passes, one table of launchers per supported mesh side N (pass_*.cu).

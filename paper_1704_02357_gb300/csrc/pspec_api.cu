@@ -656,7 +656,7 @@ pspec_status do_paint(Ctx* c, const pspec_catalog* d, const pspec_catalog* r) {
     TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scan(ta, pl.ntiles, c->stream); }));
     TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scatter(ta, total, nullptr, nullptr, N, c->nsm, c->stream); }));
     TRY(run(c, PSPEC_K_PAINT, nmesh * pl.Sr, [&] {
-      launch_ptile_paint(ta, c->p.window, c->p.interlaced, f1, f2, N, der + D_FIX, nullptr, nullptr, nullptr, c->stream);
+      launch_ptile_paint(ta, total, c->p.window, c->p.interlaced, f1, f2, N, der + D_FIX, nullptr, nullptr, nullptr, c->stream);
     }));
     c->bytes_paint = bytes + cat_bytes(d) + cat_bytes(r) + nmesh * pl.Sr;
     return PSPEC_OK;
@@ -885,7 +885,7 @@ pspec_status paint_one(Ctx* c, const PaintArgs& a, int is_randoms, bool binned, 
     TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scan(ta, pl.ntiles, c->stream); }));
     TRY(run(c, PSPEC_K_PAINT, 0.0, [&] { launch_ptile_scatter(ta, a.count, a.dc, a.cur, N, c->nsm, c->stream); }));
     TRY(run(c, PSPEC_K_PAINT, (r1 ? 2.0 : 1.0) * nmesh * pl.Sr, [&] {
-      launch_ptile_paint(ta, c->p.window, c->p.interlaced, reinterpret_cast<float*>(m1), reinterpret_cast<float*>(m2),
+      launch_ptile_paint(ta, max_count, c->p.window, c->p.interlaced, reinterpret_cast<float*>(m1), reinterpret_cast<float*>(m2),
                          N, fix, reinterpret_cast<const float*>(r1), reinterpret_cast<const float*>(r2), der + D_ALPHA,
                          c->stream);
     }));
