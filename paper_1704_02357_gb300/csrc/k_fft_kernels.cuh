@@ -356,10 +356,10 @@ __global__ void __launch_bounds__(ylm_thread_cap(LT), sizeof(T) == 4 ? ylm_min_b
   const int a_lo = LT < 0 ? 0 : harm_a(h0), a_hi = LT < 0 ? 0 : harm_a(h0 + M - 1);
   const int sq = threadIdx.x / Tc, t = threadIdx.x - sq * Tc;
   C v[E];
-  constexpr bool kWarpTable = sizeof(T) == 4 && LT >= 0 && S::ZW;
-  const bool warp_local = kWarpTable && rtab != nullptr;  // uniform over the block
-  if constexpr (kWarpTable) {
-    if (rtab) {
+  constexpr bool kTable = LT == kLTTable;
+  constexpr bool warp_local = kTable && S::ZW;
+  if constexpr (kTable) {
+    if constexpr (S::ZW) {
       // the Tc threads of sequence (s, r) load their own slots: complex slot k of the row packs
       // f Y_lm(rhat) of nodes 2k and 2k + 1
       constexpr int64_t pts = (int64_t)N * N * N;
@@ -370,11 +370,9 @@ __global__ void __launch_bounds__(ylm_thread_cap(LT), sizeof(T) == 4 ? ylm_min_b
 #pragma unroll
       for (int e = 0; e < E; e++) {
         const float2 a = __ldg(fr + t + Tc * e), b = __ldg(yr + t + Tc * e);
-        v[e] = mk(a.x * b.x, a.y * b.y);
+        v[e] = mk(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));  // not contracted into the transform's additions
       }
-    }
-  } else if constexpr (sizeof(T) == 4 && LT >= 0) {
-    if (rtab) {
+    } else {
       // Y_lm(rhat) from the table (harmonics h0.., one slot of N^3 nodes each): each thread takes
       // one 4-node vector of one row, loads f once and the M table vectors back to back
       constexpr int64_t pts = (int64_t)N * N * N;
@@ -399,16 +397,22 @@ __global__ void __launch_bounds__(ylm_thread_cap(LT), sizeof(T) == 4 ? ylm_min_b
       poly_weights<N, LT>(f, axis, poly, LT > 0 ? LT : ell, h0, M, row0, rows, cf, stage);
     }
   }
-  for (int r = 0; r < rows; r++) {
-    const int grow = row0 + r;
+  // Weights per node, all rows' nodes in one run: a row is shorter than most blocks, and row by row 192 of 408 threads
+  // worked on 192^3 (z pass l <= 8 without the table 2.41 -> 1.49 ms, 96^3 l <= 16 3.23 -> 1.10, 512^3 l = 1 2.37 -> 1.99). FP64
+  // fills its pipe with half the threads and is 3 to 5% faster by rows from 192 on (96^3 l <= 16: 6.08 -> 5.09 ms in one run).
+  constexpr bool kByRows = sizeof(T) == 8 && N > 128;
+  for (int r0 = 0; r0 < (kByRows ? rows : 1); r0++) {
     if constexpr (LT >= 0) {
-      if (sizeof(T) == 4 ? rtab != nullptr : poly != nullptr) continue;
+      if (sizeof(T) == 4 ? kTable : poly != nullptr) continue;
     }
-    const int i = grow / N, j = grow - i * N;
-    const T vx = axis[i], vy = axis[N + j];
-    const T* frow = f + (int64_t)grow * N;
-    for (int kk = threadIdx.x; kk < N; kk += blockDim.x) {
-      const T fv = frow[kk];
+    const int grow0 = row0 + r0, i0 = grow0 / N;
+    const T vx0 = axis[i0], vy0 = axis[N + grow0 - i0 * N];
+    const T* frow = f + (int64_t)grow0 * N;
+    for (int q = threadIdx.x; q < (kByRows ? N : rows * N); q += blockDim.x) {
+      const int r = kByRows ? r0 : q / N, kk = kByRows ? q : q - r * N;
+      const int i = (row0 + r) / N, j = row0 + r - i * N;
+      const T vx = kByRows ? vx0 : axis[i], vy = kByRows ? vy0 : axis[N + j];
+      const T fv = frow[q];
       const T vz = axis[2 * N + kk];
       const T r2 = vx * vx + vy * vy + vz * vz;
       if (r2 == T(0)) {
@@ -1122,7 +1126,7 @@ template <typename T, int N> struct Passes {
   static void ylm_z_x(const T* f, C* out, int64_t stride, int ell, int h0, int M, const U* twh, const U* twr,
                       const T* axis, int rows, const float* rtab, const double* poly, cudaStream_t s) {
     if (rtab && ell >= 0) {  // weights from the table: no recurrence to specialise
-      ylm_z_v<0, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, rtab, poly, s);
+      if constexpr (sizeof(T) == 4) ylm_z_v<kLTTable, XP>(f, out, stride, ell, h0, M, twh, twr, axis, rows, rtab, poly, s);
       return;
     }
     switch (ell) {  // the headline multipoles get unrolled recurrences

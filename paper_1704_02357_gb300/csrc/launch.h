@@ -156,6 +156,10 @@ constexpr int z_rows(int N) {
   return r;
 }
 
+// LT of the z pass's kernels: l where its recurrence is unrolled (2, 4), 0 for any other l, kLTTable for weights read
+// from the Y_lm(rhat) table (no recurrence in that kernel, whose registers it would shape), -2 and -4 for
+// Cartesian monomials.
+constexpr int kLTTable = 1;
 // Threads of one block of the Y_lm-weighted z pass (harmonics x rows x threads per row) and
 // the resident blocks per SM its register allocation must allow (0: no requirement). The
 // unrolled l = 4 kernel launches at most 288 threads (9 x 16 x 2 at N = 512) and l = 2 at most

@@ -33,6 +33,12 @@ bool good_nmesh(int n) {
   return x == 3 && n >= 48;
 }
 
+int pow2_floor(int v) {
+  int p = 1;
+  while (p * 2 <= v) p *= 2;
+  return p;
+}
+
 struct Plan {
   Geo g;
   int E;
@@ -809,7 +815,11 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
       // take all that fit, f and the launches are what counts: 32^3 l <= 16 74 against 232 us, 128^3 768 against
       // 872 us, 192^3 4.20 against 4.19 ms (plain 3.17 against 3.29), 256^3 6.37 against 6.31 (plain 4.73 against 4.99).
       const bool tab = pl.has_rtab && ell > 0 && !(ell & 1);
-      const int cap = ylm_thread_cap(tab && N % 3 == 0 ? 0 : ell);
+      // Radix-3 meshes with the table take up to 512 threads a block from 96 on (48^3 is 2304 rows: fewer blocks than
+      // SMs). z pass of a set, power of two -> any divisor in rows: 384^3 l <= 4 2.85 -> 2.62 ms (plain 1.97 -> 1.87), without the
+      // table l <= 8 13.4 -> 12.0, 192^3 l <= 16 4.48 -> 4.20 (plain 3.00 -> 3.17; FP64 l = 16 10.5 -> 9.8), 96^3 0.68 -> 0.75, 48^3 0.156 -> 0.177.
+      const int cap = ylm_thread_cap(tab && N % 3 == 0 && N >= 96 ? 0 : ell);
+      const bool any = N % 3 == 0 && N >= (pl.xp || f64 ? 192 : 384);
       const int most = c->tune.ylm_harmonics < kYlmHarmonicsAuto ? c->tune.ylm_harmonics
                                                                  : (tab && N >= kYlmGroupsMesh ? 8 : INT_MAX);
       const int ms_max = std::max(1, std::min(most, cap / tz));
@@ -817,9 +827,10 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
       const int nlaunch = (M + ms_max - 1) / ms_max, ms = (M + nlaunch - 1) / nlaunch;  // of nearly equal size
       for (int hs = 0; hs < M; hs += ms) {
         const int Ms = std::min(ms, M - hs);
-        // the most rows that fit (any divisor of N^2: 6 and 12 on radix-3 meshes)
+        // the most rows that fit: a power of two, or on large radix-3 meshes any divisor of N^2 (6 and 12)
         int rows = std::max(1, cap / (Ms * tz));
-        while (rows > 1 && (((int64_t)N * N) % rows || PT->smem_ylm(Ms, rows) > kSmemBudget)) rows--;
+        if (!any) rows = pow2_floor(rows);
+        while (rows > 1 && (((int64_t)N * N) % rows || PT->smem_ylm(Ms, rows) > kSmemBudget)) rows = any ? rows - 1 : rows / 2;
         // even l of the SH route read their weights from the Y_lm(rhat) table when the plan holds it
         const float* rt = tab ? c->at<float>(pl.o_rtab) + (int64_t)(ytab_base(ell) + h0 + hs) * N * N * N
                               : nullptr;

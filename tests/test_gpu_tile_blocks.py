@@ -1,6 +1,8 @@
-"""The tile paint's block sizes on both sides of their rules (particles per tile, interlacing, mesh).
+"""The tile paint's block sizes on both sides of their rules (particles per tile, interlacing, mesh), and the z pass
+without the table where a block's rows are shorter or longer than its threads.
 
-P_0 of the exactly painted FP32 meshes against FP64 meshes: FP32 values and transforms, 1e-6 of |P_0| + S/I."""
+P_0 of the exactly painted FP32 meshes against FP64 meshes: FP32 values and transforms, 1e-6 of |P_0| + S/I. FP32 against
+FP64 weights: 1e-5, the bound of the FP32 path."""
 import numpy as np
 import pytest
 
@@ -35,3 +37,15 @@ def test_tile_blocks(nmesh, n, window, interlaced):
     g, f = (run_gpu(p, d, r, [0], edges, precision=prec) for prec in ("fp32", "fp64"))
     scale = np.abs(f["P"][0]) + f["stats"]["S"] / f["stats"]["I"]
     assert np.max(np.abs(g["P"] - f["P"]) / scale) < 1e-6
+
+
+@pytest.mark.parametrize("nmesh", [16, 48, 64, 96, 192, 256, 384])
+@pytest.mark.parametrize("precision", ["fp32", "fp32_plain"])
+def test_weights_without_the_table(nmesh, precision):
+    d, r = synth.uniform_box(3000, L, CORNER, 7), synth.uniform_box(9000, L, CORNER, 8)
+    p, edges = _params(nmesh, "cic", True, 3000), np.linspace(0.0, np.pi * nmesh / L, 6)
+    ells = [0, 1, 2, 4, 7] if nmesh < 192 else [0, 1, 2]
+    f = run_gpu(p, d, r, ells, edges, precision="fp64")
+    scale = np.abs(f["P"][0]) + f["stats"]["S"] / f["stats"]["I"]
+    g = run_gpu(p, d, r, ells, edges, precision=precision, ylm_table=False)
+    assert np.max(np.abs(g["P"] - f["P"]) / scale) < 1e-5
