@@ -717,8 +717,9 @@ __global__ void __launch_bounds__(col_threads<T, N>(), min_blocks<T, Shape<N>::E
   const int c = threadIdx.x % TW, t = threadIdx.x / TW;
   constexpr int64_t si = Lay<N>::XI, modes = (int64_t)N * N * NH;
   // 24 elements (radix 3): the table values are loaded after the transform, which needs the registers
-  // (spills otherwise), and the next tile is fetched into L2 meanwhile
-  constexpr bool kLateY = E > 8;
+  // (spills otherwise), and the next tile is fetched into L2 meanwhile; not in 48^3's blocks of 16 threads, which have
+  // nothing to hide the late loads behind (plain l <= 4 binning 73 against 61 us)
+  constexpr bool kLateY = E > 8 && col_threads<T, N>() >= 32;
   __syncthreads();
   for (int q = blockIdx.x; q < ba.n_xtiles * SUB; q += gridDim.x) {
     const int tile = ba.xtiles[q / SUB];
