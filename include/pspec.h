@@ -289,7 +289,7 @@ pspec_status pspec_catalog_sums_noalloc(const pspec_params* p, const pspec_catal
  *   paint_binned       1: tile-binned paint when the catalogs fit max_particles; 0: direct atomics
  *   ylm_harmonics      most harmonics per block of the Y_lm-weighted z pass (>= 1); 64 (the default) and
  *                      more leave it to the library: 8 with the Y_lm(rhat) table on meshes of 384^3 and
- *                      more, else all that fit
+ *                      more (192^3 with exact-add transforms), else all that fit
  *   bin_blocks_per_sm  persistent blocks per SM of the combine/binning passes (0: occupancy limit)
  *   tile_y             0: the compiled y-pass tile; 1: half as many columns per block
  * pspec_autotune paints the given catalogs and times pspec_multipoles_device for candidate

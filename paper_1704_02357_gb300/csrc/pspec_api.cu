@@ -19,7 +19,6 @@ constexpr size_t kAlign = 256;
 constexpr size_t kSmemBudget = 200 * 1024;   // one block
 constexpr int kMaxElls = PSPEC_MAX_ELL / 2 + 1;
 constexpr int kYlmHarmonicsAuto = 64;  // tuning value (the default) from which the z pass chooses itself
-constexpr int kYlmGroupsMesh = 384;   // ... groups of eight harmonics with the table (do_multipoles)
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -813,7 +812,8 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
       // in one block of 264 left 9). z pass of a set, all that fit -> eight: 384^3 l <= 16 31.6 -> 28.3 ms (plain 21.1 ->
       // 20.4), 512^3 l <= 4 4.83 -> 4.79 (plain 3.18 -> 3.03), 768^3 l <= 4 23.8 -> 22.4 ms (plain 17.0 -> 17.1). Smaller ones
       // take all that fit, f and the launches are what counts: 32^3 l <= 16 74 against 232 us, 128^3 768 against
-      // 872 us, 192^3 4.20 against 4.19 ms (plain 3.17 against 3.29), 256^3 6.37 against 6.31 (plain 4.73 against 4.99).
+      // 872 us, plain 192^3 3.17 against 3.29 ms, plain 256^3 4.73 against 4.99; exact-add from 192^3 on 4.20 -> 4.19 (one
+      // l = 12: 0.70 -> 0.67), 256^3 6.37 -> 6.31 ms.
       const bool tab = pl.has_rtab && ell > 0 && !(ell & 1);
       // Radix-3 meshes with the table take up to 512 threads a block from 96 on (48^3 is 2304 rows: fewer blocks than
       // SMs). z pass of a set, power of two -> any divisor in rows: 384^3 l <= 4 2.85 -> 2.62 ms (plain 1.97 -> 1.87), without the
@@ -821,7 +821,7 @@ pspec_status do_multipoles(Ctx* c, const int32_t* ells, int n_ells, int nk, doub
       const int cap = ylm_thread_cap(tab && N % 3 == 0 && N >= 96 ? 0 : ell);
       const bool any = N % 3 == 0 && N >= (pl.xp || f64 ? 192 : 384);
       const int most = c->tune.ylm_harmonics < kYlmHarmonicsAuto ? c->tune.ylm_harmonics
-                                                                 : (tab && N >= kYlmGroupsMesh ? 8 : INT_MAX);
+                                                                 : (tab && N >= (pl.xp ? 192 : 384) ? 8 : INT_MAX);
       const int ms_max = std::max(1, std::min(most, cap / tz));
       const double* rpoly = f64 && ell <= kPolyLmax ? c->at<PolyTab>(pl.o_poly)->rz + poly_base(ell) : nullptr;
       const int nlaunch = (M + ms_max - 1) / ms_max, ms = (M + nlaunch - 1) / nlaunch;  // of nearly equal size
