@@ -426,7 +426,7 @@ pspec_status upload_tables(Ctx* c) {
   // to FP64, the same for all modes of a plane, put the power off by 2e-16 to 5e-16 of itself.
   using A = std::conditional_t<sizeof(T) == 8, long double, double>;
   const A pi = sizeof(T) == 8 ? std::acos(A(-1)) : A(M_PI);
-  std::vector<A> winv(NH + 1);  // 1 / divisor, the same for n and -n
+  std::vector<C> winv(NH + 1);  // 1 / divisor and its remainder, the same for n and -n
   for (int n = 0; n <= NH; n++) {
     const A x = pi * n / N;
     A w = A(1);
@@ -437,15 +437,13 @@ pspec_status upload_tables(Ctx* c) {
       const A v = std::sin(x) / x;
       w = sizeof(T) == 4 ? std::pow(v, A(p)) : (p == 2 ? v * v : v * v * v);
     }
-    winv[n] = A(1) / w;
+    w = A(1) / w;
+    const T hi = T(w);
+    winv[n] = mk(hi, T(w / A(hi) - A(1)));
   }
   // exp(-i pi s / N), s = nx + ny + nz in [-3N/2, 3N/2): the H/2 shift of the second mesh
   for (int i = 0; i < 3 * N; i++) phase[i] = unit_factor<T>(-M_PI * (i - 3 * N / 2) / N);
-  for (int i = 0; i < N + NH; i++) {
-    const A w = winv[i < N ? (i < NH ? i : N - i) : i - N];
-    const T hi = T(w);
-    invw[i] = mk(hi, T(w / A(hi) - A(1)));
-  }
+  for (int i = 0; i < N + NH; i++) invw[i] = winv[i < N ? (i < NH ? i : N - i) : i - N];
   cudaError_t e;
   e = cudaMemcpyAsync(c->at<U>(pl.o_twh), twh.data(), twh.size() * sizeof(U), cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->at<U>(pl.o_twf), twf.data(), twf.size() * sizeof(U), cudaMemcpyHostToDevice, c->stream);
